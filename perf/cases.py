@@ -83,7 +83,7 @@ def draw(rng):
     if what < 0.25:
         method = rng.randint(0, 1)
         return dict(kind="calibration", b=rng.choice((4, 8)), n_real=_log_int(rng, 4, 64),
-                    steps=100 * rng.randint(4, CALIB_STEPS // 100), method=method,
+                    steps=100 * rng.randint(6, CALIB_STEPS // 100), method=method,
                     H=1500.0, rate=1000.0, sample_dH=1.0, alpha=0.1, mode=1, ckpt_every=rng.choice((128, 300, 512)))
     if what < 0.3:
         return dict(kind="batch", b=0, n_real=_log_int(rng, 3, 64), steps=_log_int(rng, 20, 400), H=1500.0,
