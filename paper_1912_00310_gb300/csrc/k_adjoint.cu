@@ -374,7 +374,10 @@ cudaError_t adjoint_recompute_all(const KParams &p, int n_real, long long step0,
 {
     const long long n_seg = (n_steps + ckpt_every - 1) / ckpt_every;
     if (n_seg < 1 || n_seg > 65535) return cudaErrorInvalidValue;
-    AdjParams ap = adj_params(p, n_real, step0, ckpt_every, step0 + n_steps, 0, 0, 1);
+    // a single segment takes its length from here (several: from seg_stride and n_total), and the
+    // states buffer holds n_steps of them, which may be fewer than ckpt_every
+    const int seg_len = (int)(n_steps < ckpt_every ? n_steps : (long long)ckpt_every);
+    AdjParams ap = adj_params(p, n_real, step0, seg_len, step0 + n_steps, 0, 0, 1);
     ap.seg_stride = ckpt_every;
     ap.n_total = n_steps;
     return launch_adjoint(ap, n_real, (int)n_seg, ckpt, states, nullptr, nullptr, nullptr, st);

@@ -264,3 +264,18 @@ def test_gradient_methods_long_period_sweep(pkg, orc):
                 (method, k, out[method][1], go)
     assert np.allclose(out[1][1], out[0][1], rtol=1e-3, atol=1e-4 * np.abs(go).max())
     g.close()
+
+
+@pytest.mark.parametrize("n_steps,ckpt_every", [(100, 512), (511, 512), (512, 512), (300, 1 << 20)])
+def test_window_within_one_checkpoint_interval(pkg, n_steps, ckpt_every):
+    """A window of at most one checkpoint interval recomputes its n_steps states and no more (the
+    stored window holds n_steps of them): the same loss and gradient as with a checkpoint interval
+    that divides the window, the loss bitwise, the gradient to the regrouping of its FP32 blocks."""
+    g = grid(pkg, ROD_DIMS[4])
+    target = target_for(g)
+    g.reset(seed=3, n_real=5)
+    L, grad = g.loss_grad(n_steps, target, 0, ckpt_every)
+    Lr, gr = g.loss_grad(n_steps, target, 0, 50)
+    assert L == Lr
+    assert np.allclose(grad, gr, rtol=1e-7, atol=0)
+    g.close()
