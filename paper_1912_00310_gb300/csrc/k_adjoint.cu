@@ -116,7 +116,7 @@ __global__ void __launch_bounds__(MAXT) adjoint_segment_kernel(
         field.inc();
         const float Hn1 = field.value();
         float *sj = seg + (size_t)j * n_rods * state + rod_off;
-        float3 acc = zero3a(), h = zero3a();
+        float3 s0 = zero3a(), h = zero3a();
         if (act) {
             sj[3 * c] = m.x;
             sj[3 * c + 1] = m.y;
@@ -125,17 +125,16 @@ __global__ void __launch_bounds__(MAXT) adjoint_segment_kernel(
         }
         __syncthreads();
         if (act) {
-            h = thermal_field(keys, (uint32_t)c, n, p.sigma);
+            h = thermal_field(keys, (uint32_t)c, n, p.sigma_bm);
             const float3 H = field_of(grad::neighbour_sum(M, nb), m, h, Hn);
-            const float3 s0 = llg_torque(m, H, p.alpha);
+            s0 = llg_torque(m, H, p.alpha);
             P[q] = pad4(normalised(axpy(p.neg_dt_g1, s0, m)));
-            acc = axpy(p.neg_hdt_g1, s0, m);
         }
         __syncthreads();
         if (act) {
             const float3 t = xyz(P[q]);
             const float3 H = field_of(grad::neighbour_sum(P, nb), t, h, Hn1);
-            m = normalised(axpy(p.neg_hdt_g1, llg_torque(t, H, p.alpha), acc));
+            m = normalised(axpy(p.neg_hdt_g1, llg_torque_add(s0, t, H, p.alpha), m));
         }
         __syncthreads();
         Hn = Hn1;
@@ -208,13 +207,13 @@ __global__ void __launch_bounds__(MAXT) adjoint_segment_kernel(
         }
         float3 Nm = zero3a();
         if (act) {
-            h = thermal_field(keys, (uint32_t)c, (unsigned long long)n, p.sigma);
+            h = thermal_field(keys, (uint32_t)c, (unsigned long long)n, p.sigma_bm);
             Nm = grad::neighbour_sum(M, nb);
             H = field_of(Nm, mi, h, hn);
             c0 = cross3(mi, H);
             s0 = llg_torque(mi, H, alpha);
             const float3 pv = axpy(p.neg_dt_g1, s0, mi);
-            pn = rsqrtf(dot3(pv, pv));  // 1 / |p|
+            pn = rsqrt_fast(dot3(pv, pv));  // 1 / |p|
             t = normalised(pv);
             P[q] = pad4(t);
         }
@@ -227,7 +226,7 @@ __global__ void __launch_bounds__(MAXT) adjoint_segment_kernel(
             c1 = cross3(t, Ht);
             s1 = llg_torque(t, Ht, alpha);
             const float3 qv = axpy(p.neg_hdt_g1, add3(s0, s1), mi);
-            const float rq = rsqrtf(dot3(qv, qv));  // 1 / |q|: m' = rq q, the forward's normalisation
+            const float rq = rsqrt_fast(dot3(qv, qv));  // 1 / |q|: m' = rq q, the forward's normalisation
             const float3 mp = scale3(rq, qv);
             gq = scale3(rq, sub3(g, scale3(dot3(mp, g), mp)));
             const float3 gs1 = scale3(-ha, gq);

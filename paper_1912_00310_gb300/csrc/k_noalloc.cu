@@ -4,7 +4,7 @@
 // CUDA graph (allocation is not a capturable operation), hosts whose device memory is owned by
 // another allocator that must see every allocation, and real-time loops that cannot afford the
 // device-wide synchronisation an allocation may cause.  For them this file keeps the plain
-// engine's scratch (the predictor state, the m + dt/2 f(m) accumulator and the thermal field of
+// engine's scratch (the predictor state, the predictor's torque and the thermal field of
 // every cell, plus a status word) in one fixed array in device global memory that is part of the
 // library image: every GPU that loads the library holds it until the process exits, and no call
 // here allocates anything.  The caller passes the state and the sample buffer.
@@ -19,7 +19,7 @@
 namespace {
 
 // Scratch of the allocation-free entry point: 9 floats per (realisation, cell) for the
-// predictor state, the accumulator and the thermal field, after a 256-byte header whose first
+// predictor state, its torque and the thermal field, after a 256-byte header whose first
 // word is the status flag.
 constexpr size_t kHeaderFloats = 64;
 constexpr size_t kScratchFloats = kHeaderFloats + 9 * (size_t)LLG_NOALLOC_MAX_CELL_REALISATIONS;

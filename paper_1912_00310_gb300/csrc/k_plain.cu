@@ -3,7 +3,7 @@
 // It is the straightforward form of the method, kept as the per-step baseline against which the
 // resident engine is measured, and the engine for periodic grids that do not fit on chip.
 //
-// Layout: m, mt (predictor), acc (m + dt/2 f(m)), hth (thermal field) are [n_real][ncells][3].
+// Layout: m, mt (predictor), s0 (the predictor's torque), hth (thermal field) are [n_real][ncells][3].
 #include "llg_internal.h"
 #include "physics.cuh"
 #include "reduce.cuh"
@@ -54,7 +54,7 @@ __device__ __forceinline__ float field_at(const KParams &p, unsigned long long n
 }
 
 __global__ void plain_pred_kernel(KParams p, const float *__restrict__ m, float *__restrict__ mt,
-                                  float *__restrict__ acc, float *__restrict__ hth, int n_real,
+                                  float *__restrict__ s0_out, float *__restrict__ hth, int n_real,
                                   unsigned long long n)
 {
     const float Hz = field_at(p, n);
@@ -66,17 +66,17 @@ __global__ void plain_pred_kernel(KParams p, const float *__restrict__ m, float 
     const float *mr = m + (size_t)r * p.ncells * 3;
     const float3 mi = ld3(mr + 3 * (size_t)i);
     const float3 nb = neighbour_sum(mr, x, y, z, p);
-    const float3 h = thermal_field(p.seed, p.real0 + (uint32_t)r, (uint32_t)i, n, p.sigma);
+    const float3 h = thermal_field(p.seed, p.real0 + (uint32_t)r, (uint32_t)i, n, p.sigma_bm);
     const float3 H = p.axis ? effective_field_axis(nb, mi, h, p.c_ex, p.c_an, Hz, xyz(__ldg(p.axis + gid)))
                             : effective_field(nb, mi, h, p.c_ex, p.c_an, Hz);
     const float3 s0 = llg_torque(mi, H, p.alpha);
     st3(mt + 3 * gid, normalised(axpy(p.neg_dt_g1, s0, mi)));
-    st3(acc + 3 * gid, axpy(p.neg_hdt_g1, s0, mi));
+    st3(s0_out + 3 * gid, s0);
     st3(hth + 3 * gid, h);
 }
 
 __global__ void plain_corr_kernel(KParams p, float *__restrict__ m, const float *__restrict__ mt,
-                                  const float *__restrict__ acc, const float *__restrict__ hth,
+                                  const float *__restrict__ s0_in, const float *__restrict__ hth,
                                   int n_real, unsigned long long n)
 {
     const float Hz1 = field_at(p, n + 1);
@@ -91,8 +91,8 @@ __global__ void plain_corr_kernel(KParams p, float *__restrict__ m, const float 
     const float3 h = ld3(hth + 3 * gid);
     const float3 H = p.axis ? effective_field_axis(nb, ti, h, p.c_ex, p.c_an, Hz1, xyz(__ldg(p.axis + gid)))
                             : effective_field(nb, ti, h, p.c_ex, p.c_an, Hz1);
-    const float3 s1 = llg_torque(ti, H, p.alpha);
-    st3(m + 3 * gid, normalised(axpy(p.neg_hdt_g1, s1, ld3(acc + 3 * gid))));
+    const float3 s = llg_torque_add(ld3(s0_in + 3 * gid), ti, H, p.alpha);
+    st3(m + 3 * gid, normalised(axpy(p.neg_hdt_g1, s, ld3(m + 3 * gid))));
 }
 
 // One warp per realisation: the canonical cell-average of m_z (see reduce.cuh).
@@ -132,19 +132,19 @@ unsigned blocks_for(long long n) { return (unsigned)((n + kThreads - 1) / kThrea
 
 }  // namespace
 
-cudaError_t plain_predictor(const KParams &p, const float *m, float *mt, float *acc, float *hth,
+cudaError_t plain_predictor(const KParams &p, const float *m, float *mt, float *s0, float *hth,
                             int n_real, long long n, cudaStream_t st)
 {
     plain_pred_kernel<<<blocks_for((long long)n_real * p.ncells), kThreads, 0, st>>>(
-        p, m, mt, acc, hth, n_real, (unsigned long long)n);
+        p, m, mt, s0, hth, n_real, (unsigned long long)n);
     return cudaGetLastError();
 }
 
-cudaError_t plain_corrector(const KParams &p, float *m, const float *mt, const float *acc,
+cudaError_t plain_corrector(const KParams &p, float *m, const float *mt, const float *s0,
                             const float *hth, int n_real, long long n, cudaStream_t st)
 {
     plain_corr_kernel<<<blocks_for((long long)n_real * p.ncells), kThreads, 0, st>>>(
-        p, m, mt, acc, hth, n_real, (unsigned long long)n);
+        p, m, mt, s0, hth, n_real, (unsigned long long)n);
     return cudaGetLastError();
 }
 
@@ -171,16 +171,16 @@ cudaError_t axis_fill(float4 *ax, int n_real, int ncells, uint32_t seed, uint32_
     return cudaGetLastError();
 }
 
-cudaError_t plain_advance(const KParams &p, float *m, float *mt, float *acc, float *hth, int n_real,
+cudaError_t plain_advance(const KParams &p, float *m, float *mt, float *s0, float *hth, int n_real,
                           long long step0, long long n_steps, float *samples, int *status,
                           cudaStream_t st, long long *launches)
 {
     long long count = 0;
     for (long long s = 0; s < n_steps; ++s) {
         const long long n = step0 + s;
-        cudaError_t e = plain_predictor(p, m, mt, acc, hth, n_real, n, st);
+        cudaError_t e = plain_predictor(p, m, mt, s0, hth, n_real, n, st);
         if (e != cudaSuccess) return e;
-        e = plain_corrector(p, m, mt, acc, hth, n_real, n, st);
+        e = plain_corrector(p, m, mt, s0, hth, n_real, n, st);
         if (e != cudaSuccess) return e;
         count += 2;
         const long long done = n + 1;

@@ -102,10 +102,11 @@ __global__ void __launch_bounds__(pipelined_max_threads(R), 1) rod_pipelined_ker
     const PhiloxKeys keys = philox_keys(p.seed, p.real0 + (uint32_t)rod);
     const float4 *axr = AX ? p.axis + (size_t)rod * ncell : nullptr;  // this rod's easy axes
 
-    float3 mprev[R], mcur[R], mta[R], mtb[R], acc[R], hth[R];
+    // carried per row: m(x-1), m(x); m~(x-2), m~(x-1), the torque s0(x-1) and the thermal field h(x-1)
+    float3 mprev[R], mcur[R], mta[R], mtb[R], s0c[R], hth[R];
 #pragma unroll
     for (int j = 0; j < R; ++j) {
-        mprev[j] = mcur[j] = mta[j] = mtb[j] = acc[j] = hth[j] = zero3();
+        mprev[j] = mcur[j] = mta[j] = mtb[j] = s0c[j] = hth[j] = zero3();
     }
     __syncthreads();
 
@@ -122,7 +123,9 @@ __global__ void __launch_bounds__(pipelined_max_threads(R), 1) rod_pipelined_ker
     const int lane = threadIdx.x & 31;
 
     while (pa || ca) {
-        float3 mt_new[R], acc_new[R], h_new[R];
+        float3 mt_new[R], s0_new[R], h_new[R], mcorr[R];
+#pragma unroll
+        for (int j = 0; j < R; ++j) mcorr[j] = mprev[j];  // the state at the corrector's plane
         if (pa) {
             const unsigned long long n = (unsigned long long)(step0 + sp);
             const float4 *Mp = M + xp * PL;
@@ -132,13 +135,10 @@ __global__ void __launch_bounds__(pipelined_max_threads(R), 1) rod_pipelined_ker
             for (int j = 0; j < R; ++j) {
                 if (!act[j]) continue;
                 const int qq = q[j];
-                if (xp == 0) {
-                    mcur[j] = xyz(Mp[qq]);
-                    mprev[j] = zero3();
-                }
+                if (xp == 0) mcur[j] = xyz(Mp[qq]);
                 const float3 mnext = has_next ? xyz(Mp[qq + PL]) : zero3();
-                h_new[j] = thermal_field(keys, cbase[j] + (uint32_t)xp, n, p.sigma);
-                float3 nb = add3(mprev[j], mnext);
+                h_new[j] = thermal_field(keys, cbase[j] + (uint32_t)xp, n, p.sigma_bm);
+                float3 nb = add3(xp == 0 ? zero3() : mprev[j], mnext);
                 nb = axpy(wm[j], xyz(Mp[qq - 1]), nb);
                 nb = axpy(wp[j], xyz(Mp[qq + 1]), nb);
                 nb = add3(nb, xyz(Mp[qq - ny]));
@@ -147,7 +147,7 @@ __global__ void __launch_bounds__(pipelined_max_threads(R), 1) rod_pipelined_ker
                 const float3 H = effective_field_sel<AX>(nb, mcur[j], h_new[j], p, Hp, u);
                 const float3 s0 = llg_torque(mcur[j], H, p.alpha);
                 mt_new[j] = normalised(axpy(p.neg_dt_g1, s0, mcur[j]));
-                acc_new[j] = axpy(p.neg_hdt_g1, s0, mcur[j]);
+                s0_new[j] = s0;
                 Sw[qq] = pad4(mt_new[j]);
                 mprev[j] = mcur[j];
                 mcur[j] = mnext;
@@ -169,8 +169,8 @@ __global__ void __launch_bounds__(pipelined_max_threads(R), 1) rod_pipelined_ker
                 nb = add3(nb, xyz(Sr[qq + ny]));
                 const float3 u = AX ? xyz(__ldg(axr + cbase[j] + xc)) : zero3();
                 const float3 H = effective_field_sel<AX>(nb, mtb[j], hth[j], p, Hc, u);
-                const float3 s1 = llg_torque(mtb[j], H, p.alpha);
-                Mw[qq] = pad4(normalised(axpy(p.neg_hdt_g1, s1, acc[j])));
+                const float3 s = llg_torque_add(s0c[j], mtb[j], H, p.alpha);
+                Mw[qq] = pad4(normalised(axpy(p.neg_hdt_g1, s, mcorr[j])));
             }
         }
         if (pa) {
@@ -178,7 +178,7 @@ __global__ void __launch_bounds__(pipelined_max_threads(R), 1) rod_pipelined_ker
             for (int j = 0; j < R; ++j) {
                 mta[j] = xp == 0 ? zero3() : mtb[j];
                 mtb[j] = mt_new[j];
-                acc[j] = acc_new[j];
+                s0c[j] = s0_new[j];
                 hth[j] = h_new[j];
             }
         }
@@ -321,11 +321,12 @@ struct PipelinedRod {
         }
         const PhiloxKeys keys = philox_keys(p.seed, p.real0 + (uint32_t)rod);
         const float4 *axr = AX ? p.axis + (size_t)rod * ncell : nullptr;  // easy axes (AX)
-        // carried per row: m(x-1), m(x) for the predictor; m~(x-2), m~(x-1), acc(x-1), h(x-1)
-        // for the corrector one plane behind
-        float3 mA[R], mB[R], tA[R], tB[R], acc[R], hth[R];
+        // carried per row: m(x-1), m(x) for the predictor; m~(x-2), m~(x-1), the torque s0(x-1) and
+        // h(x-1) for the corrector one plane behind (which reads m(x-1) back from its plane: the
+        // registers are all in use)
+        float3 mA[R], mB[R], tA[R], tB[R], s0c[R], hth[R];
 #pragma unroll
-        for (int j = 0; j < R; ++j) mA[j] = mB[j] = tA[j] = tB[j] = acc[j] = hth[j] = zero3();
+        for (int j = 0; j < R; ++j) mA[j] = mB[j] = tA[j] = tB[j] = s0c[j] = hth[j] = zero3();
         __syncthreads();
 
         SweepOf<SHAPE> field;
@@ -339,7 +340,7 @@ struct PipelinedRod {
         // thermal field of the next predictor, drawn one iteration ahead (before the barrier)
         float3 hpre[R];
 #pragma unroll
-        for (int j = 0; j < R; ++j) hpre[j] = thermal_field(keys, cbase[j], (unsigned long long)s0, p.sigma);
+        for (int j = 0; j < R; ++j) hpre[j] = thermal_field(keys, cbase[j], (unsigned long long)s0, p.sigma_bm);
         // AX: the easy axis of the next predictor's cell, loaded one iteration ahead like the
         // noise, and the axis of the plane the corrector works on (the previous predictor's)
         float3 upre[R], ucor[R];
@@ -356,7 +357,7 @@ struct PipelinedRod {
                 // ---- predictor at (s, x): writes slot x & 1 ----
                 const float4 *Mp = M + x * PL;
                 float4 *Sw = S + (x & 1) * PL;
-                float3 tnew[R], anew[R], hnew[R];
+                float3 tnew[R], snew[R], hnew[R];
 #pragma unroll
                 for (int j = 0; j < R; ++j) {
                     if (!act[j]) continue;
@@ -373,9 +374,8 @@ struct PipelinedRod {
                     nb = add3(nb, xyz(Mp[qq - ny]));
                     nb = add3(nb, xyz(Mp[qq + ny]));
                     const float3 H = effective_field_sel<AX>(nb, mB[j], hnew[j], p, Hs, upre[j]);
-                    const float3 s0v = llg_torque(mB[j], H, p.alpha);
-                    tnew[j] = normalised(axpy(p.neg_dt_g1, s0v, mB[j]));
-                    anew[j] = axpy(p.neg_hdt_g1, s0v, mB[j]);
+                    snew[j] = llg_torque(mB[j], H, p.alpha);
+                    tnew[j] = normalised(axpy(p.neg_dt_g1, snew[j], mB[j]));
                     Sw[qq] = pad4(tnew[j]);
                     mA[j] = mB[j];
                     mB[j] = mnext;
@@ -397,19 +397,19 @@ struct PipelinedRod {
                         nb = add3(nb, xyz(Sr[qq - ny]));
                         nb = add3(nb, xyz(Sr[qq + ny]));
                         const float3 H = effective_field_sel<AX>(nb, tB[j], hth[j], p, Hc, ucor[j]);
-                        const float3 s1 = llg_torque(tB[j], H, p.alpha);
-                        Mw[qq] = pad4(normalised(axpy(p.neg_hdt_g1, s1, acc[j])));
+                        const float3 sv = llg_torque_add(s0c[j], tB[j], H, p.alpha);
+                        Mw[qq] = pad4(normalised(axpy(p.neg_hdt_g1, sv, xyz(Mw[qq]))));
                     }
                 }
 #pragma unroll
                 for (int j = 0; j < R; ++j) {
                     tA[j] = x == 0 ? zero3() : tB[j];
                     tB[j] = tnew[j];
-                    acc[j] = anew[j];
+                    s0c[j] = snew[j];
                     hth[j] = hnew[j];
                     // the next predictor: plane x+1 of this step, or plane 0 of the next one
-                    hpre[j] = x + 1 < NX ? thermal_field(keys, cbase[j] + (uint32_t)(x + 1), n, p.sigma)
-                                         : thermal_field(keys, cbase[j], n + 1, p.sigma);
+                    hpre[j] = x + 1 < NX ? thermal_field(keys, cbase[j] + (uint32_t)(x + 1), n, p.sigma_bm)
+                                         : thermal_field(keys, cbase[j], n + 1, p.sigma_bm);
                     if constexpr (AX) {
                         ucor[j] = upre[j];
                         upre[j] = xyz(__ldg(axr + cbase[j] + (uint32_t)(x + 1 < NX ? x + 1 : 0)));
@@ -440,8 +440,8 @@ struct PipelinedRod {
                 nb = add3(nb, xyz(Sr[qq - ny]));
                 nb = add3(nb, xyz(Sr[qq + ny]));
                 const float3 H = effective_field_sel<AX>(nb, tB[j], hth[j], p, Hprev, ucor[j]);
-                const float3 s1 = llg_torque(tB[j], H, p.alpha);
-                Mw[qq] = pad4(normalised(axpy(p.neg_hdt_g1, s1, acc[j])));
+                const float3 sv = llg_torque_add(s0c[j], tB[j], H, p.alpha);
+                Mw[qq] = pad4(normalised(axpy(p.neg_hdt_g1, sv, xyz(Mw[qq]))));
             }
             __syncthreads();
             if (s0 + ns == next_sample) sample(p, rod, next_sample / se, samples, status);

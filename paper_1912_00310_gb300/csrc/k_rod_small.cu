@@ -4,7 +4,7 @@
 //
 // Each rod is padded by a zero ghost layer so the 6-neighbour stencil has no branches.  Per Heun
 // step: every thread takes the thermal field of its cells (drawn before the previous barrier),
-// computes the predictor into the P buffer and keeps m + dt/2 f(m) in registers; barrier; the
+// computes the predictor into the P buffer and keeps its torque in registers; barrier; the
 // corrector reads P and overwrites M, then draws the next step's thermal field; barrier.  A
 // thread owns CPT cells (t, t + T, t + 2T, ... of the CTA's rods), so the per-step bookkeeping
 // is shared by CPT cell-updates.
@@ -105,45 +105,45 @@ __global__ void __launch_bounds__(MAXT) rod_twophase_kernel(KParams p, float *__
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = T >> 5;
 
     // thermal field of the next step, drawn before the barrier that ends the current one
-    float3 hpre[CPT];
+    float3 hpre[CPT], m[CPT];  // and the cells' own state, which stays in registers
 #pragma unroll
-    for (int k = 0; k < CPT; ++k) hpre[k] = thermal_field(p.seed, real[k], cell[k], (unsigned long long)step0, p.sigma);
+    for (int k = 0; k < CPT; ++k) m[k] = xyz(M[pidx[k]]);
+#pragma unroll
+    for (int k = 0; k < CPT; ++k) hpre[k] = thermal_field(p.seed, real[k], cell[k], (unsigned long long)step0, p.sigma_bm);
     unsigned long long n = (unsigned long long)step0;
     for (int s = 0; s < n_steps; ++s, ++n) {
         field.inc();
         const float Hn1 = field.value();
-        float3 acc[CPT], hth[CPT];
+        float3 t[CPT], s0[CPT], hth[CPT];
 #pragma unroll
         for (int k = 0; k < CPT; ++k) {
             if (!act[k]) continue;
             const int q = pidx[k];
             hth[k] = hpre[k];
-            const float3 mi = xyz(M[q]);
             float3 nb = add3(xyz(M[q - 1]), xyz(M[q + 1]));
             nb = add3(nb, xyz(M[q - sy]));
             nb = add3(nb, xyz(M[q + sy]));
             nb = add3(nb, xyz(M[q - sz]));
             nb = add3(nb, xyz(M[q + sz]));
-            const float3 H = effective_field_sel<AX>(nb, mi, hth[k], p, Hn, uax[k]);
-            const float3 s0 = llg_torque(mi, H, p.alpha);
-            P[q] = pad4(normalised(axpy(p.neg_dt_g1, s0, mi)));
-            acc[k] = axpy(p.neg_hdt_g1, s0, mi);
+            const float3 H = effective_field_sel<AX>(nb, m[k], hth[k], p, Hn, uax[k]);
+            s0[k] = llg_torque(m[k], H, p.alpha);
+            t[k] = normalised(axpy(p.neg_dt_g1, s0[k], m[k]));
+            P[q] = pad4(t[k]);
         }
         __syncthreads();
 #pragma unroll
         for (int k = 0; k < CPT; ++k) {
             if (!act[k]) continue;
             const int q = pidx[k];
-            const float3 ti = xyz(P[q]);
             float3 nb = add3(xyz(P[q - 1]), xyz(P[q + 1]));
             nb = add3(nb, xyz(P[q - sy]));
             nb = add3(nb, xyz(P[q + sy]));
             nb = add3(nb, xyz(P[q - sz]));
             nb = add3(nb, xyz(P[q + sz]));
-            const float3 H = effective_field_sel<AX>(nb, ti, hth[k], p, Hn1, uax[k]);
-            const float3 s1 = llg_torque(ti, H, p.alpha);
-            M[q] = pad4(normalised(axpy(p.neg_hdt_g1, s1, acc[k])));
-            hpre[k] = thermal_field(p.seed, real[k], cell[k], n + 1, p.sigma);
+            const float3 H = effective_field_sel<AX>(nb, t[k], hth[k], p, Hn1, uax[k]);
+            m[k] = normalised(axpy(p.neg_hdt_g1, llg_torque_add(s0[k], t[k], H, p.alpha), m[k]));
+            M[q] = pad4(m[k]);
+            hpre[k] = thermal_field(p.seed, real[k], cell[k], n + 1, p.sigma_bm);
         }
         __syncthreads();
         Hn = Hn1;
@@ -178,8 +178,8 @@ __global__ void __launch_bounds__(MAXT) rod_twophase_kernel(KParams p, float *__
 
 // ------------------------------------------------------------------------------------------
 // Row kernel (the b = 2, 4, 8 rods: 4x12x28, 2x6x14, 1x3x7 cells, shapes at compile time).  A
-// thread owns one x-row (fixed y, z) of NX cells and keeps the row's state, predictor, corrector
-// accumulator and thermal field in registers; the x-neighbours come from registers, the y- and
+// thread owns one x-row (fixed y, z) of NX cells and keeps the row's state, predictor, torque
+// and thermal field in registers; the x-neighbours come from registers, the y- and
 // z-neighbours from shared memory.  Shared memory holds per rod, for each x, a plane of rows
 // (y, z) with ghost lines at y = -1, NY and z = -1, NZ: M[x][(z + 1)(NY + 2) + y + 1] and the same
 // for the predictor P, so consecutive threads (consecutive y) read consecutive float4s.  Per
@@ -237,12 +237,12 @@ __global__ void __launch_bounds__(MAXT) rod_rows_kernel(KParams p, float *__rest
     // thermal field of the next step, drawn before the barrier that ends the current one
     float3 hpre[NX];
 #pragma unroll
-    for (int x = 0; x < NX; ++x) hpre[x] = thermal_field(keys, cbase + x, (unsigned long long)step0, p.sigma);
+    for (int x = 0; x < NX; ++x) hpre[x] = thermal_field(keys, cbase + x, (unsigned long long)step0, p.sigma_bm);
     unsigned long long n = (unsigned long long)step0;
     for (int s = 0; s < n_steps; ++s, ++n) {
         field.inc();
         const float Hn1 = field.value();
-        float3 mt[NX], acc[NX], hth[NX];
+        float3 mt[NX], s0[NX], hth[NX];
         if (act) {
 #pragma unroll
             for (int x = 0; x < NX; ++x) {
@@ -254,9 +254,8 @@ __global__ void __launch_bounds__(MAXT) rod_rows_kernel(KParams p, float *__rest
                 nb = add3(nb, xyz(Mx[-PY]));
                 nb = add3(nb, xyz(Mx[PY]));
                 const float3 H = effective_field_sel<AX>(nb, m[x], hth[x], p, Hn, u[x]);
-                const float3 s0 = llg_torque(m[x], H, p.alpha);
-                mt[x] = normalised(axpy(p.neg_dt_g1, s0, m[x]));
-                acc[x] = axpy(p.neg_hdt_g1, s0, m[x]);
+                s0[x] = llg_torque(m[x], H, p.alpha);
+                mt[x] = normalised(axpy(p.neg_dt_g1, s0[x], m[x]));
                 P[q + x * PLANE] = pad4(mt[x]);
             }
         }
@@ -271,12 +270,11 @@ __global__ void __launch_bounds__(MAXT) rod_rows_kernel(KParams p, float *__rest
                 nb = add3(nb, xyz(Px[-PY]));
                 nb = add3(nb, xyz(Px[PY]));
                 const float3 H = effective_field_sel<AX>(nb, mt[x], hth[x], p, Hn1, u[x]);
-                const float3 s1 = llg_torque(mt[x], H, p.alpha);
-                m[x] = normalised(axpy(p.neg_hdt_g1, s1, acc[x]));
+                m[x] = normalised(axpy(p.neg_hdt_g1, llg_torque_add(s0[x], mt[x], H, p.alpha), m[x]));
                 M[q + x * PLANE] = pad4(m[x]);
             }
 #pragma unroll
-            for (int x = 0; x < NX; ++x) hpre[x] = thermal_field(keys, cbase + x, n + 1, p.sigma);
+            for (int x = 0; x < NX; ++x) hpre[x] = thermal_field(keys, cbase + x, n + 1, p.sigma_bm);
         }
         __syncthreads();
         Hn = Hn1;

@@ -162,9 +162,9 @@ struct SlabSweep {
     bool perx, pery;
     // registers carried along z: the own state of plane z-1 (its slot is refilled before the
     // predictor of plane z reads it; the own state of plane z is re-read from its slot) and the
-    // corrector's accumulator m + dt/2 f of the last predictor; the thermal field the corrector
+    // torque of the last predictor; the thermal field the corrector
     // reuses waits in shared memory (Hs), which keeps the four-column instance in registers
-    float3 Sp[CPT], A[CPT];  // own state of the previous plane, accumulator of the last predictor
+    float3 Sp[CPT], A[CPT];  // own state of the previous plane, torque of the last predictor
     float3 rSp;              // the ring cell's state of the previous plane
     float4 *Hs;          // [CPT][blockDim.x] thermal field of the own columns' last predictor
 
@@ -249,11 +249,12 @@ struct SlabSweep {
             if (!act(k)) continue;
             const int c = q(k);
             float3 tnew = zero3s(), h = zero3s(), anew = zero3s();
+            const float3 mcorr = Sp[k];  // the state of plane z-1, which the corrector starts from
             float4 *hs = Hs + k * blockDim.x + threadIdx.x;
             if (pred) {
                 const float3 mcur = xyz(Mz[c]);
                 const float3 mnext = has_next ? xyz(Mn[c]) : zero3s();
-                h = thermal_field(keys, cell(k) + zoff, n, p.sigma);
+                h = thermal_field(keys, cell(k) + zoff, n, p.sigma_bm);
                 float3 nb = add3(xyz(Mz[c - 1]), xyz(Mz[c + 1]));
                 nb = add3(nb, xyz(Mz[c - P]));
                 nb = add3(nb, xyz(Mz[c + P]));
@@ -262,9 +263,8 @@ struct SlabSweep {
                 Sp[k] = mcur;
                 const float3 u = AX ? xyz(__ldg(axr + cell(k) + zoff)) : zero3s();
                 const float3 H = effective_field_sel<AX>(nb, mcur, h, p, Hn, u);
-                const float3 sv = llg_torque(mcur, H, p.alpha);
-                tnew = normalised(axpy(p.neg_dt_g1, sv, mcur));
-                anew = axpy(p.neg_hdt_g1, sv, mcur);
+                anew = llg_torque(mcur, H, p.alpha);
+                tnew = normalised(axpy(p.neg_dt_g1, anew, mcur));
                 Tw[c] = pad4(tnew);
             }
             if (corr) {
@@ -277,8 +277,8 @@ struct SlabSweep {
                 nb = add3(nb, pred ? tnew : zero3s());
                 const float3 u = AX ? xyz(__ldg(axr + cell(k) + zcoff)) : zero3s();
                 const float3 H = effective_field_sel<AX>(nb, tself, xyz(*hs), p, Hn1, u);
-                const float3 s1 = llg_torque(tself, H, p.alpha);
-                store(k, z - 1, pad4(normalised(axpy(p.neg_hdt_g1, s1, A[k]))));
+                const float3 sv = llg_torque_add(A[k], tself, H, p.alpha);
+                store(k, z - 1, pad4(normalised(axpy(p.neg_hdt_g1, sv, mcorr))));
             }
             if (pred) {
                 *hs = pad4(h);  // after the corrector read the previous plane's
@@ -290,7 +290,7 @@ struct SlabSweep {
             if (rin) {
                 const float3 rcur = xyz(Mz[rpos]);
                 const float3 rnext = has_next ? xyz(Mn[rpos]) : zero3s();
-                const float3 h = thermal_field(keys, rcell + zoff, n, p.sigma);
+                const float3 h = thermal_field(keys, rcell + zoff, n, p.sigma_bm);
                 float3 nb = add3(xyz(Mz[rpos - 1]), xyz(Mz[rpos + 1]));
                 nb = add3(nb, xyz(Mz[rpos - P]));
                 nb = add3(nb, xyz(Mz[rpos + P]));

@@ -93,7 +93,7 @@ __global__ void __launch_bounds__(MAXT, MAXT <= 256 ? 1 : 0) tangent_kernel(TanP
             m[k] = make_float3(src[0], src[1], src[2]);
             if (AX) u[k] = xyz(__ldg(p.axis + (size_t)rod * ncell + c));
             // thermal field of the next step, drawn before the step's last barrier
-            hpre[k] = thermal_field(keys, (uint32_t)c, (unsigned long long)tp.step0, p.sigma);
+            hpre[k] = thermal_field(keys, (uint32_t)c, (unsigned long long)tp.step0, p.sigma_bm);
         }
     }
     __syncthreads();
@@ -129,23 +129,22 @@ __global__ void __launch_bounds__(MAXT, MAXT <= 256 ? 1 : 0) tangent_kernel(TanP
         const unsigned long long n = (unsigned long long)(tp.step0 + s);
         field.inc();
         const float Hn1 = field.value();
-        float3 acc[CPT], dacc[CPT], t[CPT], dtt[CPT];
+        float3 s0[CPT], dacc[CPT], t[CPT], dtt[CPT];
 #pragma unroll
         for (int k = 0; k < CPT; ++k) {
-            acc[k] = dacc[k] = t[k] = dtt[k] = zr3();
+            s0[k] = dacc[k] = t[k] = dtt[k] = zr3();
             const int c = threadIdx.x + k * blockDim.x;
             if (c >= ncell) continue;
             const float3 N = grad::neighbour_sum(M, nb[k]), Nd = grad::neighbour_sum(Md, nb[k]);
             const float3 H = effective_field_sel<AX>(N, m[k], hpre[k], p, Hn, u[k]);
-            const float3 s0 = llg_torque(m[k], H, alpha);
+            s0[k] = llg_torque(m[k], H, alpha);
             const float3 ds0 = half_tan(m[k], dm[k], N, Nd, hpre[k], H, u[k]);
-            const float3 pv = axpy(p.neg_dt_g1, s0, m[k]);
-            const float r = rsqrtf(fmaf(pv.x, pv.x, fmaf(pv.y, pv.y, pv.z * pv.z)));
+            const float3 pv = axpy(p.neg_dt_g1, s0[k], m[k]);
+            const float r = rsqrt_fast(fmaf(pv.x, pv.x, fmaf(pv.y, pv.y, pv.z * pv.z)));
             t[k] = make_float3(pv.x * r, pv.y * r, pv.z * r);  // normalised(pv), the engines' arithmetic
-            acc[k] = axpy(p.neg_hdt_g1, s0, m[k]);
-            const float3 dp = sb3(sb3(dm[k], sc3(da, s0)), sc3(a, ds0));
+            const float3 dp = sb3(sb3(dm[k], sc3(da, s0[k])), sc3(a, ds0));
             dtt[k] = sc3(r, sb3(dp, sc3(dt3(t[k], dp), t[k])));
-            dacc[k] = sb3(sb3(dm[k], sc3(0.5f * da, s0)), sc3(0.5f * a, ds0));
+            dacc[k] = sb3(dm[k], sc3(0.5f * a, ds0));
             Pd[c] = pad4(dtt[k]);
             P[c] = pad4(t[k]);
         }
@@ -156,16 +155,16 @@ __global__ void __launch_bounds__(MAXT, MAXT <= 256 ? 1 : 0) tangent_kernel(TanP
             if (c >= ncell) continue;
             const float3 N = grad::neighbour_sum(P, nb[k]), Nd = grad::neighbour_sum(Pd, nb[k]);
             const float3 H = effective_field_sel<AX>(N, t[k], hpre[k], p, Hn1, u[k]);
-            const float3 s1 = llg_torque(t[k], H, alpha);
+            const float3 s01 = llg_torque_add(s0[k], t[k], H, alpha);
             const float3 ds1 = half_tan(t[k], dtt[k], N, Nd, hpre[k], H, u[k]);
-            const float3 qv = axpy(p.neg_hdt_g1, s1, acc[k]);
-            const float r = rsqrtf(fmaf(qv.x, qv.x, fmaf(qv.y, qv.y, qv.z * qv.z)));
+            const float3 qv = axpy(p.neg_hdt_g1, s01, m[k]);
+            const float r = rsqrt_fast(fmaf(qv.x, qv.x, fmaf(qv.y, qv.y, qv.z * qv.z)));
             m[k] = make_float3(qv.x * r, qv.y * r, qv.z * r);
-            const float3 dq = sb3(sb3(dacc[k], sc3(0.5f * da, s1)), sc3(0.5f * a, ds1));
+            const float3 dq = sb3(sb3(dacc[k], sc3(0.5f * da, s01)), sc3(0.5f * a, ds1));
             dm[k] = sc3(r, sb3(dq, sc3(dt3(m[k], dq), m[k])));
             Md[c] = pad4(dm[k]);
             M[c] = pad4(m[k]);
-            hpre[k] = thermal_field(keys, (uint32_t)c, n + 1, p.sigma);
+            hpre[k] = thermal_field(keys, (uint32_t)c, n + 1, p.sigma_bm);
         }
         __syncthreads();
         Hn = Hn1;

@@ -37,9 +37,10 @@ struct Derived {
 struct KParams {
     int nx, ny, nz, ncells;
     unsigned periodic;        // bit0 x, bit1 y, bit2 z
-    float c_ex, c_an, sigma;  // A/m
-    float neg_dt_g1;          // -dt g1   (predictor)
-    float neg_hdt_g1;         // -dt g1/2 (corrector)
+    float c_ex, c_an;         // A/m
+    float sigma_bm;           // -sigma sqrt(2 ln 2): the Box-Muller radius factor (box_muller3), A/m
+    float neg_dt_g1;          // -dt g1   (predictor: m + neg_dt_g1 s0)
+    float neg_hdt_g1;         // -dt g1/2 (corrector: m + neg_hdt_g1 (s0 + s1))
     float alpha;
     float H0, slope;          // triangle sweep, A/m and A/m per step
     long long n_half;
@@ -81,18 +82,18 @@ KParams kparams_of(const Derived &d, int nx, int ny, int nz, unsigned periodic, 
 void gk_flow(double Ts0, double h0, double g0, double b, long long n_steps, double out[4]);
 
 // ---- plain engine (k_plain.cu): state in global memory, two launches per step --------------
-// m, mt: [n_real][ncells][3]; acc, hth: same shape (scratch).
+// m, mt: [n_real][ncells][3]; s0 (the predictor's torque), hth: same shape (scratch).
 // The field of step n (predictor) and n + 1 (corrector) is evaluated on the device.
-cudaError_t plain_predictor(const KParams &p, const float *m, float *mt, float *acc, float *hth,
+cudaError_t plain_predictor(const KParams &p, const float *m, float *mt, float *s0, float *hth,
                             int n_real, long long n, cudaStream_t st);
-cudaError_t plain_corrector(const KParams &p, float *m, const float *mt, const float *acc,
+cudaError_t plain_corrector(const KParams &p, float *m, const float *mt, const float *s0,
                             const float *hth, int n_real, long long n, cudaStream_t st);
 // samples[r][k] = mean over cells of m_z; sets *status = 1 on a non-finite mean.
 cudaError_t plain_sample(const KParams &p, const float *m, int n_real, long long k, float *samples,
                          int *status, cudaStream_t st);
 // Host-side driver of the plain engine over n_steps from step0 (one predictor and one corrector
 // launch per step, a reduction launch per sample).
-cudaError_t plain_advance(const KParams &p, float *m, float *mt, float *acc, float *hth, int n_real,
+cudaError_t plain_advance(const KParams &p, float *m, float *mt, float *s0, float *hth, int n_real,
                           long long step0, long long n_steps, float *samples, int *status,
                           cudaStream_t st, long long *launches);
 

@@ -4,9 +4,18 @@
 // field sweep (triangle or sinusoid) evaluated from an integer phase.
 //
 // Eq. 1 for the unit vector m = M/Ms:  dm/dt = -g1 m x H - alpha g1 m x (m x H),
-// g1 = mu0 ge / (1 + alpha^2).  Writing s(m, H) = m x H + alpha m x (m x H), the right-hand side
-// is f = -g1 s, so the Heun predictor is m~ = normalise(m - dt g1 s(m, H_n)) and the corrector
-// m' = normalise(m - (dt g1 / 2) (s(m, H_n) + s(m~, H~_n+1))).
+// g1 = mu0 ge / (1 + alpha^2).  Writing s(m, H) = m x H + alpha m x (m x H) = m x (H + alpha m x H),
+// the right-hand side is f = -g1 s, so the Heun predictor is m~ = normalise(m - dt g1 s0), s0 =
+// s(m, H_n), and the corrector m' = normalise(m - (dt g1 / 2) (s0 + s(m~, H~_n+1))).  The engines
+// carry s0 from the predictor to the corrector, which adds its own torque into it before the one
+// multiply-add that forms the new state: the sum of two small torques is rounded at their own size
+// and the state once.
+//
+// The special functions are the approximate instructions in their flush-to-zero form: rsqrtf,
+// __log2f and the like compile to the same instruction between a comparison and two scalings for
+// subnormal arguments, which cannot occur here (the norm of a near-unit vector, log2 of a uniform
+// of at least 2^-25, a Box-Muller radius).  On GB300 that and the shorter Box-Muller below took the
+// noise draw alone from 127 to 105 scheduler cycles per warp and cell.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -69,30 +78,59 @@ __device__ __forceinline__ uint4 philox4x32_10(uint4 c, const PhiloxKeys &K)
     return c;
 }
 
-// Uniform in (0,1): (floor(x / 256) + 1/2) * 2^-24, exact in FP32.
-__device__ __forceinline__ float uniform24(uint32_t x)
+__device__ __forceinline__ float rsqrt_fast(float x)
 {
-    return fmaf(__uint2float_rn(x >> 8), 0x1p-24f, 0x1p-25f);
+    float y;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
 }
 
-// Thermal field from the four Philox words of (seed, realisation, cell, step): sigma times
-// three standard normals from Box-Muller on (u0, u1) and (u2, u3).  The angle is taken as
-// 2 pi (u - 1/2), inside the accurate range of the hardware sine, which negates both members of
-// each pair.
-__device__ __forceinline__ float3 box_muller3(uint4 x, float sigma)
+__device__ __forceinline__ float sqrt_fast(float x)
 {
-    const float u0 = uniform24(x.x), u1 = uniform24(x.y);
-    const float u2 = uniform24(x.z), u3 = uniform24(x.w);
-    const float kNeg2Ln2 = -1.3862943611198906f;  // -2 ln 2 : -2 ln u = -2 ln2 log2 u
-    const float v0 = fmaxf(kNeg2Ln2 * __log2f(u0), 1e-30f);
-    const float v2 = fmaxf(kNeg2Ln2 * __log2f(u2), 1e-30f);
-    const float r0 = -sigma * v0 * rsqrtf(v0);
-    const float r2 = -sigma * v2 * rsqrtf(v2);
-    const float kTwoPi = 6.283185307179586f;
-    float s1, c1;
-    __sincosf(kTwoPi * (u1 - 0.5f), &s1, &c1);
-    const float c3 = __cosf(kTwoPi * (u3 - 0.5f));
-    return make_float3(r0 * c1, r0 * s1, r2 * c3);
+    float y;
+    asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+
+__device__ __forceinline__ float log2_fast(float x)
+{
+    float y;
+    asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+
+__device__ __forceinline__ float sin_fast(float x)
+{
+    float y;
+    asm("sin.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+
+__device__ __forceinline__ float cos_fast(float x)
+{
+    float y;
+    asm("cos.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+
+// The 24 bits of a Philox word that form a uniform u = (floor(x / 256) + 1/2) * 2^-24, as a float.
+__device__ __forceinline__ float bits24(uint32_t x) { return __uint2float_rn(x >> 8); }
+
+__device__ __forceinline__ float uniform24(uint32_t x) { return fmaf(bits24(x), 0x1p-24f, 0x1p-25f); }
+
+// Thermal field from the four Philox words of (seed, realisation, cell, step): sigma times
+// three standard normals from Box-Muller on (u0, u1) and (u2, u3).  sqrt(-2 ln u) is taken as
+// sqrt(2 ln 2) sqrt(|log2 u|), the constant being part of sigma_bm = -sigma sqrt(2 ln 2); the angle
+// as 2 pi (u - 1/2), formed from the 24 bits by one multiply-add and inside the accurate range of
+// the hardware sine, which negates both members of each pair, hence the sign of sigma_bm.
+__device__ __forceinline__ float3 box_muller3(uint4 x, float sigma_bm)
+{
+    const float r0 = sigma_bm * sqrt_fast(fabsf(log2_fast(uniform24(x.x))));
+    const float r2 = sigma_bm * sqrt_fast(fabsf(log2_fast(uniform24(x.z))));
+    const float kStep = 6.283185307179586f * 0x1p-24f;                      // 2 pi 2^-24
+    const float kFirst = 6.283185307179586f * 0x1p-25f - 3.141592653589793f;  // 2 pi (2^-25 - 1/2)
+    const float a1 = fmaf(bits24(x.y), kStep, kFirst), a3 = fmaf(bits24(x.w), kStep, kFirst);
+    return make_float3(r0 * cos_fast(a1), r0 * sin_fast(a1), r2 * cos_fast(a3));
 }
 
 __device__ __forceinline__ uint4 noise_counter(uint32_t cell, unsigned long long step)
@@ -101,32 +139,43 @@ __device__ __forceinline__ uint4 noise_counter(uint32_t cell, unsigned long long
 }
 
 __device__ __forceinline__ float3 thermal_field(uint32_t seed, uint32_t real, uint32_t cell,
-                                                unsigned long long step, float sigma)
+                                                unsigned long long step, float sigma_bm)
 {
-    return box_muller3(philox4x32_10(noise_counter(cell, step), seed, real), sigma);
+    return box_muller3(philox4x32_10(noise_counter(cell, step), seed, real), sigma_bm);
 }
 
 __device__ __forceinline__ float3 thermal_field(const PhiloxKeys &K, uint32_t cell,
-                                                unsigned long long step, float sigma)
+                                                unsigned long long step, float sigma_bm)
 {
-    return box_muller3(philox4x32_10(noise_counter(cell, step), K), sigma);
+    return box_muller3(philox4x32_10(noise_counter(cell, step), K), sigma_bm);
 }
 
-// s(m, H) = m x H + alpha m x (m x H)
-__device__ __forceinline__ float3 llg_torque(float3 m, float3 H, float alpha)
+__device__ __forceinline__ float3 torque_arm(float3 m, float3 H, float alpha)  // H + alpha m x H
 {
     const float ax = fmaf(m.y, H.z, -m.z * H.y);
     const float ay = fmaf(m.z, H.x, -m.x * H.z);
     const float az = fmaf(m.x, H.y, -m.y * H.x);
-    const float bx = fmaf(m.y, az, -m.z * ay);
-    const float by = fmaf(m.z, ax, -m.x * az);
-    const float bz = fmaf(m.x, ay, -m.y * ax);
-    return make_float3(fmaf(alpha, bx, ax), fmaf(alpha, by, ay), fmaf(alpha, bz, az));
+    return make_float3(fmaf(alpha, ax, H.x), fmaf(alpha, ay, H.y), fmaf(alpha, az, H.z));
+}
+
+// s(m, H) = m x (H + alpha m x H)
+__device__ __forceinline__ float3 llg_torque(float3 m, float3 H, float alpha)
+{
+    const float3 B = torque_arm(m, H, alpha);
+    return make_float3(fmaf(m.y, B.z, -m.z * B.y), fmaf(m.z, B.x, -m.x * B.z), fmaf(m.x, B.y, -m.y * B.x));
+}
+
+// s0 + s(m, H)
+__device__ __forceinline__ float3 llg_torque_add(float3 s0, float3 m, float3 H, float alpha)
+{
+    const float3 B = torque_arm(m, H, alpha);
+    return make_float3(fmaf(m.y, B.z, fmaf(-m.z, B.y, s0.x)), fmaf(m.z, B.x, fmaf(-m.x, B.z, s0.y)),
+                       fmaf(m.x, B.y, fmaf(-m.y, B.x, s0.z)));
 }
 
 __device__ __forceinline__ float3 normalised(float3 v)
 {
-    const float r = rsqrtf(fmaf(v.x, v.x, fmaf(v.y, v.y, v.z * v.z)));
+    const float r = rsqrt_fast(fmaf(v.x, v.x, fmaf(v.y, v.y, v.z * v.z)));
     return make_float3(v.x * r, v.y * r, v.z * r);
 }
 

@@ -130,7 +130,7 @@ KParams kparams_of(const Derived &d, int nx, int ny, int nz, unsigned periodic, 
     p.periodic = periodic;
     p.c_ex = (float)d.c_ex;
     p.c_an = (float)d.c_an;
-    p.sigma = (float)d.sigma;
+    p.sigma_bm = (float)(-d.sigma * std::sqrt(2.0 * std::log(2.0)));
     p.neg_dt_g1 = (float)(-dt * d.g1);
     p.neg_hdt_g1 = (float)(-0.5 * dt * d.g1);
     p.alpha = (float)d.alpha;
