@@ -348,7 +348,7 @@ def run_ours(args):
             "roofline": {"bound": "alu", "achieved": achieved / 1e9, "peak": peak / 1e9,
                          "unit": "Gop/s", "frac": achieved / peak, "traffic": measured_traffic(),
                          "traffic_unit": "bytes per launch (ncu dram read + write)",
-                         "kernel": "rod_pipelined_nx_kernel<3, 8, 24, 56>",
+                         "kernel": "rod_pairs_kernel<3, 4, 24, 56>",
                          "ops_per_cell_step": ALU_OPS_PER_CELL_STEP,
                          "peak_basis": "measured: FP32 FMA issue microbenchmark (llg_measure_alu_peak) "
                                        f"at {alu['ffma_sm_mhz']:.0f} MHz",

@@ -27,6 +27,8 @@ struct llg_ctx {
     double disp = 0.0;    // easy-axis dispersion: cone half-angle (rad) about z, 0 = axis z
     float4 *d_axis = nullptr;  // [n_real][ncells] easy axes when disp > 0
     size_t axis_cap = 0;       // float4 entries
+    float *d_axis_pairs = nullptr;  // the same in the pair kernel's layout (grids that have one)
+    size_t axis_pairs_cap = 0;      // floats
     bool axis_ok = false;      // d_axis holds the axes of (ax_seed, ax_real0, ax_n, ax_disp)
     uint32_t ax_seed = 0, ax_real0 = 0;
     int ax_n = 0;
@@ -119,39 +121,51 @@ llg_status grow(float **buf, size_t *cap, size_t need_floats)
 }
 
 // The easy axes of the ensemble in the dispersed-axis mode, drawn on the context's stream when
-// the ensemble's keys or the dispersion changed; *out = NULL in the z-axis mode.
-llg_status ensure_axes(llg_ctx *c, const float4 **out)
+// the ensemble's keys or the dispersion changed; kp's axes = NULL in the z-axis mode.
+llg_status ensure_axes(llg_ctx *c, llg::KParams *kp)
 {
-    *out = nullptr;
+    kp->axis = nullptr;
+    kp->axis_pairs = kp->axis_pairs_z = nullptr;
     if (!(c->disp > 0.0)) return LLG_OK;
     if (c->n_real < 1) return fail(LLG_EINVAL, "no ensemble (llg_reset first)");
-    if (c->axis_ok && c->ax_seed == c->seed && c->ax_real0 == c->real0 && c->ax_n == c->n_real &&
-        c->ax_disp == c->disp) {
-        *out = c->d_axis;
-        return LLG_OK;
-    }
     const size_t need = (size_t)c->n_real * (size_t)ncells_of(c);
-    if (c->axis_cap < need) {
-        cudaFree(c->d_axis);
-        c->d_axis = nullptr;
-        c->axis_cap = 0;
-        cudaError_t e = cudaMalloc(&c->d_axis, need * sizeof(float4));
-        if (e != cudaSuccess) {
+    const size_t need_pairs = llg::pairs_axis_floats(c->nx, c->ny, c->nz, c->n_real);
+    if (!(c->axis_ok && c->ax_seed == c->seed && c->ax_real0 == c->real0 && c->ax_n == c->n_real &&
+          c->ax_disp == c->disp)) {
+        c->axis_ok = false;
+        if (c->axis_cap < need) {
+            cudaFree(c->d_axis);
             c->d_axis = nullptr;
-            cudaGetLastError();
-            return fail(LLG_ENOMEM, "cudaMalloc of %zu bytes (easy axes) failed", need * sizeof(float4));
+            c->axis_cap = 0;
+            cudaError_t e = cudaMalloc(&c->d_axis, need * sizeof(float4));
+            if (e != cudaSuccess) {
+                c->d_axis = nullptr;
+                cudaGetLastError();
+                return fail(LLG_ENOMEM, "cudaMalloc of %zu bytes (easy axes) failed", need * sizeof(float4));
+            }
+            c->axis_cap = need;
         }
-        c->axis_cap = need;
+        if (need_pairs > 0) {
+            const llg_status s = grow(&c->d_axis_pairs, &c->axis_pairs_cap, need_pairs);
+            if (s != LLG_OK) return s;
+        }
+        const float w_max = (float)(1.0 - std::cos(c->disp));
+        LLG_CUDA(llg::axis_fill(c->d_axis, c->n_real, (int)ncells_of(c), c->seed, c->real0, w_max, c->stream),
+                 "easy-axis draw");
+        if (need_pairs > 0)
+            LLG_CUDA(llg::pairs_axis_fill(c->d_axis_pairs, c->n_real, c->ny, c->nz, c->seed, c->real0, w_max, c->stream),
+                     "easy-axis draw");
+        c->axis_ok = true;
+        c->ax_seed = c->seed;
+        c->ax_real0 = c->real0;
+        c->ax_n = c->n_real;
+        c->ax_disp = c->disp;
     }
-    const float w_max = (float)(1.0 - std::cos(c->disp));
-    LLG_CUDA(llg::axis_fill(c->d_axis, c->n_real, (int)ncells_of(c), c->seed, c->real0, w_max, c->stream),
-             "easy-axis draw");
-    c->axis_ok = true;
-    c->ax_seed = c->seed;
-    c->ax_real0 = c->real0;
-    c->ax_n = c->n_real;
-    c->ax_disp = c->disp;
-    *out = c->d_axis;
+    kp->axis = c->d_axis;
+    if (need_pairs > 0) {
+        kp->axis_pairs = c->d_axis_pairs;
+        kp->axis_pairs_z = c->d_axis_pairs + need_pairs / 6 * 4;
+    }
     return LLG_OK;
 }
 
@@ -224,7 +238,7 @@ llg_status ctx_view(llg_ctx *c, CtxView *v)
     v->kp.real0 = c->real0;
     if (c->n_real > 0) {
         DeviceGuard g(c->device);
-        const llg_status sa = ensure_axes(c, &v->kp.axis);
+        const llg_status sa = ensure_axes(c, &v->kp);
         if (sa != LLG_OK) return sa;
     }
     v->tune_kind = c->tune_kind;
@@ -305,6 +319,7 @@ void llg_destroy(llg_ctx *c)
     cudaFree(c->d_flags);
     cudaFree(c->d_slab);
     cudaFree(c->d_axis);
+    cudaFree(c->d_axis_pairs);
     cudaGetLastError();
     delete c;
 }
@@ -415,9 +430,10 @@ llg_status llg_get_axes(llg_ctx *c, float *u)
     if (c->n_real < 1 || !c->d_m) return fail(LLG_EINVAL, "no ensemble (llg_reset first)");
     DeviceGuard g(c->device);
     const size_t n = (size_t)c->n_real * (size_t)ncells_of(c);
-    const float4 *ax = nullptr;
-    llg_status s = ensure_axes(c, &ax);
+    llg::KParams kp{};
+    llg_status s = ensure_axes(c, &kp);
     if (s != LLG_OK) return s;
+    const float4 *ax = kp.axis;
     const bool dev = is_device_ptr(u);
     if (!ax) {  // z-axis mode
         if (dev) {
@@ -556,7 +572,7 @@ llg_status llg_advance(llg_ctx *c, int64_t n_steps, float *m_samples)
     llg::KParams kp = llg::kparams_of(d, c->nx, c->ny, c->nz, c->periodic, c->sw.dt);
     kp.seed = c->seed;
     kp.real0 = c->real0;
-    s = ensure_axes(c, &kp.axis);
+    s = ensure_axes(c, &kp);
     if (s != LLG_OK) return s;
     llg::RodPlan plan{};
     llg::SlabPlan splan{};
@@ -809,7 +825,7 @@ llg_status llg_loop_area_grad(llg_ctx *c, int64_t n_steps, int objective, const 
     llg::KParams kp = llg::kparams_of(d, c->nx, c->ny, c->nz, c->periodic, c->sw.dt);
     kp.seed = c->seed;
     kp.real0 = c->real0;
-    s = ensure_axes(c, &kp.axis);
+    s = ensure_axes(c, &kp);
     if (s != LLG_OK) return s;
     const long long step0 = c->step, N = n_steps, C = ckpt_every;
     const long long S = (N + C - 1) / C;

@@ -54,6 +54,9 @@ struct KParams {
     // per-cell easy axes [n_real][ncells] (x, y, z, 0) of the dispersed-axis mode, or NULL for
     // the axis z in every cell; indexed by the rod's position in this ensemble
     const float4 *axis;
+    // the same axes in the layout of the pair kernel (k_rod_pairs.cu), for the b = 1 rod: (xa, xb, ya,
+    // yb) and (za, zb) per pair of x-neighbours
+    const float *axis_pairs, *axis_pairs_z;
 };
 
 // Host helpers (scaling.cpp)
@@ -133,6 +136,15 @@ int rows_max_threads(const KParams &p);
 size_t rows_rod_bytes(const KParams &p);
 cudaError_t rows_advance(const KParams &p, const RodPlan &plan, float *m, int n_real, long long step0, int n_steps,
                          float *samples, int *status, cudaStream_t st);
+// Pair kernel (k_rod_pairs.cu, plan kind 2): rods eight cells wide; flags as for rod_advance.  Its
+// copy of the easy axes: the floats it needs (0: this grid has none; 4 of 6 for the x and y, then z)
+// and the draw.
+size_t pairs_axis_floats(int nx, int ny, int nz, int n_real);
+cudaError_t pairs_axis_fill(float *out, int n_real, int ny, int nz, uint32_t seed, uint32_t real0, float w_max,
+                            cudaStream_t st);
+bool pairs_supported(const KParams &p);
+cudaError_t pairs_advance(const KParams &p, const RodPlan &plan, float *m, int n_real, long long step0, int n_steps,
+                          float *samples, int *status, unsigned *flags, cudaStream_t st);
 int twophase_max_threads(const KParams &p, int cpt);
 cudaError_t twophase_advance(const KParams &p, const RodPlan &plan, float *m, int n_real, long long step0,
                              int n_steps, float *samples, int *status, cudaStream_t st);

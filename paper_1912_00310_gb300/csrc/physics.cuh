@@ -78,6 +78,32 @@ __device__ __forceinline__ uint4 philox4x32_10(uint4 c, const PhiloxKeys &K)
     return c;
 }
 
+// The first two rounds for the counters (cell, step, 0) of one rod and step.  Round 1 mixes the cell
+// and the step separately and round 2 multiplies one word of each, so what depends on the step
+// alone is formed once per rod and step (PhiloxStep), and a cell is left with its product
+// kPhiloxM0 * cell -- an addition from cell to cell along a row -- and 17 of the 20 multiplies.
+struct PhiloxStep {
+    uint32_t a, b, w;
+};
+
+__device__ __forceinline__ PhiloxStep philox_step(const PhiloxKeys &K, unsigned long long step)
+{
+    const unsigned long long p1 = (unsigned long long)kPhiloxM1 * (uint32_t)(step >> 32);
+    const unsigned long long p0 =
+        (unsigned long long)kPhiloxM0 * ((uint32_t)(p1 >> 32) ^ (uint32_t)step ^ K.k0[0]);
+    return PhiloxStep{(uint32_t)p1 ^ K.k0[1], (uint32_t)(p0 >> 32) ^ K.k1[1], (uint32_t)p0};
+}
+
+// The words of the cell whose product kPhiloxM0 * cell is cell_m0.
+__device__ __forceinline__ uint4 philox4x32_10(const PhiloxKeys &K, const PhiloxStep &S, unsigned long long cell_m0)
+{
+    const unsigned long long p1 = (unsigned long long)kPhiloxM1 * ((uint32_t)(cell_m0 >> 32) ^ K.k1[0]);
+    uint4 c = make_uint4((uint32_t)(p1 >> 32) ^ S.a, (uint32_t)p1, (uint32_t)cell_m0 ^ S.b, S.w);
+#pragma unroll
+    for (int r = 2; r < 10; ++r) c = philox_round(c, K.k0[r], K.k1[r]);
+    return c;
+}
+
 __device__ __forceinline__ float rsqrt_fast(float x)
 {
     float y;
@@ -123,13 +149,14 @@ __device__ __forceinline__ float uniform24(uint32_t x) { return fmaf(bits24(x), 
 // sqrt(2 ln 2) sqrt(|log2 u|), the constant being part of sigma_bm = -sigma sqrt(2 ln 2); the angle
 // as 2 pi (u - 1/2), formed from the 24 bits by one multiply-add and inside the accurate range of
 // the hardware sine, which negates both members of each pair, hence the sign of sigma_bm.
+constexpr float kAngleStep = (float)(6.283185307179586476925 * 0x1p-24);                          // 2 pi 2^-24
+constexpr float kAngleFirst = (float)(6.283185307179586476925 * 0x1p-25 - 3.141592653589793238463);  // 2 pi (2^-25 - 1/2)
+
 __device__ __forceinline__ float3 box_muller3(uint4 x, float sigma_bm)
 {
     const float r0 = sigma_bm * sqrt_fast(fabsf(log2_fast(uniform24(x.x))));
     const float r2 = sigma_bm * sqrt_fast(fabsf(log2_fast(uniform24(x.z))));
-    const float kStep = 6.283185307179586f * 0x1p-24f;                      // 2 pi 2^-24
-    const float kFirst = 6.283185307179586f * 0x1p-25f - 3.141592653589793f;  // 2 pi (2^-25 - 1/2)
-    const float a1 = fmaf(bits24(x.y), kStep, kFirst), a3 = fmaf(bits24(x.w), kStep, kFirst);
+    const float a1 = fmaf(bits24(x.y), kAngleStep, kAngleFirst), a3 = fmaf(bits24(x.w), kAngleStep, kAngleFirst);
     return make_float3(r0 * cos_fast(a1), r0 * sin_fast(a1), r2 * cos_fast(a3));
 }
 
