@@ -840,7 +840,7 @@ llg_status llg_loop_area_grad(llg_ctx *c, int64_t n_steps, int objective, const 
     if (!llg::adjoint_supported(kp, c->device))
         return fail(LLG_EUNSUPPORTED, "the adjoint handles rods of at most 1024 cells with free faces");
     llg::RodPlan plan{};
-    if (!llg::rod_plan(kp, c->n_real, c->device, &plan, 1, 0, 0))
+    if (!llg::rod_plan(kp, c->n_real, c->device, &plan))
         return fail(LLG_EUNSUPPORTED, "no resident forward plan for this grid");
     const long long ns_total = std::max<long long>(d.n_samples, k_last + 1);
     // store the whole window's states when they fit the budget and a quarter of the free memory

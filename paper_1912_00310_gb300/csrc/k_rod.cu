@@ -3,8 +3,9 @@
 //
 // Two kernels, chosen by rod size:
 //
-//  rod_twophase_kernel  (rods whose state and predictor state both fit: b >= 2 in the paper's
-//      ladder), in k_rod_small.cu.  Several rods per CTA, each padded with a zero ghost layer.
+//  rod_zpairs_kernel (rods whose state and predictor state both fit), in k_rod_zpairs.cu; for the
+//      b = 2, 4, 8 rods of the paper's ladder rod_rows_kernel and rod_cells_kernel, in k_rod_small.cu.
+//      One or several rods per CTA, two barriers a step.
 //
 //  rod_pipelined_kernel (the b = 1 rod, 8x24x56 = 10752 cells: M alone is 129 KB, M and a full
 //      predictor copy do not fit).  One rod per CTA.  Each thread owns rows along x (fixed y, z);
@@ -250,12 +251,17 @@ bool rod_plan(const KParams &p, int n_real, int dev, RodPlan *plan, int force_ki
     const size_t pipe_bytes = ((size_t)p.nx + 2) * PL * sizeof(float4);
     const bool twophase_fits = rod_bytes <= (size_t)smem_optin && p.ncells <= 4 * kMaxThreads;
     const bool pipelined_fits = pipe_bytes <= (size_t)smem_optin && rows <= 4 * 672;
-    // Default (measured on GB300): the b = 2, 4, 8 rods of the paper's ladder use the row kernel;
-    // other rods of at most one CTA of threads the two-phase kernel with one rod per CTA (many
-    // small CTAs per SM); larger rods the plane-pipelined kernel.
+    // Default (measured on GB300): the b = 2, 4, 8 rods of the paper's ladder use the row kernel (four
+    // b = 4 rods 0.47 us a step against 0.60 with the two-phase kernel, 608 0.86 against 0.96); other
+    // rods whose pairs fit one to a thread the two-phase kernel with one rod per CTA (152 rods of
+    // 5x11x23 cells 2.15 us against 3.09 with the plane-pipelined one, 7x9x13 1.57 against 3.42; with
+    // several rods to an SM the two are level); larger rods the plane-pipelined kernels.
     int kind = force_kind;
-    if (kind == 0)
-        kind = rows_supported(p) ? 3 : ((p.ncells <= kMaxThreads && twophase_fits) ? 1 : (pipelined_fits ? 2 : 1));
+    if (kind == 0) {
+        RodPlan one{};
+        const bool pair_each = twophase_fits && twophase_shape(p, 1, &one) && one.pairs_per_thread == 1;
+        kind = rows_supported(p) ? 3 : (pair_each ? 1 : (pipelined_fits ? 2 : 1));
+    }
     if (kind == 3) {
         if (!rows_supported(p)) return false;
         const int maxt = rows_max_threads(p);
@@ -263,9 +269,9 @@ bool rod_plan(const KParams &p, int n_real, int dev, RodPlan *plan, int force_ki
         const int by_smem = (int)std::max<size_t>(1, (size_t)smem_optin / rbytes);
         int rods = force_rods;
         if (rods == 0) {
-            // one rod per CTA (measured on GB300 ahead of packing rods: 608 b = 4 rods at 9.9e10
-            // cell-steps/s), unless that leaves over a quarter of the last warp idle (the b = 8
-            // rod's 21 rows): then the fewest rods that leave at most a tenth of it
+            // one rod per CTA (608 b = 4 rods 0.87 us a step; 0.90, 0.98 and 1.23 with 2, 4 and 6),
+            // unless that leaves over a quarter of the last warp idle (the b = 8 rod's 21 cells): then
+            // the fewest rods that leave at most a tenth of it (4096 rods 0.82 us with 3, 1.13 with 1)
             rods = 1;
             if (4 * (round_warp(rows) - rows) > round_warp(rows))
                 for (int r = 2; r * rows <= maxt && r <= by_smem; ++r)
@@ -280,7 +286,7 @@ bool rod_plan(const KParams &p, int n_real, int dev, RodPlan *plan, int force_ki
         plan->cells_per_thread = p.nx;
         plan->threads = round_warp(rods * rows);
         plan->rows_per_thread = 1;
-        plan->smem_bytes = rods * rbytes;
+        plan->smem_bytes = rows_smem_bytes(p, rods);
         plan->ctas = (n_real + rods - 1) / rods;
         return true;
     }
@@ -299,12 +305,15 @@ bool rod_plan(const KParams &p, int n_real, int dev, RodPlan *plan, int force_ki
         int rods = 1;
         if (force_rods > 0) rods = force_rods;
         if (rods > by_smem || round_warp((rods * p.ncells + cpt - 1) / cpt) > maxt) return false;
+        // what was asked for is accepted by the sizes of one cell a thread in a ghost-padded rod; the
+        // pairs take less, except for several flat rods at once: then as many of them as fit
+        while (rods > 1 && (rods * twophase_rod_bytes(p) > (size_t)smem_optin || !twophase_shape(p, rods, plan))) --rods;
+        if (!twophase_shape(p, rods, plan)) return false;
         plan->kind = 1;
         plan->rods_per_cta = rods;
         plan->cells_per_thread = cpt;
-        plan->threads = round_warp((rods * p.ncells + cpt - 1) / cpt);
         plan->rows_per_thread = 0;
-        plan->smem_bytes = rods * rod_bytes;
+        plan->smem_bytes = rods * twophase_rod_bytes(p);
         plan->ctas = (n_real + rods - 1) / rods;
         return true;
     }

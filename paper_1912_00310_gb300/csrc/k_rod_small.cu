@@ -1,23 +1,9 @@
-// k_rod_small.cu -- the resident engine's two-phase kernel, for rods whose state and predictor
-// state both fit in shared memory with room for several rods per CTA (b >= 2 in the paper's
-// ladder: 4x12x28, 2x6x14, 1x3x7 cells).
-//
-// Each rod is padded by a zero ghost layer so the 6-neighbour stencil has no branches.  Per Heun
-// step: every thread takes the thermal field of its cells (drawn before the previous barrier),
-// computes the predictor into the P buffer and keeps its torque in registers; barrier; the
-// corrector reads P and overwrites M, then draws the next step's thermal field; barrier.  A
-// thread owns CPT cells (t, t + T, t + 2T, ... of the CTA's rods), so the per-step bookkeeping
-// is shared by CPT cell-updates.
-//
-// Instances: the b = 4 and b = 8 rods with their shape at compile time (every stencil offset an
-// immediate), the sweep shape at compile time with its phase and the sample countdown in 32 bits
-// (loops of fewer than 2^31 steps), and a register budget that grows with CPT (launch bound
-// 768 / CPT threads); and, for any other grid, a runtime-shape instance with 64-bit sweep
-// bookkeeping.  All use the neighbour order x-, x+, y-, y+, z-, z+ and the physics.cuh arithmetic
-// of every other engine, so their trajectories are bitwise those of the plain engine.
+// k_rod_small.cu -- the resident engine's row kernel for the b = 2, 4, 8 rods of the paper's ladder
+// (plan kind 3).
 #include <algorithm>
 
 #include "llg_internal.h"
+#include "pair.cuh"
 #include "physics.cuh"
 #include "reduce.cuh"
 #include "sweep32.cuh"
@@ -27,254 +13,127 @@ namespace {
 
 constexpr int kMaxThreads = 768;
 
-__device__ __forceinline__ float3 zero3t() { return make_float3(0.f, 0.f, 0.f); }
-
-// Rod extents: NXC > 0 at compile time, else from the kernel parameters.
-template <int NXC, int NYC, int NZC>
-struct RodDims {
-    int nx_, ny_, nz_;
-    __device__ __forceinline__ int nx() const { if constexpr (NXC > 0) return NXC; return nx_; }
-    __device__ __forceinline__ int ny() const { if constexpr (NYC > 0) return NYC; return ny_; }
-    __device__ __forceinline__ int nz() const { if constexpr (NZC > 0) return NZC; return nz_; }
-    __device__ __forceinline__ int ncell() const { return nx() * ny() * nz(); }
-    __device__ __forceinline__ int sy() const { return nx() + 2; }
-    __device__ __forceinline__ int sz() const { return (nx() + 2) * (ny() + 2); }
-    __device__ __forceinline__ int pad() const { return sz() * (nz() + 2); }
-    // position of cell c (x + nx (y + ny z)) in a ghost-padded rod
-    __device__ __forceinline__ int at(int c) const
-    {
-        const int x = c % nx(), y = (c / nx()) % ny(), z = c / (nx() * ny());
-        return (x + 1) + sy() * (y + 1) + sz() * (z + 1);
-    }
-};
-
-// Shared memory: M[tot] and P[tot] float4 (x, y, z, 0), tot = rods_per_cta * padded rod.
-template <int CPT, bool AX, int SHAPE, int NXC, int NYC, int NZC, int MAXT>
-__global__ void __launch_bounds__(MAXT) rod_twophase_kernel(KParams p, float *__restrict__ m_glob, int n_real,
-                                                            int rods_per_cta, long long step0, int n_steps,
-                                                            float *__restrict__ samples, int *__restrict__ status)
-{
-    extern __shared__ float4 sm4[];
-    RodDims<NXC, NYC, NZC> D{p.nx, p.ny, p.nz};
-    const int sy = D.sy(), sz = D.sz();
-    const int rod_pad = D.pad();
-    const int rod0 = blockIdx.x * rods_per_cta;
-    const int nrod = min(rods_per_cta, n_real - rod0);
-    const int tot = rods_per_cta * rod_pad;
-    float4 *M = sm4, *P = sm4 + tot;
-    const int T = blockDim.x;
-    const int ncell = D.ncell();
-    const int cta_cells = nrod * ncell;
-
-    for (int i = threadIdx.x; i < 2 * tot; i += T) sm4[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-    __syncthreads();
-    for (int i = threadIdx.x; i < cta_cells; i += T) {
-        const int rod = i / ncell, c = i - rod * ncell;
-        const float *g = m_glob + ((size_t)(rod0 + rod) * ncell + c) * 3;
-        M[rod * rod_pad + D.at(c)] = make_float4(g[0], g[1], g[2], 0.f);
-    }
-
-    int pidx[CPT];
-    uint32_t cell[CPT], real[CPT];
-    bool act[CPT];
-    float3 uax[CPT];  // easy axes (dispersed-axis mode only)
-#pragma unroll
-    for (int k = 0; k < CPT; ++k) {
-        const int i = threadIdx.x + k * T;
-        act[k] = i < cta_cells;
-        const int ii = act[k] ? i : 0;
-        const int rod = ii / ncell, c = ii - rod * ncell;
-        pidx[k] = rod * rod_pad + D.at(c);
-        cell[k] = (uint32_t)c;
-        real[k] = p.real0 + (uint32_t)(rod0 + rod);
-        uax[k] = zero3t();
-        if constexpr (AX) {
-            if (act[k]) uax[k] = xyz(__ldg(p.axis + (size_t)(rod0 + rod) * ncell + c));
-        }
-    }
-    __syncthreads();
-
-    typename SweepSel<SHAPE>::type field;
-    field.init(step0, p);
-    float Hn = field.value();
-    // steps to the next sample (32-bit countdown; the host keeps sample_every below 2^31)
-    const long long se = p.sample_every;
-    const bool sampling = samples && se > 0;
-    long long k_next = sampling ? step0 / se + 1 : 0;
-    int to_sample = sampling ? (int)(k_next * se - step0) : -1;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = T >> 5;
-
-    // thermal field of the next step, drawn before the barrier that ends the current one
-    float3 hpre[CPT], m[CPT];  // and the cells' own state, which stays in registers
-#pragma unroll
-    for (int k = 0; k < CPT; ++k) m[k] = xyz(M[pidx[k]]);
-#pragma unroll
-    for (int k = 0; k < CPT; ++k) hpre[k] = thermal_field(p.seed, real[k], cell[k], (unsigned long long)step0, p.sigma_bm);
-    unsigned long long n = (unsigned long long)step0;
-    for (int s = 0; s < n_steps; ++s, ++n) {
-        field.inc();
-        const float Hn1 = field.value();
-        float3 t[CPT], s0[CPT], hth[CPT];
-#pragma unroll
-        for (int k = 0; k < CPT; ++k) {
-            if (!act[k]) continue;
-            const int q = pidx[k];
-            hth[k] = hpre[k];
-            float3 nb = add3(xyz(M[q - 1]), xyz(M[q + 1]));
-            nb = add3(nb, xyz(M[q - sy]));
-            nb = add3(nb, xyz(M[q + sy]));
-            nb = add3(nb, xyz(M[q - sz]));
-            nb = add3(nb, xyz(M[q + sz]));
-            const float3 H = effective_field_sel<AX>(nb, m[k], hth[k], p, Hn, uax[k]);
-            s0[k] = llg_torque(m[k], H, p.alpha);
-            t[k] = normalised(axpy(p.neg_dt_g1, s0[k], m[k]));
-            P[q] = pad4(t[k]);
-        }
-        __syncthreads();
-#pragma unroll
-        for (int k = 0; k < CPT; ++k) {
-            if (!act[k]) continue;
-            const int q = pidx[k];
-            float3 nb = add3(xyz(P[q - 1]), xyz(P[q + 1]));
-            nb = add3(nb, xyz(P[q - sy]));
-            nb = add3(nb, xyz(P[q + sy]));
-            nb = add3(nb, xyz(P[q - sz]));
-            nb = add3(nb, xyz(P[q + sz]));
-            const float3 H = effective_field_sel<AX>(nb, t[k], hth[k], p, Hn1, uax[k]);
-            m[k] = normalised(axpy(p.neg_hdt_g1, llg_torque_add(s0[k], t[k], H, p.alpha), m[k]));
-            M[q] = pad4(m[k]);
-            hpre[k] = thermal_field(p.seed, real[k], cell[k], n + 1, p.sigma_bm);
-        }
-        __syncthreads();
-        Hn = Hn1;
-        if (--to_sample == 0) {
-            // M now holds the state after step n; the next phase only reads M until the
-            // barrier that precedes its next write, so no extra barrier is needed here.
-            to_sample = (int)se;
-            const long long k = k_next++;
-            if (k < p.n_samples) {
-                for (int rod = warp; rod < nrod; rod += nwarps) {
-                    float part = 0.f;
-                    for (int c = lane; c < ncell; c += 32) part += M[rod * rod_pad + D.at(c)].z;
-                    const float mean = warp_cell_mean(part, ncell);
-                    if (lane == 0) {
-                        samples[(size_t)(rod0 + rod) * p.n_samples + k] = mean;
-                        if (!isfinite(mean)) atomicOr(status, 1);
-                    }
-                }
-            }
-        }
-    }
-
-    for (int i = threadIdx.x; i < cta_cells; i += T) {
-        const int rod = i / ncell, c = i - rod * ncell;
-        const float4 v = M[rod * rod_pad + D.at(c)];
-        float *g = m_glob + ((size_t)(rod0 + rod) * ncell + c) * 3;
-        g[0] = v.x;
-        g[1] = v.y;
-        g[2] = v.z;
-    }
-}
-
 // ------------------------------------------------------------------------------------------
-// Row kernel (the b = 2, 4, 8 rods: 4x12x28, 2x6x14, 1x3x7 cells, shapes at compile time).  A
-// thread owns one x-row (fixed y, z) of NX cells and keeps the row's state, predictor, torque
-// and thermal field in registers; the x-neighbours come from registers, the y- and
-// z-neighbours from shared memory.  Shared memory holds per rod, for each x, a plane of rows
-// (y, z) with ghost lines at y = -1, NY and z = -1, NZ: M[x][(z + 1)(NY + 2) + y + 1] and the same
-// for the predictor P, so consecutive threads (consecutive y) read consecutive float4s.  Per
-// step: predictor of the row into P, barrier, corrector into M, next thermal fields, barrier --
-// 8 shared loads per cell-step where the ghost-padded one-cell-per-thread layout needed 14.
-// The row's cells share their rod's Philox round keys, computed once per thread.
+// Row kernel (the b = 2 and 4 rods: 4x12x28, 2x6x14 cells, shapes at compile time) on pairs of cells
+// with the packed FP32 instructions (pair.cuh).  A thread owns one x-row (fixed y, z) of a rod, NX / 2
+// pairs of x-neighbours; it keeps the row's state, predictor, torque and thermal field in registers.
+// The x-neighbours come from registers, the y- and z-neighbours, whole pairs, from shared memory, which
+// holds per rod NX / 2 planes of pairs for the state M and for the predictor P: (xa, xb, ya, yb) in one
+// array and (za, zb) in another, 24 bytes a pair, the rows of a plane in order with a line of zeros
+// before the first plane and after every plane; the y faces are 0/1 weights, so that consecutive threads
+// read consecutive entries without gaps (with ghost columns in y the b = 4 rod's neighbour loads took
+// twice their wavefronts and shared memory was 78 % busy).  Per step: thermal fields and the predictor of
+// the row into P, barrier, corrector into M, barrier.
+//
+// What bounds it: the heavy FMA pipe, 61 % busy with 608 b = 4 rods (the noise's 32-bit multiplies and
+// half of every packed operation), and the two barriers' chains between (three warps a scheduler).
+// 608 b = 4 rods 0.87 us a step (1.03 with one cell an instruction), 1216 1.61 (1.83), four alone 0.51
+// (0.71); 152 b = 2 rods 1.57 (1.77).  Drawing the next step's noise beside the corrector: 0.88, 0.54
+// and 1.73.
 // ------------------------------------------------------------------------------------------
 template <int NX, int NY, int NZ, int SHAPE, bool AX, int MAXT>
 __global__ void __launch_bounds__(MAXT) rod_rows_kernel(KParams p, float *__restrict__ m_glob, int n_real,
                                                         int rods_per_cta, long long step0, int n_steps,
                                                         float *__restrict__ samples, int *__restrict__ status)
 {
-    constexpr int PY = NY + 2;                   // pitch of a row plane (ghost columns in y)
-    constexpr int PLANE = (NZ + 2) * PY;         // one x-plane with ghost lines
-    constexpr int ROD = NX * PLANE;              // one buffer of one rod
+    constexpr int NXP = NX / 2;                    // pairs of a row
+    constexpr int PL = (NZ + 1) * NY;              // a plane and the ghost line after it
+    constexpr int ROD = NXP * PL + NY;             // entries of one buffer of one rod
     constexpr int ROWS = NY * NZ, NCELL = NX * ROWS;
-    extern __shared__ float4 sm4[];
+    static_assert(NX % 2 == 0, "rows of pairs");
+    extern __shared__ __align__(16) unsigned char rsm[];
     const int rod0 = blockIdx.x * rods_per_cta;
     const int nrod = min(rods_per_cta, n_real - rod0);
-    float4 *M = sm4, *P = sm4 + rods_per_cta * ROD;
+    const int tot = rods_per_cta * ROD;
+    ulonglong2 *MA = reinterpret_cast<ulonglong2 *>(rsm), *PA = MA + tot;
+    pair_t *MB = reinterpret_cast<pair_t *>(PA + tot), *PB = MB + tot;
     const int T = blockDim.x;
-    for (int i = threadIdx.x; i < 2 * rods_per_cta * ROD; i += T) sm4[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int i = threadIdx.x; i < tot; i += T) {
+        MA[i] = PA[i] = make_ulonglong2(0ull, 0ull);
+        MB[i] = PB[i] = 0ull;
+    }
     __syncthreads();
     // this thread's row
-    const int t = threadIdx.x;
-    const int rl = t / ROWS, row = t - rl * ROWS;  // rod within the CTA, row y + NY z
-    const bool act = t < nrod * ROWS;
-    const int y = row % NY, z = row / NY;
-    const int q = rl * ROD + (z + 1) * PY + (y + 1);  // row position in plane x = 0 of its rod
-    const uint32_t cbase = (uint32_t)(row * NX);      // cell index of x = 0: x + NX (y + NY z)
-    const uint32_t real = p.real0 + (uint32_t)(rod0 + rl);
-    float3 m[NX], u[NX];
+    const int t0 = threadIdx.x;
+    const bool act = t0 < nrod * ROWS;
+    const int rl = act ? t0 / ROWS : 0, row = act ? t0 - rl * ROWS : 0;  // rod within the CTA, row y + NY z
+    const int y = row % NY;
+    const int q = rl * ROD + NY + row;             // entry of the row's first pair
+    const pair_t wm = both(y > 0 ? 1.f : 0.f), wp = both(y < NY - 1 ? 1.f : 0.f);
+    auto load = [](const ulonglong2 *A, const pair_t *B, int i) {
+        const ulonglong2 v = A[i];
+        return Pair3{v.x, v.y, B[i]};
+    };
+    auto store = [](ulonglong2 *A, pair_t *B, int i, Pair3 v) {
+        A[i] = make_ulonglong2(v.x, v.y);
+        B[i] = v.z;
+    };
+    Pair3 m[NXP], u[NXP];
 #pragma unroll
-    for (int x = 0; x < NX; ++x) {
-        m[x] = u[x] = zero3t();
+    for (int X = 0; X < NXP; ++X) {
+        m[X] = u[X] = zero_p3();
         if (act) {
-            const float *g = m_glob + ((size_t)(rod0 + rl) * NCELL + cbase + x) * 3;
-            m[x] = make_float3(g[0], g[1], g[2]);
-            M[q + x * PLANE] = pad4(m[x]);
-            if constexpr (AX) u[x] = xyz(__ldg(p.axis + (size_t)(rod0 + rl) * NCELL + cbase + x));
+            const size_t c = (size_t)(rod0 + rl) * NCELL + row * NX + 2 * X;
+            const float *g = m_glob + 3 * c;
+            m[X] = pair3(make_float3(g[0], g[1], g[2]), make_float3(g[3], g[4], g[5]));
+            store(MA, MB, q + X * PL, m[X]);
+            if constexpr (AX) u[X] = pair3(xyz(__ldg(p.axis + c)), xyz(__ldg(p.axis + c + 1)));
         }
     }
-    const PhiloxKeys keys = philox_keys(p.seed, act ? real : p.real0);
+    const PairCoeffs cf = pair_coeffs(p);
+    const PhiloxKeys keys = philox_keys(p.seed, p.real0 + (uint32_t)(rod0 + rl));
+    const unsigned long long row_m0 = (unsigned long long)kPhiloxM0 * (uint32_t)(row * NX);
     __syncthreads();
 
-    typename SweepSel<SHAPE>::type field;
-    field.init(step0, p);
-    float Hn = field.value();
+    FieldAhead<SHAPE> field;
+    field.init(step0);
+    float Hn = field.next(p);
     const long long se = p.sample_every;
     const bool sampling = samples && se > 0;
     long long k_next = sampling ? step0 / se + 1 : 0;
     int to_sample = sampling ? (int)(k_next * se - step0) : -1;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = T >> 5;
 
-    // thermal field of the next step, drawn before the barrier that ends the current one
-    float3 hpre[NX];
-#pragma unroll
-    for (int x = 0; x < NX; ++x) hpre[x] = thermal_field(keys, cbase + x, (unsigned long long)step0, p.sigma_bm);
+    // x- + x+ of pair X of a row
+    auto x_sum = [](const Pair3 *v, int X) {
+        const float3 none = make_float3(0.f, 0.f, 0.f);
+        const float3 l = X > 0 ? hi3(v[X > 0 ? X - 1 : 0]) : none, r = X + 1 < NXP ? lo3(v[X + 1 < NXP ? X + 1 : X]) : none;
+        const float3 a = X > 0 ? add3(l, hi3(v[X])) : hi3(v[X]), b = X + 1 < NXP ? add3(lo3(v[X]), r) : lo3(v[X]);
+        return pair3(a, b);
+    };
+    auto neighbour_sum = [&](const Pair3 *v, int X, const ulonglong2 *A, const pair_t *B) {
+        const int i = q + X * PL;
+        Pair3 nb = axpy_p3(wm, load(A, B, i - 1), x_sum(v, X));
+        nb = axpy_p3(wp, load(A, B, i + 1), nb);
+        nb = add_p3(nb, load(A, B, i - NY));
+        return add_p3(nb, load(A, B, i + NY));
+    };
     unsigned long long n = (unsigned long long)step0;
     for (int s = 0; s < n_steps; ++s, ++n) {
-        field.inc();
-        const float Hn1 = field.value();
-        float3 mt[NX], s0[NX], hth[NX];
+        const float Hn1 = field.next(p);
+        Pair3 t[NXP], s0[NXP], h[NXP];
         if (act) {
+            const PhiloxStep now = philox_step(keys, n);
+            const pair_t H0 = both(Hn);
 #pragma unroll
-            for (int x = 0; x < NX; ++x) {
-                const float4 *Mx = M + q + x * PLANE;
-                hth[x] = hpre[x];
-                float3 nb = add3(x > 0 ? m[x - 1] : zero3t(), x + 1 < NX ? m[x + 1] : zero3t());
-                nb = add3(nb, xyz(Mx[-1]));
-                nb = add3(nb, xyz(Mx[1]));
-                nb = add3(nb, xyz(Mx[-PY]));
-                nb = add3(nb, xyz(Mx[PY]));
-                const float3 H = effective_field_sel<AX>(nb, m[x], hth[x], p, Hn, u[x]);
-                s0[x] = llg_torque(m[x], H, p.alpha);
-                mt[x] = normalised(axpy(p.neg_dt_g1, s0[x], m[x]));
-                P[q + x * PLANE] = pad4(mt[x]);
+            for (int X = 0; X < NXP; ++X) {
+                h[X] = thermal_field_p3(keys, now, row_m0 + (unsigned long long)kPhiloxM0 * (2 * X), p.sigma_bm);
+                const Pair3 nb = neighbour_sum(m, X, MA, MB);
+                s0[X] = llg_torque_p3(m[X], effective_field_p3<AX>(nb, m[X], h[X], cf, H0, u[X]), cf.alpha);
+                t[X] = normalised_p3(axpy_p3(cf.neg_dt_g1, s0[X], m[X]));
+                store(PA, PB, q + X * PL, t[X]);
             }
         }
         __syncthreads();
         if (act) {
+            const pair_t H1 = both(Hn1);
 #pragma unroll
-            for (int x = 0; x < NX; ++x) {
-                const float4 *Px = P + q + x * PLANE;
-                float3 nb = add3(x > 0 ? mt[x - 1] : zero3t(), x + 1 < NX ? mt[x + 1] : zero3t());
-                nb = add3(nb, xyz(Px[-1]));
-                nb = add3(nb, xyz(Px[1]));
-                nb = add3(nb, xyz(Px[-PY]));
-                nb = add3(nb, xyz(Px[PY]));
-                const float3 H = effective_field_sel<AX>(nb, mt[x], hth[x], p, Hn1, u[x]);
-                m[x] = normalised(axpy(p.neg_hdt_g1, llg_torque_add(s0[x], mt[x], H, p.alpha), m[x]));
-                M[q + x * PLANE] = pad4(m[x]);
+            for (int X = 0; X < NXP; ++X) {
+                const Pair3 nb = neighbour_sum(t, X, PA, PB);
+                const Pair3 sv = llg_torque_add_p3(s0[X], t[X], effective_field_p3<AX>(nb, t[X], h[X], cf, H1, u[X]), cf.alpha);
+                m[X] = normalised_p3(axpy_p3(cf.neg_hdt_g1, sv, m[X]));
+                store(MA, MB, q + X * PL, m[X]);
             }
-#pragma unroll
-            for (int x = 0; x < NX; ++x) hpre[x] = thermal_field(keys, cbase + x, n + 1, p.sigma_bm);
         }
         __syncthreads();
         Hn = Hn1;
@@ -285,10 +144,12 @@ __global__ void __launch_bounds__(MAXT) rod_rows_kernel(KParams p, float *__rest
             const long long k = k_next++;
             if (k < p.n_samples) {
                 for (int r = warp; r < nrod; r += nwarps) {
+                    const pair_t *B = MB + r * ROD + NY;
                     float part = 0.f;
                     for (int c = lane; c < NCELL; c += 32) {
                         const int cx = c % NX, cr = c / NX;
-                        part += M[r * ROD + cx * PLANE + (cr / NY + 1) * PY + (cr % NY + 1)].z;
+                        const pair_t v = B[(cx >> 1) * PL + cr];
+                        part += cx & 1 ? hi2(v) : lo2(v);
                     }
                     const float mean = warp_cell_mean(part, NCELL);
                     if (lane == 0) {
@@ -301,12 +162,107 @@ __global__ void __launch_bounds__(MAXT) rod_rows_kernel(KParams p, float *__rest
     }
     if (act) {
 #pragma unroll
-        for (int x = 0; x < NX; ++x) {
-            float *g = m_glob + ((size_t)(rod0 + rl) * NCELL + cbase + x) * 3;
-            g[0] = m[x].x;
-            g[1] = m[x].y;
-            g[2] = m[x].z;
+        for (int X = 0; X < NXP; ++X) {
+            const size_t c = (size_t)(rod0 + rl) * NCELL + row * NX + 2 * X;
+            float *g = m_glob + 3 * c;
+            const float3 a = lo3(m[X]), b = hi3(m[X]);
+            g[0] = a.x;
+            g[1] = a.y;
+            g[2] = a.z;
+            g[3] = b.x;
+            g[4] = b.y;
+            g[5] = b.z;
         }
+    }
+}
+
+// The same for rods one cell wide (the b = 8 rod, 1x3x7 cells): a thread is a cell, there are no pairs
+// of neighbours to take, and several rods share a CTA's warps.  Two rods to a packed thread measured
+// slower (four alone 0.47 us a step against 0.37, 4096 0.84 against 0.85): half the warps hide less of
+// the chain.  Float4 cells in the row kernel's gapless order.
+template <int NY, int NZ, int SHAPE, bool AX, int MAXT>
+__global__ void __launch_bounds__(MAXT) rod_cells_kernel(KParams p, float *__restrict__ m_glob, int n_real,
+                                                         int rods_per_cta, long long step0, int n_steps,
+                                                         float *__restrict__ samples, int *__restrict__ status)
+{
+    constexpr int NCELL = NY * NZ, ROD = NCELL + 2 * NY;
+    extern __shared__ __align__(16) float4 csm[];
+    const int rod0 = blockIdx.x * rods_per_cta;
+    const int nrod = min(rods_per_cta, n_real - rod0);
+    const int tot = rods_per_cta * ROD;
+    float4 *M = csm, *P = csm + tot;
+    const int T = blockDim.x;
+    for (int i = threadIdx.x; i < 2 * tot; i += T) csm[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+    __syncthreads();
+    const int t0 = threadIdx.x;
+    const bool act = t0 < nrod * NCELL;
+    const int rl = act ? t0 / NCELL : 0, c = act ? t0 - rl * NCELL : 0;
+    const int y = c % NY, q = rl * ROD + NY + c;
+    const float wm = y > 0 ? 1.f : 0.f, wp = y < NY - 1 ? 1.f : 0.f;
+    float *g = m_glob + ((size_t)(rod0 + rl) * NCELL + c) * 3;
+    float3 m = make_float3(0.f, 0.f, 0.f), u = make_float3(0.f, 0.f, 1.f);
+    if (act) {
+        m = make_float3(g[0], g[1], g[2]);
+        M[q] = pad4(m);
+        if constexpr (AX) u = xyz(__ldg(p.axis + (size_t)(rod0 + rl) * NCELL + c));
+    }
+    const PhiloxKeys keys = philox_keys(p.seed, p.real0 + (uint32_t)(rod0 + rl));
+    const unsigned long long cell_m0 = (unsigned long long)kPhiloxM0 * (uint32_t)c;
+    __syncthreads();
+    FieldAhead<SHAPE> field;
+    field.init(step0);
+    float Hn = field.next(p);
+    const long long se = p.sample_every;
+    const bool sampling = samples && se > 0;
+    long long k_next = sampling ? step0 / se + 1 : 0;
+    int to_sample = sampling ? (int)(k_next * se - step0) : -1;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = T >> 5;
+    // the neighbour sum in every engine's order (x- + x+ = 0)
+    auto neighbour_sum = [&](const float4 *A) {
+        const float3 l = xyz(A[q - 1]);
+        float3 nb = make_float3(wm * l.x, wm * l.y, wm * l.z);
+        nb = axpy(wp, xyz(A[q + 1]), nb);
+        nb = add3(nb, xyz(A[q - NY]));
+        return add3(nb, xyz(A[q + NY]));
+    };
+    unsigned long long n = (unsigned long long)step0;
+    for (int s = 0; s < n_steps; ++s, ++n) {
+        const float Hn1 = field.next(p);
+        float3 t = m, s0 = m, h = m;
+        if (act) {
+            h = box_muller3(philox4x32_10(keys, philox_step(keys, n), cell_m0), p.sigma_bm);
+            s0 = llg_torque(m, effective_field_sel<AX>(neighbour_sum(M), m, h, p, Hn, u), p.alpha);
+            t = normalised(axpy(p.neg_dt_g1, s0, m));
+            P[q] = pad4(t);
+        }
+        __syncthreads();
+        if (act) {
+            const float3 sv = llg_torque_add(s0, t, effective_field_sel<AX>(neighbour_sum(P), t, h, p, Hn1, u), p.alpha);
+            m = normalised(axpy(p.neg_hdt_g1, sv, m));
+            M[q] = pad4(m);
+        }
+        __syncthreads();
+        Hn = Hn1;
+        if (--to_sample == 0) {
+            to_sample = (int)se;
+            const long long k = k_next++;
+            if (k < p.n_samples) {
+                for (int r = warp; r < nrod; r += nwarps) {
+                    float part = 0.f;
+                    for (int i = lane; i < NCELL; i += 32) part += M[r * ROD + NY + i].z;
+                    const float mean = warp_cell_mean(part, NCELL);
+                    if (lane == 0) {
+                        samples[(size_t)(rod0 + r) * p.n_samples + k] = mean;
+                        if (!isfinite(mean)) atomicOr(status, 1);
+                    }
+                }
+            }
+        }
+    }
+    if (act) {
+        g[0] = m.x;
+        g[1] = m.y;
+        g[2] = m.z;
     }
 }
 
@@ -321,32 +277,19 @@ cudaError_t launch(K kern, const KParams &p, const RodPlan &plan, float *m, int 
     return cudaGetLastError();
 }
 
-// the compile-time rod shape and sweep shape instance, CPT cells per thread
-template <int CPT, int NX, int NY, int NZ>
-cudaError_t launch_shaped(const KParams &p, const RodPlan &plan, float *m, int n_real, long long step0, int n_steps,
-                          float *samples, int *status, cudaStream_t st)
-{
-    constexpr int MAXT = kMaxThreads / CPT;
-    if (p.axis)
-        return p.shape == 1 ? launch(rod_twophase_kernel<CPT, true, 1, NX, NY, NZ, MAXT>, p, plan, m, n_real, step0,
-                                     n_steps, samples, status, st)
-                            : launch(rod_twophase_kernel<CPT, true, 0, NX, NY, NZ, MAXT>, p, plan, m, n_real, step0,
-                                     n_steps, samples, status, st);
-    return p.shape == 1 ? launch(rod_twophase_kernel<CPT, false, 1, NX, NY, NZ, MAXT>, p, plan, m, n_real, step0,
-                                 n_steps, samples, status, st)
-                        : launch(rod_twophase_kernel<CPT, false, 0, NX, NY, NZ, MAXT>, p, plan, m, n_real, step0,
-                                 n_steps, samples, status, st);
-}
-
-template <int CPT>
-cudaError_t launch_generic(const KParams &p, const RodPlan &plan, float *m, int n_real, long long step0, int n_steps,
-                           float *samples, int *status, cudaStream_t st)
+template <int NY, int NZ, int MAXT>
+cudaError_t launch_cells(const KParams &p, const RodPlan &plan, float *m, int n_real, long long step0, int n_steps,
+                         float *samples, int *status, cudaStream_t st)
 {
     if (p.axis)
-        return launch(rod_twophase_kernel<CPT, true, -1, 0, 0, 0, kMaxThreads>, p, plan, m, n_real, step0, n_steps,
-                      samples, status, st);
-    return launch(rod_twophase_kernel<CPT, false, -1, 0, 0, 0, kMaxThreads>, p, plan, m, n_real, step0, n_steps,
-                  samples, status, st);
+        return p.shape == 1 ? launch(rod_cells_kernel<NY, NZ, 1, true, MAXT>, p, plan, m, n_real, step0, n_steps, samples,
+                                     status, st)
+                            : launch(rod_cells_kernel<NY, NZ, 0, true, MAXT>, p, plan, m, n_real, step0, n_steps, samples,
+                                     status, st);
+    return p.shape == 1 ? launch(rod_cells_kernel<NY, NZ, 1, false, MAXT>, p, plan, m, n_real, step0, n_steps, samples,
+                                 status, st)
+                        : launch(rod_cells_kernel<NY, NZ, 0, false, MAXT>, p, plan, m, n_real, step0, n_steps, samples,
+                                 status, st);
 }
 
 template <int NX, int NY, int NZ, int MAXT>
@@ -382,13 +325,21 @@ bool rows_supported(const KParams &p)
            p.sample_every < (1LL << 31);
 }
 
-// Largest CTA of the rows kernel: 768 threads (85 registers) for rows of 1 or 2 cells, 384 (170
+// Largest CTA of the rows kernel: 768 threads (80 registers) for rows of 1 or 2 cells, 384 (168
 // registers) for the 4-cell rows of the b = 2 rod.
 int rows_max_threads(const KParams &p) { return p.nx == 4 ? 384 : kMaxThreads; }
 
+// What a request for rods per CTA may ask for (ghost-padded float4 rows); rows_smem_bytes, less, is
+// what the launch takes.
 size_t rows_rod_bytes(const KParams &p)
 {
     return (size_t)2 * p.nx * (p.nz + 2) * (p.ny + 2) * sizeof(float4);
+}
+
+size_t rows_smem_bytes(const KParams &p, int rods)
+{
+    if (p.nx == 1) return 32 * (size_t)rods * (p.nz + 2) * p.ny;
+    return 48 * (size_t)rods * ((size_t)(p.nx / 2) * (p.nz + 1) * p.ny + p.ny);
 }
 
 cudaError_t rows_advance(const KParams &p, const RodPlan &plan, float *m, int n_real, long long step0, int n_steps,
@@ -400,56 +351,19 @@ cudaError_t rows_advance(const KParams &p, const RodPlan &plan, float *m, int n_
         case 4:
             return launch_rows_shaped<2, 6, 14, kMaxThreads>(p, plan, m, n_real, step0, n_steps, samples, status, st);
         case 8:
-            return launch_rows_shaped<1, 3, 7, kMaxThreads>(p, plan, m, n_real, step0, n_steps, samples, status, st);
+            return launch_cells<3, 7, kMaxThreads>(p, plan, m, n_real, step0, n_steps, samples, status, st);
         default:
             return cudaErrorInvalidValue;
     }
 }
 
-// Largest CTA of a two-phase instance: the compile-time-shape instances (b = 4 and b = 8 rods)
-// give CPT cells per thread a register budget of 768 / CPT threads; the runtime-shape instance
-// keeps 768 threads for every CPT.
+// Largest CTA that a request for cpt cells per thread may ask for (the b = 4 and b = 8 rods 768 / cpt
+// threads, other grids 768); what it asks for beyond that is refused.
 int twophase_max_threads(const KParams &p, int cpt)
 {
-    return twophase_shaped(p) ? kMaxThreads / cpt : kMaxThreads;
-}
-
-bool twophase_shaped(const KParams &p)
-{
     const bool b4 = p.nx == 2 && p.ny == 6 && p.nz == 14, b8 = p.nx == 1 && p.ny == 3 && p.nz == 7;
-    const long long period = p.shape == 1 ? p.period : 2 * p.n_half;
-    return (b4 || b8) && (p.shape == 0 || p.shape == 1) && period < (1LL << 31) && p.sample_every < (1LL << 31);
-}
-
-cudaError_t twophase_advance(const KParams &p, const RodPlan &plan, float *m, int n_real, long long step0,
-                             int n_steps, float *samples, int *status, cudaStream_t st)
-{
-    if (twophase_shaped(p)) {
-        const bool b4 = p.nx == 2;
-        switch (plan.cells_per_thread) {
-            case 1:
-                return b4 ? launch_shaped<1, 2, 6, 14>(p, plan, m, n_real, step0, n_steps, samples, status, st)
-                          : launch_shaped<1, 1, 3, 7>(p, plan, m, n_real, step0, n_steps, samples, status, st);
-            case 2:
-                return b4 ? launch_shaped<2, 2, 6, 14>(p, plan, m, n_real, step0, n_steps, samples, status, st)
-                          : launch_shaped<2, 1, 3, 7>(p, plan, m, n_real, step0, n_steps, samples, status, st);
-            case 4:
-                return b4 ? launch_shaped<4, 2, 6, 14>(p, plan, m, n_real, step0, n_steps, samples, status, st)
-                          : launch_shaped<4, 1, 3, 7>(p, plan, m, n_real, step0, n_steps, samples, status, st);
-            default:
-                return cudaErrorInvalidValue;
-        }
-    }
-    switch (plan.cells_per_thread) {
-        case 1:
-            return launch_generic<1>(p, plan, m, n_real, step0, n_steps, samples, status, st);
-        case 2:
-            return launch_generic<2>(p, plan, m, n_real, step0, n_steps, samples, status, st);
-        case 4:
-            return launch_generic<4>(p, plan, m, n_real, step0, n_steps, samples, status, st);
-        default:
-            return cudaErrorInvalidValue;
-    }
+    const bool shaped = (b4 || b8) && sweep_fits_32(p) && p.sample_every < (1LL << 31);
+    return shaped ? kMaxThreads / cpt : kMaxThreads;
 }
 
 }  // namespace llg

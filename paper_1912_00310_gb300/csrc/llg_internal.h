@@ -113,7 +113,8 @@ struct RodPlan {
     int rods_per_cta;  // kind 1
     int threads;
     int rows_per_thread;  // kind 2
-    int cells_per_thread; // kind 1
+    int cells_per_thread; // kind 1: as asked for (the launch takes pairs_per_thread from the sizes)
+    int pairs_per_thread = 0;  // kind 1
     size_t smem_bytes;
     int ctas;
     bool generic = false;  // kind 2: use the runtime-nx kernel even where a specialised one exists
@@ -126,14 +127,17 @@ struct RodPlan {
 // force_kind / force_rods: 0 = automatic.
 bool rod_plan(const KParams &p, int n_real, int dev, RodPlan *plan, int force_kind = 0,
               int force_rods = 0, int force_rows = 0, int force_cpt = 0);
-// Two-phase kernel (k_rod_small.cu): whether the grid and sweep have a compile-time instance,
-// the largest CTA for cpt cells per thread, and the launch of n_steps (< 2^31) steps.
-bool twophase_shaped(const KParams &p);
+// Two-phase kernel (k_rod_zpairs.cu): shared memory of one rod, the pairs per thread and threads of
+// `rods` rods in a CTA (false: too many), the largest CTA of a request for cpt cells per thread, and
+// the launch of n_steps (< 2^31) steps.
+size_t twophase_rod_bytes(const KParams &p);
+bool twophase_shape(const KParams &p, int rods, RodPlan *plan);
 // Row kernel (k_rod_small.cu, plan kind 3): the b = 2, 4, 8 rods with a compile-time instance,
 // its largest CTA, the shared memory of one rod, and the launch.
 bool rows_supported(const KParams &p);
 int rows_max_threads(const KParams &p);
 size_t rows_rod_bytes(const KParams &p);
+size_t rows_smem_bytes(const KParams &p, int rods);  // shared memory of a CTA of that many rods
 cudaError_t rows_advance(const KParams &p, const RodPlan &plan, float *m, int n_real, long long step0, int n_steps,
                          float *samples, int *status, cudaStream_t st);
 // Pair kernel (k_rod_pairs.cu, plan kind 2): rods eight cells wide; flags as for rod_advance.  Its

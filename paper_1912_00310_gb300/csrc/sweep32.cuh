@@ -52,6 +52,36 @@ struct SweepSel<-1> {
     using type = Sweep;
 };
 
+// The field of consecutive steps, 32 at a time: lane l of a warp evaluates the step l ahead, and each
+// step's value is broadcast from its lane.  The sinusoid's cosine is some forty instructions, which every
+// thread of a small rod otherwise spends every step (4096 b = 8 rods with the sinusoid and dispersed
+// axes: 0.93 us a step).  The values are the sweep's own: its phase is n mod period either way.  A warp's
+// lanes call next() together.
+template <int SHAPE>
+struct FieldAhead {
+    float v;
+    int i;
+    long long n;  // step of the next value
+
+    __device__ __forceinline__ void init(long long step)
+    {
+        n = step;
+        i = 32;
+        v = 0.f;
+    }
+    __device__ __forceinline__ float next(const KParams &p)
+    {
+        if (i == 32) {
+            typename SweepSel<SHAPE>::type f;
+            f.init(n + (threadIdx.x & 31), p);
+            v = f.value();
+            n += 32;
+            i = 0;
+        }
+        return __shfl_sync(0xffffffffu, v, i++);
+    }
+};
+
 // Whether the 32-bit instances cover a sweep: its period (or the held field's zero) below 2^31.
 inline bool sweep_fits_32(const KParams &p)
 {

@@ -19,13 +19,13 @@ def pkg():
     return P
 
 
-def ensemble(pkg, dims, n_real, *, b=1, dt=2e-15, disp=0.0, shape=0, rate=10000.0, steps=(113, 37), tune=(), plain=False,
-             seed=5):
+def ensemble(pkg, dims, n_real, *, b=1, dt=2e-15, disp=0.0, shape=0, rate=10000.0, sample_dH=1.0, steps=(113, 37), tune=(),
+             plain=False, seed=5):
     """State and samples after `steps` (one advance each) from +z."""
     g = pkg.Grid(*dims, a0=M["a0"], b=b)
     g.set_material(A0=M["A0"], Ms=M["Ms"], K0=M["K0"], alpha=M["alpha"], T=M["T"])
     g.set_scaling(mode=1, Tc=M["Tc"])
-    g.set_sweep(H_start=1500.0, H_turn=-1500.0, rate=rate, dt=dt, sample_dH=1.0, shape=shape)
+    g.set_sweep(H_start=1500.0, H_turn=-1500.0, rate=rate, dt=dt, sample_dH=sample_dH, shape=shape)
     g.set_axis_dispersion(disp)
     g.set_engine(pkg.ENGINE_PLAIN if plain else pkg.ENGINE_RESIDENT)
     for key, value in tune:
@@ -61,3 +61,39 @@ def test_eight_wide_rods_equal_plain_engine(pkg, dims, disp, shape):
         assert torch.equal(m, ref) and torch.equal(s, ref_s), rows
         ran += 1
     assert ran >= 4
+
+
+@pytest.mark.parametrize("dims", [(1, 1, 1), (1, 1, 2), (1, 1, 9), (3, 1, 4), (4, 3, 1), (2, 2, 2), (1, 3, 7), (2, 6, 14),
+                                  (5, 11, 23), (7, 5, 6), (3, 2, 65), (9, 16, 20), (16, 21, 9)])
+@pytest.mark.parametrize("disp,shape", [(0.0, 0), (0.3, 1)])
+def test_two_phase_rods_equal_plain_engine(pkg, dims, disp, shape):
+    """The two-phase kernel on pairs across the rod's halves: even and odd nz (a last line without its
+    upper cells), flat and thin grids (the pair axis moves to y or x), the single cell, one and several
+    rods per CTA with a partial last CTA, one, two and four pairs per thread."""
+    n_real = 1 if np.prod(dims) > 2000 else 5
+    ref, ref_s = ensemble(pkg, dims, n_real, disp=disp, shape=shape, plain=True)
+    for rods in (0, 3):
+        try:
+            m, s = ensemble(pkg, dims, n_real, disp=disp, shape=shape,
+                            tune=((pkg.TUNE_ROD_KIND, 1), (pkg.TUNE_RODS_PER_CTA, rods)))
+        except pkg.LLGError as e:
+            assert e.status == 6 and rods == 3 and np.prod(dims) > 256  # three do not fit a CTA
+            continue
+        assert torch.equal(m, ref) and torch.equal(s, ref_s), rods
+
+
+@pytest.mark.parametrize("b,dims,dt", [(2, (4, 12, 28), 5e-15), (4, (2, 6, 14), 10e-15), (8, (1, 3, 7), 20e-15)])
+@pytest.mark.parametrize("disp,shape", [(0.0, 0), (0.3, 1)])
+def test_row_kernels_equal_plain_engine(pkg, b, dims, dt, disp, shape):
+    """The b = 2, 4, 8 rods: one and several rods per CTA, the last CTA partly filled; more steps than
+    the 32 whose fields a warp evaluates at once, and a sweep that turns within them."""
+    per_step = 1e7 * 1e9 * dt  # Oe: loops of 120, 60 and 30 steps
+    kw = dict(b=b, dt=dt, disp=disp, shape=shape, rate=1e7, sample_dH=5 * per_step)
+    ref, ref_s = ensemble(pkg, dims, 8, plain=True, **kw)
+    for rods in (0, 1, 3):
+        try:
+            m, s = ensemble(pkg, dims, 8, tune=((pkg.TUNE_ROD_KIND, 3), (pkg.TUNE_RODS_PER_CTA, rods)), **kw)
+        except pkg.LLGError as e:
+            assert e.status == 6 and rods == 3 and b == 2
+            continue
+        assert torch.equal(m, ref) and torch.equal(s, ref_s), rods
