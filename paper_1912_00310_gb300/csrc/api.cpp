@@ -187,7 +187,8 @@ int resolve_engine(const llg_ctx *c, const llg::KParams &kp, int n_real, llg::Ro
                    llg::SlabPlan *splan)
 {
     const bool rod_ok =
-        llg::rod_plan(kp, n_real, c->device, plan, c->tune_kind, c->tune_rods, c->tune_rows, c->tune_cpt);
+        llg::rod_plan(kp, n_real, c->device, plan, c->tune_kind, c->tune_rods, c->tune_rows, c->tune_cpt,
+                       !c->tune_generic && c->tune_balance);
     plan->generic = c->tune_generic != 0;
     plan->balance = c->tune_balance != 0;
     plan->handoff_timeout_ns = (unsigned long long)c->handoff_timeout_ms * 1000000ull;
@@ -840,7 +841,7 @@ llg_status llg_loop_area_grad(llg_ctx *c, int64_t n_steps, int objective, const 
     if (!llg::adjoint_supported(kp, c->device))
         return fail(LLG_EUNSUPPORTED, "the adjoint handles rods of at most 1024 cells with free faces");
     llg::RodPlan plan{};
-    if (!llg::rod_plan(kp, c->n_real, c->device, &plan))
+    if (!llg::rod_plan(kp, c->n_real, c->device, &plan, 0, 0, 0, 0, true))
         return fail(LLG_EUNSUPPORTED, "no resident forward plan for this grid");
     const long long ns_total = std::max<long long>(d.n_samples, k_last + 1);
     // store the whole window's states when they fit the budget and a quarter of the free memory

@@ -152,6 +152,7 @@ extern "C" llg_status llg_autotune(llg_ctx *ctx, int64_t trial_steps, double *be
     }
     // candidates: (kind, rods per CTA, rows per thread, cells per thread); 0 = automatic
     std::vector<std::tuple<int, int, int, int>> cand;
+    cand.emplace_back(0, 0, 0, 0);  // the automatic plan (few rods: several SMs to each)
     for (int rows : {0, 1, 2, 3, 4}) cand.emplace_back(2, 0, rows, 0);
     for (int cpt : {0, 1, 2, 4})
         for (int rods : {0, 1, 2, 3, 4, 6, 8, 12, 16, 24, 32}) cand.emplace_back(1, rods, 0, cpt);
@@ -172,7 +173,7 @@ extern "C" llg_status llg_autotune(llg_ctx *ctx, int64_t trial_steps, double *be
     double best_ms = 0.0;
     for (auto [kind, rods, rows, cpt] : cand) {
         llg::RodPlan plan{};
-        if (!llg::rod_plan(v.kp, v.n_real, v.device, &plan, kind, rods, rows, cpt)) continue;
+        if (!llg::rod_plan(v.kp, v.n_real, v.device, &plan, kind, rods, rows, cpt, true)) continue;
         if (kind == 2 && rows == 0 && plan.kind != 2) continue;
         plan.balance = true;
         double t_best = 1e30;

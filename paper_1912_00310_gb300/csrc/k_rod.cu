@@ -237,7 +237,7 @@ int round_warp(int n) { return (n + 31) / 32 * 32; }
 }  // namespace
 
 bool rod_plan(const KParams &p, int n_real, int dev, RodPlan *plan, int force_kind, int force_rods,
-              int force_rows, int force_cpt)
+              int force_rows, int force_cpt, bool alone)
 {
     int smem_optin = 0, nsm = 0;
     if (cudaDeviceGetAttribute(&smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess ||
@@ -261,6 +261,16 @@ bool rod_plan(const KParams &p, int n_real, int dev, RodPlan *plan, int force_ki
         RodPlan one{};
         const bool pair_each = twophase_fits && twophase_shape(p, 1, &one) && one.pairs_per_thread == 1;
         kind = rows_supported(p) ? 3 : (pair_each ? 1 : (pipelined_fits ? 2 : 1));
+        // few rods: several SMs to each, where that is faster than what a step of one rod on one SM takes
+        // (us, measured: b = 2, 4, 8 rods 1.63, 0.47, 0.38; two-phase rods of 75, 441 and 660 pairs 0.63,
+        // 1.54 and 2.15; the b = 1 rod 11.2; 6x16x30 cells on the runtime-size pipelined kernel 5.4)
+        if (alone && force_rods == 0 && force_rows == 0 && force_cpt == 0 && n_real < nsm) {
+            const double us = kind == 3   ? 0.35 + 0.00095 * p.ncells
+                              : kind == 1 ? 0.42 + 0.0013 * p.ncells
+                              : pairs_supported(p) ? 0.3 + 0.00101 * p.ncells
+                                                   : 0.00186 * p.ncells;
+            if (split_plan(p, n_real, nsm, smem_optin, us, plan)) return true;
+        }
     }
     if (kind == 3) {
         if (!rows_supported(p)) return false;
@@ -362,6 +372,8 @@ cudaError_t rod_advance(const KParams &p, const RodPlan &plan, float *m, int n_r
     if (plan.kind == 1) {
         e = twophase_advance(p, plan, m, n_real, step0, (int)n_steps, samples, status, st);
         if (e != cudaSuccess) return e;
+    } else if (plan.kind == 4) {
+        return split_advance(p, plan, m, n_real, step0, (int)n_steps, samples, status, st);
     } else if (plan.kind == 3) {
         e = rows_advance(p, plan, m, n_real, step0, (int)n_steps, samples, status, st);
         if (e != cudaSuccess) return e;

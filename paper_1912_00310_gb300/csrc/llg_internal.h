@@ -109,12 +109,14 @@ cudaError_t axis_fill(float4 *ax, int n_real, int ncells, uint32_t seed, uint32_
 // ---- resident engine (k_rod.cu): rods in shared memory for the whole launch ------------------
 struct RodPlan {
     int kind;          // 1: two-phase (small rods, several per CTA); 2: plane-pipelined (one per CTA);
-                       // 3: rows (the b = 2, 4, 8 rods, a thread per x-row, several rods per CTA)
+                       // 3: rows (the b = 2, 4, 8 rods, a thread per x-row, several rods per CTA);
+                       // 4: split (a cluster of CTAs per rod)
     int rods_per_cta;  // kind 1
     int threads;
     int rows_per_thread;  // kind 2
     int cells_per_thread; // kind 1: as asked for (the launch takes pairs_per_thread from the sizes)
-    int pairs_per_thread = 0;  // kind 1
+    int pairs_per_thread = 0;  // kinds 1 and 4
+    int split = 0, physics_warps = 0;  // kind 4: CTAs per rod, a CTA's warps without the sampler
     size_t smem_bytes;
     int ctas;
     bool generic = false;  // kind 2: use the runtime-nx kernel even where a specialised one exists
@@ -124,14 +126,20 @@ struct RodPlan {
 };
 // Choose a launch plan for n_real rods of this grid on device `dev`; returns false if no
 // resident kernel can hold the rod.
-// force_kind / force_rods: 0 = automatic.
+// force_kind / force_rods: 0 = automatic.  alone: nothing else is meant to run beside this launch, so
+// that an ensemble of few rods may take several SMs for each (automatic plans only).
 bool rod_plan(const KParams &p, int n_real, int dev, RodPlan *plan, int force_kind = 0,
-              int force_rods = 0, int force_rows = 0, int force_cpt = 0);
+              int force_rods = 0, int force_rows = 0, int force_cpt = 0, bool alone = false);
 // Two-phase kernel (k_rod_zpairs.cu): shared memory of one rod, the pairs per thread and threads of
 // `rods` rods in a CTA (false: too many), the largest CTA of a request for cpt cells per thread, and
 // the launch of n_steps (< 2^31) steps.
 size_t twophase_rod_bytes(const KParams &p);
 bool twophase_shape(const KParams &p, int rods, RodPlan *plan);
+// Split kernel (k_rod_split.cu, plan kind 4): whether and over how many CTAs the rods of an ensemble that
+// leaves SMs idle are cut (base_us: a step's time with one rod per SM), and the launch.
+bool split_plan(const KParams &p, int n_real, int nsm, int smem_optin, double base_us, RodPlan *plan);
+cudaError_t split_advance(const KParams &p, const RodPlan &plan, float *m, int n_real, long long step0, int n_steps,
+                          float *samples, int *status, cudaStream_t st);
 // Row kernel (k_rod_small.cu, plan kind 3): the b = 2, 4, 8 rods with a compile-time instance,
 // its largest CTA, the shared memory of one rod, and the launch.
 bool rows_supported(const KParams &p);

@@ -97,3 +97,18 @@ def test_row_kernels_equal_plain_engine(pkg, b, dims, dt, disp, shape):
             assert e.status == 6 and rods == 3 and b == 2
             continue
         assert torch.equal(m, ref) and torch.equal(s, ref_s), rods
+
+
+@pytest.mark.parametrize("dims,n_real", [((8, 24, 56), 2), ((8, 24, 56), 20), ((8, 24, 56), 40), ((4, 12, 28), 3),
+                                         ((4, 12, 28), 70), ((5, 11, 23), 3), ((7, 9, 13), 2), ((6, 16, 30), 3),
+                                         ((6, 16, 30), 30), ((1, 15, 40), 2), ((3, 30, 20), 2), ((8, 5, 40), 1)])
+@pytest.mark.parametrize("disp,shape", [(0.0, 0), (0.3, 1)])
+def test_rods_cut_over_several_ctas_equal_plain_engine(pkg, dims, n_real, disp, shape):
+    """Few rods: the automatic plan cuts each along z over a cluster of CTAs (2 to 8, even and uneven
+    slabs, odd widths, one to four pairs per thread, more clusters than run at once).  Samples after every
+    step (the snapshots' double buffer and the partial sums' way through the slabs) and every fifth."""
+    for rate, sample_dH, steps in ((1e5, 0.2, (1, 41, 30)), (1e5, 1.0, (113, 37))):
+        kw = dict(disp=disp, shape=shape, rate=rate, sample_dH=sample_dH, steps=steps)
+        ref, ref_s = ensemble(pkg, dims, n_real, plain=True, **kw)
+        m, s = ensemble(pkg, dims, n_real, **kw)
+        assert torch.equal(m, ref) and torch.equal(s, ref_s)
