@@ -193,17 +193,19 @@ int resolve_engine(const llg_ctx *c, const llg::KParams &kp, int n_real, llg::Ro
     plan->balance = c->tune_balance != 0;
     plan->handoff_timeout_ns = (unsigned long long)c->handoff_timeout_ms * 1000000ull;
     plan->withhold_handoff = c->withhold_handoff != 0;
-    llg::SlabPlan tmp;
-    const bool slab_ok = llg::slab_plan(kp, c->device, splan ? splan : &tmp);
+    auto slab_ok = [&]() {  // planned only where it may be taken
+        llg::SlabPlan tmp;
+        return llg::slab_plan(kp, n_real, c->device, splan ? splan : &tmp);
+    };
     switch (c->engine) {
         case LLG_ENGINE_RESIDENT:
             return rod_ok ? LLG_ENGINE_RESIDENT : -1;
         case LLG_ENGINE_PLAIN:
             return LLG_ENGINE_PLAIN;
         case LLG_ENGINE_STREAM:
-            return slab_ok ? LLG_ENGINE_STREAM : -1;
+            return slab_ok() ? LLG_ENGINE_STREAM : -1;
         default:
-            return rod_ok ? LLG_ENGINE_RESIDENT : (slab_ok ? LLG_ENGINE_STREAM : LLG_ENGINE_PLAIN);
+            return rod_ok ? LLG_ENGINE_RESIDENT : (slab_ok() ? LLG_ENGINE_STREAM : LLG_ENGINE_PLAIN);
     }
 }
 

@@ -8,7 +8,8 @@
 // which the Tensor Memory Accelerator copies into shared memory with one instruction (a 5-D
 // tiled box: float component, x, y, z, realisation) -- no per-thread staging, no index wrapping.
 //
-// Each CTA owns an (x, y) tile of columns and sweeps z.  At iteration z it computes, column by
+// Each CTA owns an (x, y) tile of columns and sweeps z, or a part of it with one more predictor
+// plane on either side (films of few columns, slab_plan).  At iteration z it computes, column by
 // column, the predictor of plane z and then the corrector of plane z-1 of the same column (the
 // corrector needs the predictor of its z+ neighbour, which is that column's value just
 // computed), and the predictor of a one-cell ring around the tile (the lateral neighbours the
@@ -27,9 +28,19 @@
 //
 // The arithmetic, the neighbour order (x-, x+, y-, y+, z-, z+) and the noise keys are those of
 // every other engine, so the trajectory is bitwise that of the plain engine on the same grid.
+//
+// What bounds it: 512x512x56 takes 192 us a step on a GB300 (205 before: the noise's first rounds,
+// which depend on the step only, are made once per launch; shorter noise and torque arithmetic; the
+// next launch's set-up runs under the tail of this one).  The state alone is 470 MB there and back,
+// 70 us at the copy rate; the rest is instructions: 260 a warp-cell with the ring's second predictor,
+// issued at 0.58 a cycle by the 16 warps that 128 registers leave an SM, which wait on fixed
+// latencies (1.4 cycles an instruction) and on the barrier of every plane (0.9).  A thread on pairs
+// of columns with packed arithmetic has fewer instructions, but holds both columns' planes in
+// registers: 266 us.
 #include <cuda.h>  // CUtensorMap and its enums; the encoder is fetched from the driver at run time
 
 #include <algorithm>
+#include <cmath>
 #include <cstring>
 
 #include "llg_internal.h"
@@ -100,7 +111,7 @@ __device__ __forceinline__ void tma_load_plane(void *dst, const CUtensorMap *map
 struct SlabGeom {
     int NX, NY, NZ;
     int NXp, NYp;        // padded extents NX + 4, NY + 4
-    int tiles_x, tiles_y;
+    int tiles_x, tiles_y, parts;  // parts: CTAs along z
     int TXmax, TYmax;
     int pitch, rows;     // copied box: (TXmax + 4) x (TYmax + 4) float4
     int slot;            // float4 entries per state slot (box rounded up to 128 bytes)
@@ -121,6 +132,9 @@ struct SlabSweep {
     float4 *Mb, *Tb;     // [3][slot] state planes; [3][tslot] predictor planes (Tb one row early)
     uint64_t *bar;       // [3] one mbarrier per state slot
     int pitch_rt, slot_rt, NZ;
+    // the CTA's part of z: planes [za, zb) get their corrector, [zs, ze) their predictor (one more on either
+    // side), [l0, l1) are staged (one more again)
+    int za, zb, zs, ze, l0, l1;
     bool lead;           // the thread that issues the copies
     int tile_x, tile_y, real;
     const CUtensorMap *tin;
@@ -128,6 +142,7 @@ struct SlabSweep {
     int plane_p;         // float4 entries per padded plane
     uint32_t plane_c;    // cells per interior plane
     PhiloxKeys keys;
+    PhiloxStep now;      // the noise's first rounds for this step
     const float4 *axr;
     float Hn, Hn1;
     unsigned long long n;
@@ -190,6 +205,11 @@ struct SlabSweep {
     unsigned box_bytes;
     int last_issued;  // lead thread: the last plane whose copy was issued
 
+    __device__ __forceinline__ float3 noise(const KParams &p, uint32_t c) const
+    {
+        return box_muller3(philox4x32_10(keys, now, (unsigned long long)kPhiloxM0 * c), p.sigma_bm);
+    }
+
     __device__ __forceinline__ void issue(int z, int s)
     {
         mbar_expect_tx(bar + s, box_bytes);
@@ -198,10 +218,12 @@ struct SlabSweep {
     }
 
     // After a staging wait gave up: let the copies still in flight land before the CTA's shared
-    // memory is released (each wait bounded).  Plane z used its slot for the (z / 3)-th time.
+    // memory is released (each wait bounded).  The CTA's t-th plane (t = z - l0) uses slot t mod 3 for the
+    // (t / 3)-th time.
     __device__ void drain()
     {
-        for (int z = max(0, last_issued - 2); z <= last_issued; ++z) mbar_wait(bar + z % 3, (unsigned)((z / 3) & 1));
+        for (int t = max(0, last_issued - l0 - 2); t <= last_issued - l0; ++t)
+            mbar_wait(bar + t % 3, (unsigned)((t / 3) & 1));
     }
 
     // A column's new state goes to its padded position and, near a periodic face, to the images
@@ -220,26 +242,27 @@ struct SlabSweep {
         }
     }
 
-    // Iteration z of the sweep, z = 3 j + U: predictor of plane z (z < NZ) and corrector of
-    // plane z - 1 (z >= 1).  Ends in a CTA barrier; returns true (in every thread) when some
-    // thread's staging wait gave up.
+    // Iteration t = z - l0 of the sweep, t = 3 j + U: predictor of plane z and corrector of plane z - 1,
+    // where they belong to the CTA's part (a first plane staged only for the predictor above it is just
+    // remembered).  Ends in a CTA barrier; returns true (in every thread) when some thread's staging wait
+    // gave up.
     template <int U>
     __device__ __forceinline__ bool iteration(const KParams &p, int z)
     {
         constexpr int s0 = U % 3, sm1 = (U + 2) % 3, sp1 = (U + 1) % 3;  // slots of planes z, z-1, z+1 (and z-2 = sp1)
-        // plane z+1 is the ((z + 1) / 3)-th use of its slot
-        const unsigned par_next = (unsigned)(((z + 1) / 3) & 1);
+        // plane z+1 is the ((t + 1) / 3)-th use of its slot
+        const unsigned par_next = (unsigned)(((z - l0 + 1) / 3) & 1);
         const int P = pitch();
-        const bool pred = z < NZ, corr = z >= 1;
-        const bool has_next = z + 1 < NZ;
+        const bool pred = z >= zs && z < ze, corr = z > za;
+        const bool has_next = z + 1 < l1;
         int fail = 0;
         // plane z+1, issued an iteration ago
-        if (pred && has_next && !mbar_wait(bar + sp1, par_next)) {
+        if (has_next && !mbar_wait(bar + sp1, par_next)) {
             atomicOr(status, 4);
             fail = 1;
         }
         // plane z+2 into the slot plane z-1 left (freed by the previous iteration's barrier)
-        if (lead && z + 2 < NZ) issue(z + 2, sm1);
+        if (lead && z + 2 < l1) issue(z + 2, sm1);
         const float4 *Mz = Mb + s0 * slot(), *Mn = Mb + sp1 * slot();
         float4 *Tw = Tb + s0 * tslot();
         const float4 *Tr = Tb + sm1 * tslot(), *Tp = Tb + sp1 * tslot();
@@ -254,7 +277,7 @@ struct SlabSweep {
             if (pred) {
                 const float3 mcur = xyz(Mz[c]);
                 const float3 mnext = has_next ? xyz(Mn[c]) : zero3s();
-                h = thermal_field(keys, cell(k) + zoff, n, p.sigma_bm);
+                h = noise(p, cell(k) + zoff);
                 float3 nb = add3(xyz(Mz[c - 1]), xyz(Mz[c + 1]));
                 nb = add3(nb, xyz(Mz[c - P]));
                 nb = add3(nb, xyz(Mz[c + P]));
@@ -285,12 +308,18 @@ struct SlabSweep {
                 A[k] = anew;
             }
         }
+        if (z < zs) {
+#pragma unroll
+            for (int k = 0; k < CPT; ++k)
+                if (act(k)) Sp[k] = xyz(Mz[q(k)]);
+            if (rin) rSp = xyz(Mz[rpos]);
+        }
         if (pred && ract) {
             float3 rt = zero3s();
             if (rin) {
                 const float3 rcur = xyz(Mz[rpos]);
                 const float3 rnext = has_next ? xyz(Mn[rpos]) : zero3s();
-                const float3 h = thermal_field(keys, rcell + zoff, n, p.sigma_bm);
+                const float3 h = noise(p, rcell + zoff);
                 float3 nb = add3(xyz(Mz[rpos - 1]), xyz(Mz[rpos + 1]));
                 nb = add3(nb, xyz(Mz[rpos - P]));
                 nb = add3(nb, xyz(Mz[rpos + P]));
@@ -339,7 +368,13 @@ __global__ void __launch_bounds__(kSlabThreads, 1) slab_step_kernel(KParams p, S
     w.box_bytes = G.box_bytes;
     w.n = n;
     w.status = status;
-    const int tx = blockIdx.x, ty = blockIdx.y, real = blockIdx.z;
+    const int tx = blockIdx.x, ty = blockIdx.y, real = blockIdx.z / G.parts, part = blockIdx.z % G.parts;
+    w.za = (int)((long long)part * G.NZ / G.parts);
+    w.zb = (int)((long long)(part + 1) * G.NZ / G.parts);
+    w.zs = max(0, w.za - 1);
+    w.ze = min(G.NZ, w.zb + 1);
+    w.l0 = max(0, w.zs - 1);
+    w.l1 = min(G.NZ, w.ze + 1);
     const int x0 = (int)((long long)tx * G.NX / G.tiles_x), x1 = (int)((long long)(tx + 1) * G.NX / G.tiles_x);
     const int y0 = (int)((long long)ty * G.NY / G.tiles_y), y1 = (int)((long long)(ty + 1) * G.NY / G.tiles_y);
     const int TX = x1 - x0, TY = y1 - y0;
@@ -351,6 +386,7 @@ __global__ void __launch_bounds__(kSlabThreads, 1) slab_step_kernel(KParams p, S
     w.plane_c = (uint32_t)G.NX * (uint32_t)G.NY;
     w.dst = mout + (size_t)real * (size_t)w.plane_p * G.NZ;
     w.keys = philox_keys(p.seed, p.real0 + (uint32_t)real);
+    w.now = philox_step(w.keys, n);
     w.axr = AX ? p.axis + (size_t)real * w.plane_c * G.NZ : nullptr;
     {
         Sweep sw;
@@ -414,42 +450,51 @@ __global__ void __launch_bounds__(kSlabThreads, 1) slab_step_kernel(KParams p, S
     }
     __syncthreads();
     w.last_issued = -1;
+    // Everything above is this launch's own; the state that the previous step writes, and the buffer that it
+    // still reads, are touched from here on.  The next step's CTAs may set themselves up meanwhile (its wait
+    // is for this whole launch).
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     if (w.lead) {
-        w.issue(0, 0);
-        if (G.NZ > 1) w.issue(1, 1);
+        asm volatile("fence.proxy.async;" ::: "memory");  // the copies read what the step before wrote
+        w.issue(w.l0, 0);
+        if (w.l0 + 1 < w.l1) w.issue(w.l0 + 1, 1);
     }
-    // plane 0 before the sweep starts
+    // the first plane before the sweep starts
     int fail = 0;
     if (!mbar_wait(w.bar, 0u)) {
         atomicOr(status, 4);
         fail = 1;
     }
 #pragma unroll
-    for (int k = 0; k < CPT; ++k) w.Sp[k] = w.A[k] = zero3s();  // plane -1: the free z face
+    for (int k = 0; k < CPT; ++k) w.Sp[k] = w.A[k] = zero3s();  // plane -1 of a first part: the free z face
     w.rSp = zero3s();
     bool aborted = __syncthreads_or(fail) != 0;
-    for (int zz = 0; zz <= G.NZ && !aborted; zz += 3) {
+    for (int zz = w.l0; zz <= w.zb && !aborted; zz += 3) {
         aborted = w.template iteration<0>(p, zz);
-        if (!aborted && zz + 1 <= G.NZ) aborted = w.template iteration<1>(p, zz + 1);
-        if (!aborted && zz + 2 <= G.NZ) aborted = w.template iteration<2>(p, zz + 2);
+        if (!aborted && zz + 1 <= w.zb) aborted = w.template iteration<1>(p, zz + 1);
+        if (!aborted && zz + 2 <= w.zb) aborted = w.template iteration<2>(p, zz + 2);
     }
     if (aborted && w.lead) w.drain();
 }
 
 // Pack the AoS float3 state into the padded float4 layout (frame = periodic images or zeros),
 // and back.
+// (I: the index type, 32 bits wherever the padded state has fewer entries -- three 64-bit divisions an entry
+// otherwise took as long as the copy.)
+template <typename I>
 __global__ void pack_padded_kernel(const float *__restrict__ m, float4 *__restrict__ out, int NX, int NY, int NZ,
-                                   unsigned periodic, long long total)
+                                   unsigned periodic, I total)
 {
-    const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+    const I i = (I)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= total) return;
-    const int NXp = NX + 4, NYp = NY + 4;
+    const I NXp = NX + 4, NYp = NY + 4;
     const int xp = (int)(i % NXp);
-    const long long t = i / NXp;
+    const I t = i / NXp;
     const int yp = (int)(t % NYp);
-    const long long t2 = t / NYp;
-    const int z = (int)(t2 % NZ);
-    const long long r = t2 / NZ;
+    const I t2 = t / NYp;
+    const int z = (int)(t2 % (I)NZ);
+    const I r = t2 / (I)NZ;
     int x = xp - 2, y = yp - 2;
     bool in = true;
     if (x < 0 || x >= NX) {
@@ -468,18 +513,19 @@ __global__ void pack_padded_kernel(const float *__restrict__ m, float4 *__restri
     out[i] = v;
 }
 
-__global__ void unpack_padded_kernel(const float4 *__restrict__ in, float *__restrict__ m, int NX, int NY, int NZ,
-                                     long long total)
+template <typename I>
+__global__ void unpack_padded_kernel(const float4 *__restrict__ in, float *__restrict__ m, int NX, int NY, int NZ, I total)
 {
-    const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+    const I i = (I)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= total) return;
-    const long long ncell = (long long)NX * NY * NZ;
-    const long long r = i / ncell, c = i - r * ncell;
-    const int x = (int)(c % NX), y = (int)((c / NX) % NY), z = (int)(c / ((long long)NX * NY));
+    const I t = i / (I)NX, t2 = t / (I)NY;
+    const int x = (int)(i - t * (I)NX), y = (int)(t - t2 * (I)NY), z = (int)(t2 % (I)NZ);
+    const I r = t2 / (I)NZ;
     const float4 v = in[(size_t)r * (NX + 4) * (NY + 4) * NZ + ((size_t)z * (NY + 4) + (y + 2)) * (NX + 4) + (x + 2)];
-    m[3 * i] = v.x;
-    m[3 * i + 1] = v.y;
-    m[3 * i + 2] = v.z;
+    float *o = m + 3 * (size_t)i;
+    o[0] = v.x;
+    o[1] = v.y;
+    o[2] = v.z;
 }
 
 // Deterministic two-pass mean of m_z per realisation: pass 1 sums fixed contiguous chunks of the
@@ -572,12 +618,22 @@ template <int C, bool AX>
 cudaError_t launch_step(const KParams &p, const SlabGeom &G, const SlabPlan &plan, const CUtensorMap &map,
                         float4 *out, int n_real, unsigned long long n, int *status, cudaStream_t st)
 {
-    const dim3 grid(G.tiles_x, G.tiles_y, n_real);
+    const dim3 grid(G.tiles_x, G.tiles_y, n_real * G.parts);
     auto go = [&](auto kern) {
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)plan.smem_bytes);
         if (e != cudaSuccess) return e;
-        kern<<<grid, plan.threads, plan.smem_bytes, st>>>(p, G, map, out, n, status);
-        return cudaGetLastError();
+        // a step may be launched while the one before it drains (griddepcontrol in the kernel)
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = grid;
+        cfg.blockDim = dim3(plan.threads);
+        cfg.dynamicSmemBytes = plan.smem_bytes;
+        cfg.stream = st;
+        cudaLaunchAttribute at[1];
+        at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        at[0].val.programmaticStreamSerializationAllowed = 1;
+        cfg.attrs = at;
+        cfg.numAttrs = 1;
+        return cudaLaunchKernelEx(&cfg, kern, p, G, map, out, n, status);
     };
     if constexpr (C == 4) {
         // the 512-wide slab in 64 x 27 tiles of 512 threads: every thread's four columns share x
@@ -592,7 +648,7 @@ cudaError_t launch_step(const KParams &p, const SlabGeom &G, const SlabPlan &pla
 
 }  // namespace
 
-bool slab_plan(const KParams &p, int dev, SlabPlan *plan)
+bool slab_plan(const KParams &p, int n_real, int dev, SlabPlan *plan)
 {
     if (p.periodic & 4u) return false;  // free z faces only
     // a periodic axis needs at least four cells, so that each cell has at most one image per axis
@@ -604,38 +660,58 @@ bool slab_plan(const KParams &p, int dev, SlabPlan *plan)
         cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
         return false;
     const int tiles_x = (p.nx + 63) / 64;
-    int tiles_y = std::max(1, std::min(p.ny, nsm / tiles_x));
     const int TXmax = (p.nx + tiles_x - 1) / tiles_x;
-    int TYmax = (p.ny + tiles_y - 1) / tiles_y;
     // three state slots, three predictor slots, the thermal-field store of every column slot of the
     // CTA, three mbarriers
-    auto smem_of = [&](int ty) {
-        const int cols = TXmax * ty;
-        const int thr = std::min(kSlabThreads, std::max(32, (std::max(cols, 2 * TXmax + 2 * ty) + 31) / 32 * 32));
-        const int cpt = (cols + kSlabThreads - 1) / kSlabThreads;
-        return (size_t)3 * (slot_of(TXmax + 4, ty + 4) + slot_of(TXmax + 4, ty + 2)) * sizeof(float4) +
-               (size_t)cpt * thr * sizeof(float4) + 3 * sizeof(uint64_t);
+    auto threads_of = [&](int ty) {
+        return std::min(kSlabThreads, std::max(32, (std::max(TXmax * ty, 2 * TXmax + 2 * ty) + 31) / 32 * 32));
     };
-    while (TYmax > 1 && (TXmax * TYmax > 4 * kSlabThreads || smem_of(TYmax) > (size_t)smem_optin ||
-                         TYmax + 4 > 256)) {
-        ++tiles_y;
-        TYmax = (p.ny + tiles_y - 1) / tiles_y;
-    }
-    if (TXmax * TYmax > 4 * kSlabThreads || smem_of(TYmax) > (size_t)smem_optin || TXmax + 4 > 256 || TYmax + 4 > 256)
-        return false;
-    const int cols = TXmax * TYmax;
-    const int cpt = (cols + kSlabThreads - 1) / kSlabThreads;
-    const int ring = 2 * TXmax + 2 * TYmax;
-    const int threads = std::min(kSlabThreads, std::max(32, (std::max(cols, ring) + 31) / 32 * 32));
-    if (ring > threads) return false;
-    plan->tiles_x = tiles_x;
-    plan->tiles_y = tiles_y;
-    plan->TXmax = TXmax;
-    plan->TYmax = TYmax;
-    plan->cols_per_thread = cpt;
-    plan->threads = threads;
-    plan->smem_bytes = smem_of(TYmax);
-    return true;
+    auto smem_of = [&](int ty) {
+        const int cpt = (TXmax * ty + kSlabThreads - 1) / kSlabThreads;
+        return (size_t)3 * (slot_of(TXmax + 4, ty + 4) + slot_of(TXmax + 4, ty + 2)) * sizeof(float4) +
+               (size_t)cpt * threads_of(ty) * sizeof(float4) + 3 * sizeof(uint64_t);
+    };
+    auto holds = [&](int ty) {
+        return TXmax * ty <= 4 * kSlabThreads && smem_of(ty) <= (size_t)smem_optin && TXmax + 4 <= 256 && ty + 4 <= 256 &&
+               2 * TXmax + 2 * ty <= threads_of(ty);
+    };
+    // The tiles and the parts of z, by the step time that fits the measured ones within a fifth: 1 us of launch,
+    // and for every plane that a CTA sweeps (its part, two more predictor planes where z is cut, one more for
+    // the corrector's lag) 0.63 us of latency -- copy, predictor, corrector, barrier -- and 0.05 us for every 32
+    // columns (the ring's predictor counts 0.6).  A film of few columns leaves SMs idle or its CTAs with few
+    // warps, so cutting z pays: 131x72x39 cells 40.9 -> 13.5 us a step (3x6 tiles, 8 parts), 64x64x20
+    // 24.7 -> 8.5, 30x450x50 51.3 -> 18.1 (of which 2.5 to 4.5 us come from the overlapped launch);
+    // 512x512x56 (8x19 tiles) stays whole (208.9 in two parts where it took 198.7).
+    double best = 0.0;
+    bool found = false;
+    auto consider = [&](int tiles_y, int parts) {
+        tiles_y = std::max(1, std::min(p.ny, tiles_y));
+        int ty = (p.ny + tiles_y - 1) / tiles_y;
+        while (ty > 1 && !holds(ty)) {
+            ++tiles_y;
+            ty = (p.ny + tiles_y - 1) / tiles_y;
+        }
+        if (!holds(ty) || (parts > 1 && (long long)n_real * parts > 65535)) return;  // the grid's z extent
+        const double ctas = (double)tiles_x * tiles_y * parts * n_real;
+        const int planes = (p.nz + parts - 1) / parts + 1 + (parts > 1 ? 2 : 0);
+        const double warps = (TXmax * ty + 0.6 * (2 * TXmax + 2 * ty)) / 32.0;
+        const double us = 1.0 + std::ceil(ctas / nsm) * planes * (0.63 + 0.05 * warps);
+        if (found && us > 0.95 * best) return;
+        best = us;
+        found = true;
+        plan->tiles_x = tiles_x;
+        plan->tiles_y = tiles_y;
+        plan->parts = parts;
+        plan->TXmax = TXmax;
+        plan->TYmax = ty;
+        plan->cols_per_thread = (TXmax * ty + kSlabThreads - 1) / kSlabThreads;
+        plan->threads = threads_of(ty);
+        plan->smem_bytes = smem_of(ty);
+    };
+    consider(nsm / tiles_x, 1);
+    for (int parts = 1; parts <= 8 && 3 * parts <= std::max(3, p.nz); ++parts)
+        for (int per_sm : {1, 2}) consider((int)(per_sm * (long long)nsm / ((long long)tiles_x * parts * n_real)), parts);
+    return found;
 }
 
 size_t slab_state_float4s(const KParams &p, int n_real)
@@ -655,6 +731,7 @@ cudaError_t slab_advance(const KParams &p, const SlabPlan &plan, float *m, int n
     G.NYp = p.ny + 4;
     G.tiles_x = plan.tiles_x;
     G.tiles_y = plan.tiles_y;
+    G.parts = plan.parts;
     G.TXmax = plan.TXmax;
     G.TYmax = plan.TYmax;
     G.pitch = plan.TXmax + 4;
@@ -667,17 +744,24 @@ cudaError_t slab_advance(const KParams &p, const SlabPlan &plan, float *m, int n
         return cudaErrorInvalidValue;
     const long long padded = (long long)slab_state_float4s(p, n_real);
     const long long total = (long long)p.ncells * n_real;
-    pack_padded_kernel<<<(unsigned)((padded + 255) / 256), 256, 0, st>>>(m, buf_a, p.nx, p.ny, p.nz, p.periodic,
-                                                                         padded);
-    // the output buffer's frame: its periodic images are rewritten every step, and a free face's
-    // zeros must be there from the start
-    pack_padded_kernel<<<(unsigned)((padded + 255) / 256), 256, 0, st>>>(m, buf_b, p.nx, p.ny, p.nz, p.periodic,
-                                                                         padded);
+    const bool narrow = padded < (1LL << 31) && total < (1LL << 31);
+    auto pack = [&](float4 *out) {
+        const unsigned blocks = (unsigned)((padded + 255) / 256);
+        if (narrow)
+            pack_padded_kernel<unsigned><<<blocks, 256, 0, st>>>(m, out, p.nx, p.ny, p.nz, p.periodic, (unsigned)padded);
+        else
+            pack_padded_kernel<long long><<<blocks, 256, 0, st>>>(m, out, p.nx, p.ny, p.nz, p.periodic, padded);
+    };
+    pack(buf_a);
+    // the output buffer's frame: its periodic images are rewritten every step, but a free face's zeros must
+    // be there from the start
+    const bool framed = (p.periodic & 3u) == 3u;
+    if (!framed) pack(buf_b);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     float4 *a = buf_a, *b = buf_b;
     const CUtensorMap *ma = &map_a, *mb = &map_b;
-    long long count = 2;
+    long long count = framed ? 1 : 2;
     for (long long s = 0; s < n_steps; ++s) {
         const unsigned long long n = (unsigned long long)(step0 + s);
         switch (plan.cols_per_thread) {
@@ -713,7 +797,11 @@ cudaError_t slab_advance(const KParams &p, const SlabPlan &plan, float *m, int n
             count += 2;
         }
     }
-    unpack_padded_kernel<<<(unsigned)((total + 255) / 256), 256, 0, st>>>(a, m, p.nx, p.ny, p.nz, total);
+    const unsigned blocks = (unsigned)((total + 255) / 256);
+    if (narrow)
+        unpack_padded_kernel<unsigned><<<blocks, 256, 0, st>>>(a, m, p.nx, p.ny, p.nz, (unsigned)total);
+    else
+        unpack_padded_kernel<long long><<<blocks, 256, 0, st>>>(a, m, p.nx, p.ny, p.nz, total);
     ++count;
     if (launches) *launches += count;
     return cudaGetLastError();

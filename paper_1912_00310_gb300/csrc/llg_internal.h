@@ -168,10 +168,10 @@ cudaError_t rod_advance(const KParams &p, const RodPlan &plan, float *m, int n_r
 
 // ---- streaming engine (k_slab.cu): one fused Heun step per launch over HBM ----------------
 struct SlabPlan {
-    int tiles_x, tiles_y, TXmax, TYmax, cols_per_thread, threads;
+    int tiles_x, tiles_y, parts, TXmax, TYmax, cols_per_thread, threads;
     size_t smem_bytes;
 };
-bool slab_plan(const KParams &p, int dev, SlabPlan *plan);
+bool slab_plan(const KParams &p, int n_real, int dev, SlabPlan *plan);
 // buf_a, buf_b: slab_state_float4s(p, n_real) float4 each (the padded layout
 // [n_real][nz][ny + 4][nx + 4]); partial: slab_partial_floats(n_real) floats.
 // status bit 2 (value 4): a staging wait of the streaming kernel gave up.

@@ -97,3 +97,34 @@ def test_full_slab_launch_shape(pkg):
     assert float(got[..., 2].min()) < 0.999  # the noise acted
     g.close()
     gp.close()
+
+
+@pytest.mark.parametrize("dims,n_real,periodic,disp", [
+    ((40, 40, 20), 1, 0b011, 0.0),   # five parts of four planes
+    ((70, 33, 9), 3, 0b011, 0.3),    # three parts of three, several realisations
+    ((9, 5, 6), 1, 0b000, 0.3),      # two parts of three planes: each predictor plane but one is made twice
+    ((20, 14, 7), 2, 0b010, 0.0),    # uneven parts of three and four
+    ((12, 70, 26), 1, 0b001, 0.3),   # seven uneven parts
+    ((66, 40, 24), 2, 0b011, 0.0),   # six parts, two tiles in x
+    ((5, 4, 3), 1, 0b011, 0.0),      # too few planes to cut
+    ((64, 2, 24), 1, 0b000, 0.3),    # eight parts
+    ((1, 9, 30), 1, 0b000, 0.0),
+])
+def test_films_cut_along_z_equal_plain_engine(pkg, dims, n_real, periodic, disp):
+    """Films of few columns: the automatic plan cuts z into parts.  An even and an odd number of
+    steps in several calls (the next step's launch overlaps the tail of the one before), samples
+    between them; states are the plain engine's bit for bit, samples within the reduction's rounding."""
+    out = []
+    for engine in (pkg.ENGINE_STREAM, pkg.ENGINE_PLAIN):
+        g = make(pkg, dims, periodic, engine, rate=1e5)  # 0.2 Oe a step: a sample every 5 steps
+        g.set_axis_dispersion(disp)
+        assert g.engine == engine
+        g.reset(seed=4, n_real=n_real, real_offset=1)
+        S = torch.zeros((n_real, g.n_samples), device="cuda")
+        for k in (1, 64, 37):
+            g.advance(k, S)
+        out.append((state(g, n_real), S[:, 1:102 // g.sample_every + 1].clone()))
+        g.close()
+    assert out[0][1].shape[1] >= 20
+    assert torch.equal(out[0][0], out[1][0])
+    assert torch.allclose(out[0][1], out[1][1], rtol=0, atol=1e-6)
