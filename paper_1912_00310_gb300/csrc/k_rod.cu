@@ -280,10 +280,11 @@ bool rod_plan(const KParams &p, int n_real, int dev, RodPlan *plan, int force_ki
         int rods = force_rods;
         if (rods == 0) {
             // one rod per CTA (608 b = 4 rods 0.87 us a step; 0.90, 0.98 and 1.23 with 2, 4 and 6),
-            // unless that leaves over a quarter of the last warp idle (the b = 8 rod's 21 cells): then
-            // the fewest rods that leave at most a tenth of it (4096 rods 0.82 us with 3, 1.13 with 1)
+            // unless that leaves over a quarter of the last warp idle (the b = 8 rod's 21 cells) and there
+            // are more rods than eight to an SM: then the fewest rods that leave at most a tenth of it
+            // (4096 rods 0.82 us with 3, 1.13 with 1; 1024 rods 0.43 and 0.42, 256 rods 0.365 and 0.359)
             rods = 1;
-            if (4 * (round_warp(rows) - rows) > round_warp(rows))
+            if (4 * (round_warp(rows) - rows) > round_warp(rows) && n_real > 8 * nsm)
                 for (int r = 2; r * rows <= maxt && r <= by_smem; ++r)
                     if (10 * (round_warp(r * rows) - r * rows) <= round_warp(r * rows)) {
                         rods = r;
