@@ -22,21 +22,23 @@
 // before the next plane's corrector reads and frees a state slot before it is refilled.  The
 // corrector writes the new state straight to the output buffer, and the cells within two of a
 // periodic face also to their images in the frame, so the next step's copies see a complete
-// frame.  The z loop is unrolled by three (the three state planes rotate), so the register
-// rotation and the slot offsets are compile-time; for the slab's 64 x 27 tiles the plane pitch is
-// compile-time too.
+// frame.  The three slots rotate in registers and the planes with nothing missing (no free face, no
+// end of a part) run an instance of the plane without those questions: unrolling the loop by three
+// instead, for compile-time slots, made it 50 KB long (458x338x45 cells 123 us a step, now 109).
 //
 // The arithmetic, the neighbour order (x-, x+, y-, y+, z-, z+) and the noise keys are those of
 // every other engine, so the trajectory is bitwise that of the plain engine on the same grid.
 //
-// What bounds it: 512x512x56 takes 192 us a step on a GB300 (205 before: the noise's first rounds,
+// What bounds it: 512x512x56 takes 187 us a step on a GB300 (205 before: the noise's first rounds,
 // which depend on the step only, are made once per launch; shorter noise and torque arithmetic; the
-// next launch's set-up runs under the tail of this one).  The state alone is 470 MB there and back,
-// 70 us at the copy rate; the rest is instructions: 260 a warp-cell with the ring's second predictor,
-// issued at 0.58 a cycle by the 16 warps that 128 registers leave an SM, which wait on fixed
-// latencies (1.4 cycles an instruction) and on the barrier of every plane (0.9).  A thread on pairs
-// of columns with packed arithmetic has fewer instructions, but holds both columns' planes in
-// registers: 266 us.
+// next launch's set-up runs under the tail of this one; the shorter loop).  The state alone is 470 MB
+// there and back, 70 us at the copy rate; the rest is instructions: 256 a warp-cell with the ring's
+// second predictor, issued at 0.58 a cycle by the 16 warps that 128 registers leave an SM, which wait
+// on fixed latencies (1.4 cycles an instruction) and on the barrier of every plane (0.9).  Tried: 20
+// warps with three columns a thread at 96 registers issue at 0.64 but need a tenth more instructions
+// (192 us before the shorter loop, 254 with it, from spills); noise drawn between arriving at the
+// barrier and waiting for it 187; pairs of columns with packed arithmetic 266 (spills).  With
+// dispersed axes 285 us (304): their loads' latency is exposed, so each plane asks L2 for the next.
 #include <cuda.h>  // CUtensorMap and its enums; the encoder is fetched from the driver at run time
 
 #include <algorithm>
@@ -50,6 +52,11 @@ namespace llg {
 namespace {
 
 constexpr int kSlabThreads = 512;
+// With one column a thread: the ring's cells then have warps of their own, so that no warp makes two
+// predictors in a row (201x139x17 cells, two films: 24.0 -> 22.8 us a step; 64x64x20 8.5 -> 8.0).
+constexpr int kSlabThreads1 = 576;
+constexpr int kFixedThreads = 512, kFixedRows = kFixedThreads / 64;  // tiles of 64 columns in x, four a thread
+constexpr int kFixedPitch = 64 + 4, kFixedBoxRows = 27 + 4;
 constexpr unsigned long long kStageWaitNs = 2000000000ull;  // longest wait for a staged plane
 
 __device__ __forceinline__ float3 zero3s() { return make_float3(0.f, 0.f, 0.f); }
@@ -121,14 +128,14 @@ struct SlabGeom {
 
 __host__ __device__ constexpr int slot_of(int pitch, int rows) { return (pitch * rows + 7) / 8 * 8; }
 
-// Per-CTA state of the z sweep.  PITCH, ROWS > 0: the box geometry at compile time.  NXC > 0:
-// the slab's x extent at compile time, with tiles of exactly PITCH - 4 = 64 columns and blockDim.x
-// a multiple of 64 -- then the columns of a thread share their x and lie blockDim.x / 64 rows
-// apart, so their positions are compile-time strides from the first column's (kept in
-// registers for one column only).
-template <int CPT, int PITCH, int ROWS, bool AX, int NXC = 0>
+// Per-CTA state of the z sweep.  PITCH, ROWS > 0: the slots' geometry at compile time.  FIXED: tiles of
+// exactly PITCH - 4 = 64 columns in x and kFixedThreads threads -- then the columns of a thread share
+// their x and lie kFixedRows rows apart, so their positions are strides from the first column's (kept in
+// registers for one column only).  Every film of a multiple of 64 cells in x whose tiles are 25 to 27
+// rows high runs it (the box may have fewer rows than its slot).
+template <int CPT, int PITCH, int ROWS, bool AX, bool FIXED = false>
 struct SlabSweep {
-    static constexpr bool kFixed = NXC > 0;
+    static constexpr bool kFixed = FIXED;
     float4 *Mb, *Tb;     // [3][slot] state planes; [3][tslot] predictor planes (Tb one row early)
     uint64_t *bar;       // [3] one mbarrier per state slot
     int pitch_rt, slot_rt, NZ;
@@ -155,19 +162,20 @@ struct SlabSweep {
     unsigned ghost;      // bit k: column k lies within two cells of a periodic face
     __device__ __forceinline__ int q(int k) const
     {
-        if constexpr (kFixed) return q_[0] + k * (kSlabThreads / 64) * PITCH;  // rows between columns: 512 / 64
+        if constexpr (kFixed) return q_[0] + k * kFixedRows * PITCH;
         return q_[k];
     }
     __device__ __forceinline__ uint32_t cell(int k) const
     {
-        if constexpr (kFixed) return cell_[0] + (uint32_t)(k * (kSlabThreads / 64) * NXC);
+        if constexpr (kFixed) return cell_[0] + (uint32_t)(k * kFixedRows * NX);
         return cell_[k];
     }
     __device__ __forceinline__ int gofs(int k) const
     {
-        if constexpr (kFixed) return gofs_[0] + k * (kSlabThreads / 64) * (NXC + 4);
+        if constexpr (kFixed) return gofs_[0] + k * kFixedRows * NXp;
         return gofs_[k];
     }
+    __device__ __forceinline__ int nthreads() const { return FIXED ? kFixedThreads : (int)blockDim.x; }
     __device__ __forceinline__ bool act(int k) const { return (actm >> k) & 1u; }
     // ring cell of this thread (predictor only)
     int rpos;
@@ -203,6 +211,8 @@ struct SlabSweep {
     int tslot_rt;
 
     unsigned box_bytes;
+    int s0, sm1, sp1;  // slots of planes z, z-1, z+1 (and z-2)
+    unsigned par_next;  // parity of plane z+1's use of its slot
     int last_issued;  // lead thread: the last plane whose copy was issued
 
     __device__ __forceinline__ float3 noise(const KParams &p, uint32_t c) const
@@ -246,15 +256,12 @@ struct SlabSweep {
     // where they belong to the CTA's part (a first plane staged only for the predictor above it is just
     // remembered).  Ends in a CTA barrier; returns true (in every thread) when some thread's staging wait
     // gave up.
-    template <int U>
+    template <bool INNER>
     __device__ __forceinline__ bool iteration(const KParams &p, int z)
     {
-        constexpr int s0 = U % 3, sm1 = (U + 2) % 3, sp1 = (U + 1) % 3;  // slots of planes z, z-1, z+1 (and z-2 = sp1)
-        // plane z+1 is the ((t + 1) / 3)-th use of its slot
-        const unsigned par_next = (unsigned)(((z - l0 + 1) / 3) & 1);
         const int P = pitch();
-        const bool pred = z >= zs && z < ze, corr = z > za;
-        const bool has_next = z + 1 < l1;
+        const bool pred = INNER || (z >= zs && z < ze), corr = INNER || z > za;
+        const bool has_next = INNER || z + 1 < l1;
         int fail = 0;
         // plane z+1, issued an iteration ago
         if (has_next && !mbar_wait(bar + sp1, par_next)) {
@@ -273,7 +280,7 @@ struct SlabSweep {
             const int c = q(k);
             float3 tnew = zero3s(), h = zero3s(), anew = zero3s();
             const float3 mcorr = Sp[k];  // the state of plane z-1, which the corrector starts from
-            float4 *hs = Hs + k * blockDim.x + threadIdx.x;
+            float4 *hs = Hs + k * nthreads() + threadIdx.x;
             if (pred) {
                 const float3 mcur = xyz(Mz[c]);
                 const float3 mnext = has_next ? xyz(Mn[c]) : zero3s();
@@ -292,7 +299,7 @@ struct SlabSweep {
             }
             if (corr) {
                 const float3 tself = xyz(Tr[c]);
-                const float3 tprev = z >= 2 ? xyz(Tp[c]) : zero3s();
+                const float3 tprev = INNER || z >= 2 ? xyz(Tp[c]) : zero3s();
                 float3 nb = add3(xyz(Tr[c - 1]), xyz(Tr[c + 1]));
                 nb = add3(nb, xyz(Tr[c - P]));
                 nb = add3(nb, xyz(Tr[c + P]));
@@ -308,7 +315,12 @@ struct SlabSweep {
                 A[k] = anew;
             }
         }
-        if (z < zs) {
+        if (AX && z + 1 < ze) {  // the next plane's axes on their way to L2 (their loads' latency is exposed)
+#pragma unroll
+            for (int k = 0; k < CPT; ++k)
+                if (act(k)) asm volatile("prefetch.global.L2 [%0];" ::"l"(axr + cell(k) + zoff + plane_c));
+        }
+        if (!INNER && z < zs) {
 #pragma unroll
             for (int k = 0; k < CPT; ++k)
                 if (act(k)) Sp[k] = xyz(Mz[q(k)]);
@@ -336,8 +348,8 @@ struct SlabSweep {
     }
 };
 
-template <int CPT, int PITCH, int ROWS, bool AX, int NXC = 0>
-__global__ void __launch_bounds__(kSlabThreads, 1) slab_step_kernel(KParams p, SlabGeom G,
+template <int CPT, int PITCH, int ROWS, bool AX, bool FIXED = false>
+__global__ void __launch_bounds__(FIXED ? kFixedThreads : CPT == 1 ? kSlabThreads1 : kSlabThreads, 1) slab_step_kernel(KParams p, SlabGeom G,
                                                                     const __grid_constant__ CUtensorMap tin,
                                                                     float4 *__restrict__ mout, unsigned long long n,
                                                                     int *__restrict__ status)
@@ -348,7 +360,7 @@ __global__ void __launch_bounds__(kSlabThreads, 1) slab_step_kernel(KParams p, S
         if (threadIdx.x == 0) atomicOr(status, 4);
         return;
     }
-    SlabSweep<CPT, PITCH, ROWS, AX, NXC> w;
+    SlabSweep<CPT, PITCH, ROWS, AX, FIXED> w;
     w.pitch_rt = G.pitch;
     w.slot_rt = G.slot;
     w.tslot_rt = G.tslot;
@@ -400,7 +412,7 @@ __global__ void __launch_bounds__(kSlabThreads, 1) slab_step_kernel(KParams p, S
     w.actm = 0u;
 #pragma unroll
     for (int k = 0; k < CPT; ++k) {
-        const int c = threadIdx.x + k * blockDim.x;
+        const int c = threadIdx.x + k * w.nthreads();
         const bool a = c < TX * TY;
         const int cc = a ? c : (int)threadIdx.x;  // an idle slot keeps the first column's position
         const int lx = cc % TX, ly = cc / TX;
@@ -470,10 +482,19 @@ __global__ void __launch_bounds__(kSlabThreads, 1) slab_step_kernel(KParams p, S
     for (int k = 0; k < CPT; ++k) w.Sp[k] = w.A[k] = zero3s();  // plane -1 of a first part: the free z face
     w.rSp = zero3s();
     bool aborted = __syncthreads_or(fail) != 0;
-    for (int zz = w.l0; zz <= w.zb && !aborted; zz += 3) {
-        aborted = w.template iteration<0>(p, zz);
-        if (!aborted && zz + 1 <= w.zb) aborted = w.template iteration<1>(p, zz + 1);
-        if (!aborted && zz + 2 <= w.zb) aborted = w.template iteration<2>(p, zz + 2);
+    w.s0 = 0;
+    w.sp1 = 1;
+    w.sm1 = 2;
+    w.par_next = 0u;
+    // from a part's second corrector plane to its last predictor plane but one nothing is missing
+    const int inner0 = max(w.za + 1, 2), inner1 = min(w.ze, w.l1 - 1);
+    for (int z = w.l0; z <= w.zb && !aborted; ++z) {
+        aborted = z >= inner0 && z < inner1 ? w.template iteration<true>(p, z) : w.template iteration<false>(p, z);
+        const int s = w.s0;
+        w.s0 = w.sp1;
+        w.sp1 = w.sm1;
+        w.sm1 = s;
+        if (w.sp1 == 0) w.par_next ^= 1u;
     }
     if (aborted && w.lead) w.drain();
 }
@@ -611,9 +632,6 @@ bool encode_state_map(CUtensorMap *map, float4 *base, const SlabGeom &G, int n_r
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// Compile-time box of the 512 x 512 slab's 64 x 27 tiles.
-constexpr int kSpecPitch = 68, kSpecRows = 31, kSpecNX = 512;
-
 template <int C, bool AX>
 cudaError_t launch_step(const KParams &p, const SlabGeom &G, const SlabPlan &plan, const CUtensorMap &map,
                         float4 *out, int n_real, unsigned long long n, int *status, cudaStream_t st)
@@ -635,14 +653,11 @@ cudaError_t launch_step(const KParams &p, const SlabGeom &G, const SlabPlan &pla
         cfg.numAttrs = 1;
         return cudaLaunchKernelEx(&cfg, kern, p, G, map, out, n, status);
     };
-    if constexpr (C == 4) {
-        // the 512-wide slab in 64 x 27 tiles of 512 threads: every thread's four columns share x
-        if (G.pitch == kSpecPitch && G.rows == kSpecRows && G.NX == kSpecNX && G.NX % 64 == 0 &&
-            G.tiles_x * 64 == G.NX && plan.threads == kSlabThreads)
-            return go(slab_step_kernel<4, kSpecPitch, kSpecRows, AX, kSpecNX>);
-        if (G.pitch == kSpecPitch && G.rows == kSpecRows)
-            return go(slab_step_kernel<4, kSpecPitch, kSpecRows, AX>);
-    }
+    if constexpr (C == 4)
+        if (plan.fixed) return go(slab_step_kernel<4, kFixedPitch, kFixedBoxRows, AX, true>);
+    if constexpr (C == 4)
+        if (G.pitch == kFixedPitch && G.rows == kFixedBoxRows)
+            return go(slab_step_kernel<4, kFixedPitch, kFixedBoxRows, AX>);
     return go(slab_step_kernel<C, 0, 0, AX>);
 }
 
@@ -663,13 +678,18 @@ bool slab_plan(const KParams &p, int n_real, int dev, SlabPlan *plan)
     const int TXmax = (p.nx + tiles_x - 1) / tiles_x;
     // three state slots, three predictor slots, the thermal-field store of every column slot of the
     // CTA, three mbarriers
+    auto fixed = [&](int ty) { return p.nx % 64 == 0 && 64 * ty > 3 * kSlabThreads && ty + 4 <= kFixedBoxRows; };
     auto threads_of = [&](int ty) {
-        return std::min(kSlabThreads, std::max(32, (std::max(TXmax * ty, 2 * TXmax + 2 * ty) + 31) / 32 * 32));
+        if (fixed(ty)) return +kFixedThreads;
+        const int cols = (TXmax * ty + 31) / 32 * 32, ring = (2 * TXmax + 2 * ty + 31) / 32 * 32;
+        if (cols <= kSlabThreads && cols + ring <= kSlabThreads1) return cols + ring;
+        return std::min(+kSlabThreads, std::max(cols, ring));
     };
+    auto cpt_of = [&](int ty) { return fixed(ty) ? 4 : (TXmax * ty + kSlabThreads - 1) / kSlabThreads; };
     auto smem_of = [&](int ty) {
-        const int cpt = (TXmax * ty + kSlabThreads - 1) / kSlabThreads;
-        return (size_t)3 * (slot_of(TXmax + 4, ty + 4) + slot_of(TXmax + 4, ty + 2)) * sizeof(float4) +
-               (size_t)cpt * threads_of(ty) * sizeof(float4) + 3 * sizeof(uint64_t);
+        const int rows = fixed(ty) ? kFixedBoxRows : ty + 4;
+        return (size_t)3 * (slot_of(TXmax + 4, rows) + slot_of(TXmax + 4, rows - 2)) * sizeof(float4) +
+               (size_t)cpt_of(ty) * threads_of(ty) * sizeof(float4) + 3 * sizeof(uint64_t);
     };
     auto holds = [&](int ty) {
         return TXmax * ty <= 4 * kSlabThreads && smem_of(ty) <= (size_t)smem_optin && TXmax + 4 <= 256 && ty + 4 <= 256 &&
@@ -704,7 +724,8 @@ bool slab_plan(const KParams &p, int n_real, int dev, SlabPlan *plan)
         plan->parts = parts;
         plan->TXmax = TXmax;
         plan->TYmax = ty;
-        plan->cols_per_thread = (TXmax * ty + kSlabThreads - 1) / kSlabThreads;
+        plan->fixed = fixed(ty);
+        plan->cols_per_thread = cpt_of(ty);
         plan->threads = threads_of(ty);
         plan->smem_bytes = smem_of(ty);
     };
@@ -736,8 +757,8 @@ cudaError_t slab_advance(const KParams &p, const SlabPlan &plan, float *m, int n
     G.TYmax = plan.TYmax;
     G.pitch = plan.TXmax + 4;
     G.rows = plan.TYmax + 4;
-    G.slot = slot_of(G.pitch, G.rows);
-    G.tslot = slot_of(G.pitch, G.rows - 2);
+    G.slot = slot_of(G.pitch, plan.fixed ? kFixedBoxRows : G.rows);
+    G.tslot = slot_of(G.pitch, (plan.fixed ? kFixedBoxRows : G.rows) - 2);
     G.box_bytes = (unsigned)(G.pitch * G.rows * sizeof(float4));
     CUtensorMap map_a, map_b;
     if (!encode_state_map(&map_a, buf_a, G, n_real) || !encode_state_map(&map_b, buf_b, G, n_real))

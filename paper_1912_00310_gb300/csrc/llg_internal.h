@@ -169,6 +169,7 @@ cudaError_t rod_advance(const KParams &p, const RodPlan &plan, float *m, int n_r
 // ---- streaming engine (k_slab.cu): one fused Heun step per launch over HBM ----------------
 struct SlabPlan {
     int tiles_x, tiles_y, parts, TXmax, TYmax, cols_per_thread, threads;
+    bool fixed;  // tiles of 64 columns in x, the instance with their geometry at compile time
     size_t smem_bytes;
 };
 bool slab_plan(const KParams &p, int n_real, int dev, SlabPlan *plan);

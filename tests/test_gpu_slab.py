@@ -109,6 +109,8 @@ def test_full_slab_launch_shape(pkg):
     ((5, 4, 3), 1, 0b011, 0.0),      # too few planes to cut
     ((64, 2, 24), 1, 0b000, 0.3),    # eight parts
     ((1, 9, 30), 1, 0b000, 0.0),
+    ((64, 320, 3), 12, 0b011, 0.3),  # 64 x 27 tiles: the instance with their geometry at compile time
+    ((128, 160, 2), 12, 0b001, 0.0),  # the same, the last rows of its slots unused
 ])
 def test_films_cut_along_z_equal_plain_engine(pkg, dims, n_real, periodic, disp):
     """Films of few columns: the automatic plan cuts z into parts.  An even and an odd number of
