@@ -262,10 +262,10 @@ bool rod_plan(const KParams &p, int n_real, int dev, RodPlan *plan, int force_ki
         const bool pair_each = twophase_fits && twophase_shape(p, 1, &one) && one.pairs_per_thread == 1;
         kind = rows_supported(p) ? 3 : (pair_each ? 1 : (pipelined_fits ? 2 : 1));
         // few rods: several SMs to each, where that is faster than what a step of one rod on one SM takes
-        // (us, measured: b = 2, 4, 8 rods 1.63, 0.47, 0.38; two-phase rods of 75, 441 and 660 pairs 0.63,
+        // (us, measured: b = 2, 4, 8 rods 1.63, 0.44, 0.25; two-phase rods of 75, 441 and 660 pairs 0.63,
         // 1.54 and 2.15; the b = 1 rod 11.2; 6x16x30 cells on the runtime-size pipelined kernel 5.4)
         if (alone && force_rods == 0 && force_rows == 0 && force_cpt == 0 && n_real < nsm) {
-            const double us = kind == 3   ? 0.35 + 0.00095 * p.ncells
+            const double us = kind == 3   ? 0.29 + 0.001 * p.ncells
                               : kind == 1 ? 0.42 + 0.0013 * p.ncells
                               : pairs_supported(p) ? 0.3 + 0.00101 * p.ncells
                                                    : 0.00186 * p.ncells;
@@ -281,10 +281,10 @@ bool rod_plan(const KParams &p, int n_real, int dev, RodPlan *plan, int force_ki
         if (rods == 0) {
             // one rod per CTA (608 b = 4 rods 0.87 us a step; 0.90, 0.98 and 1.23 with 2, 4 and 6),
             // unless that leaves over a quarter of the last warp idle (the b = 8 rod's 21 cells) and there
-            // are more rods than eight to an SM: then the fewest rods that leave at most a tenth of it
-            // (4096 rods 0.82 us with 3, 1.13 with 1; 1024 rods 0.43 and 0.42, 256 rods 0.365 and 0.359)
+            // are more rods than ten to an SM: then the fewest rods that leave at most a tenth of it
+            // (4096 rods 0.71 us with 3, 0.88 with 1; 2432 0.47 and 0.52; 1216 0.37 and 0.33)
             rods = 1;
-            if (4 * (round_warp(rows) - rows) > round_warp(rows) && n_real > 8 * nsm)
+            if (4 * (round_warp(rows) - rows) > round_warp(rows) && n_real > 10 * nsm)
                 for (int r = 2; r * rows <= maxt && r <= by_smem; ++r)
                     if (10 * (round_warp(r * rows) - r * rows) <= round_warp(r * rows)) {
                         rods = r;

@@ -27,9 +27,11 @@ constexpr int kMaxThreads = 768;
 //
 // What bounds it: the heavy FMA pipe, 61 % busy with 608 b = 4 rods (the noise's 32-bit multiplies and
 // half of every packed operation), and the two barriers' chains between (three warps a scheduler).
-// 608 b = 4 rods 0.87 us a step (1.03 with one cell an instruction), 1216 1.61 (1.83), four alone 0.51
-// (0.71); 152 b = 2 rods 1.57 (1.77).  Drawing the next step's noise beside the corrector: 0.88, 0.54
-// and 1.73.
+// 608 b = 4 rods 0.83 us a step (1.03 with one cell an instruction), 1216 1.58 (1.83), four alone 0.44
+// (0.71); 152 b = 2 rods 1.63 (1.77), 256 3.22.  Threads without a row compute row 0's again and store
+// nothing: with branches around the work its parts cannot be interleaved (608 b = 4 rods 0.86, four
+// 0.47, 256 b = 2 rods 3.31).  Drawing the next step's noise beside the corrector: 608 b = 4 rods 0.82,
+// but 1216 1.61 and 256 b = 2 rods 3.50.
 // ------------------------------------------------------------------------------------------
 template <int NX, int NY, int NZ, int SHAPE, bool AX, int MAXT>
 __global__ void __launch_bounds__(MAXT) rod_rows_kernel(KParams p, float *__restrict__ m_glob, int n_real,
@@ -112,28 +114,23 @@ __global__ void __launch_bounds__(MAXT) rod_rows_kernel(KParams p, float *__rest
     for (int s = 0; s < n_steps; ++s, ++n) {
         const float Hn1 = field.next(p);
         Pair3 t[NXP], s0[NXP], h[NXP];
-        if (act) {
-            const PhiloxStep now = philox_step(keys, n);
-            const pair_t H0 = both(Hn);
+        const pair_t H0 = both(Hn), H1 = both(Hn1);
+        const PhiloxStep now = philox_step(keys, n);
 #pragma unroll
-            for (int X = 0; X < NXP; ++X) {
-                h[X] = thermal_field_p3(keys, now, row_m0 + (unsigned long long)kPhiloxM0 * (2 * X), p.sigma_bm);
-                const Pair3 nb = neighbour_sum(m, X, MA, MB);
-                s0[X] = llg_torque_p3(m[X], effective_field_p3<AX>(nb, m[X], h[X], cf, H0, u[X]), cf.alpha);
-                t[X] = normalised_p3(axpy_p3(cf.neg_dt_g1, s0[X], m[X]));
-                store(PA, PB, q + X * PL, t[X]);
-            }
+        for (int X = 0; X < NXP; ++X) {
+            h[X] = thermal_field_p3(keys, now, row_m0 + (unsigned long long)kPhiloxM0 * (2 * X), p.sigma_bm);
+            const Pair3 nb = neighbour_sum(m, X, MA, MB);
+            s0[X] = llg_torque_p3(m[X], effective_field_p3<AX>(nb, m[X], h[X], cf, H0, u[X]), cf.alpha);
+            t[X] = normalised_p3(axpy_p3(cf.neg_dt_g1, s0[X], m[X]));
+            if (act) store(PA, PB, q + X * PL, t[X]);
         }
         __syncthreads();
-        if (act) {
-            const pair_t H1 = both(Hn1);
 #pragma unroll
-            for (int X = 0; X < NXP; ++X) {
-                const Pair3 nb = neighbour_sum(t, X, PA, PB);
-                const Pair3 sv = llg_torque_add_p3(s0[X], t[X], effective_field_p3<AX>(nb, t[X], h[X], cf, H1, u[X]), cf.alpha);
-                m[X] = normalised_p3(axpy_p3(cf.neg_hdt_g1, sv, m[X]));
-                store(MA, MB, q + X * PL, m[X]);
-            }
+        for (int X = 0; X < NXP; ++X) {
+            const Pair3 nb = neighbour_sum(t, X, PA, PB);
+            const Pair3 sv = llg_torque_add_p3(s0[X], t[X], effective_field_p3<AX>(nb, t[X], h[X], cf, H1, u[X]), cf.alpha);
+            m[X] = normalised_p3(axpy_p3(cf.neg_hdt_g1, sv, m[X]));
+            if (act) store(MA, MB, q + X * PL, m[X]);
         }
         __syncthreads();
         Hn = Hn1;
@@ -179,7 +176,8 @@ __global__ void __launch_bounds__(MAXT) rod_rows_kernel(KParams p, float *__rest
 // The same for rods one cell wide (the b = 8 rod, 1x3x7 cells): a thread is a cell, there are no pairs
 // of neighbours to take, and several rods share a CTA's warps.  Two rods to a packed thread measured
 // slower (four alone 0.47 us a step against 0.37, 4096 0.84 against 0.85): half the warps hide less of
-// the chain.  Float4 cells in the row kernel's gapless order.
+// the chain.  Float4 cells in the row kernel's gapless order, and no branches around the work either:
+// 4096 rods 0.71 us a step (0.77 with them).
 template <int NY, int NZ, int SHAPE, bool AX, int MAXT>
 __global__ void __launch_bounds__(MAXT) rod_cells_kernel(KParams p, float *__restrict__ m_glob, int n_real,
                                                          int rods_per_cta, long long step0, int n_steps,
@@ -228,19 +226,14 @@ __global__ void __launch_bounds__(MAXT) rod_cells_kernel(KParams p, float *__res
     unsigned long long n = (unsigned long long)step0;
     for (int s = 0; s < n_steps; ++s, ++n) {
         const float Hn1 = field.next(p);
-        float3 t = m, s0 = m, h = m;
-        if (act) {
-            h = box_muller3(philox4x32_10(keys, philox_step(keys, n), cell_m0), p.sigma_bm);
-            s0 = llg_torque(m, effective_field_sel<AX>(neighbour_sum(M), m, h, p, Hn, u), p.alpha);
-            t = normalised(axpy(p.neg_dt_g1, s0, m));
-            P[q] = pad4(t);
-        }
+        const float3 h = box_muller3(philox4x32_10(keys, philox_step(keys, n), cell_m0), p.sigma_bm);
+        const float3 s0 = llg_torque(m, effective_field_sel<AX>(neighbour_sum(M), m, h, p, Hn, u), p.alpha);
+        const float3 t = normalised(axpy(p.neg_dt_g1, s0, m));
+        if (act) P[q] = pad4(t);
         __syncthreads();
-        if (act) {
-            const float3 sv = llg_torque_add(s0, t, effective_field_sel<AX>(neighbour_sum(P), t, h, p, Hn1, u), p.alpha);
-            m = normalised(axpy(p.neg_hdt_g1, sv, m));
-            M[q] = pad4(m);
-        }
+        const float3 sv = llg_torque_add(s0, t, effective_field_sel<AX>(neighbour_sum(P), t, h, p, Hn1, u), p.alpha);
+        m = normalised(axpy(p.neg_hdt_g1, sv, m));
+        if (act) M[q] = pad4(m);
         __syncthreads();
         Hn = Hn1;
         if (--to_sample == 0) {
@@ -255,6 +248,80 @@ __global__ void __launch_bounds__(MAXT) rod_cells_kernel(KParams p, float *__res
                         samples[(size_t)(rod0 + r) * p.n_samples + k] = mean;
                         if (!isfinite(mean)) atomicOr(status, 1);
                     }
+                }
+            }
+        }
+    }
+    if (act) {
+        g[0] = m.x;
+        g[1] = m.y;
+        g[2] = m.z;
+    }
+}
+
+// One such rod to a CTA of one warp, for ensembles that leave the SMs few warps: its barriers are the
+// warp's, and each step draws the next one's noise, whose chain is as long as a half-step's, beside the
+// corrector.  What bounds it is that chain: 1 to 608 rods 0.25 us a step (the kernel above 0.30 alone,
+// 0.37 before it was free of branches), 1216 0.33 (0.37), 2432 0.52 (0.47).
+template <int NY, int NZ, int SHAPE, bool AX>
+__global__ void __launch_bounds__(32) rod_warp_kernel(KParams p, float *__restrict__ m_glob, int n_real, int rods_per_cta,
+                                                      long long step0, int n_steps, float *__restrict__ samples,
+                                                      int *__restrict__ status)
+{
+    constexpr int NCELL = NY * NZ, ROD = NCELL + 2 * NY;
+    __shared__ float4 M[ROD], P[ROD];
+    const int rod = blockIdx.x, lane = threadIdx.x;
+    for (int i = lane; i < ROD; i += 32) M[i] = P[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+    __syncwarp();
+    const bool act = lane < NCELL;
+    const int c = act ? lane : 0, y = c % NY, q = NY + c;
+    const float wm = y > 0 ? 1.f : 0.f, wp = y < NY - 1 ? 1.f : 0.f;
+    float *g = m_glob + ((size_t)rod * NCELL + c) * 3;
+    float3 m = make_float3(g[0], g[1], g[2]), u = make_float3(0.f, 0.f, 1.f);
+    if (act) M[q] = pad4(m);
+    if constexpr (AX) u = xyz(__ldg(p.axis + (size_t)rod * NCELL + c));
+    const PhiloxKeys keys = philox_keys(p.seed, p.real0 + (uint32_t)rod);
+    const unsigned long long cell_m0 = (unsigned long long)kPhiloxM0 * (uint32_t)c;
+    __syncwarp();
+    FieldAhead<SHAPE> field;
+    field.init(step0);
+    float Hn = field.next(p);
+    const long long se = p.sample_every;
+    const bool sampling = samples && se > 0;
+    long long k_next = sampling ? step0 / se + 1 : 0;
+    int to_sample = sampling ? (int)(k_next * se - step0) : -1;
+    auto neighbour_sum = [&](const float4 *A) {
+        const float3 l = xyz(A[q - 1]);
+        float3 nb = make_float3(wm * l.x, wm * l.y, wm * l.z);
+        nb = axpy(wp, xyz(A[q + 1]), nb);
+        nb = add3(nb, xyz(A[q - NY]));
+        return add3(nb, xyz(A[q + NY]));
+    };
+    auto bits = [&](unsigned long long n) { return philox4x32_10(keys, philox_step(keys, n), cell_m0); };
+    unsigned long long n = (unsigned long long)step0;
+    float3 h = box_muller3(bits(n), p.sigma_bm);
+    for (int s = 0; s < n_steps; ++s) {
+        ++n;
+        const float Hn1 = field.next(p);
+        const float3 s0 = llg_torque(m, effective_field_sel<AX>(neighbour_sum(M), m, h, p, Hn, u), p.alpha);
+        const float3 t = normalised(axpy(p.neg_dt_g1, s0, m));
+        if (act) P[q] = pad4(t);
+        __syncwarp();
+        const float3 next = box_muller3(bits(n), p.sigma_bm);
+        const float3 sv = llg_torque_add(s0, t, effective_field_sel<AX>(neighbour_sum(P), t, h, p, Hn1, u), p.alpha);
+        m = normalised(axpy(p.neg_hdt_g1, sv, m));
+        if (act) M[q] = pad4(m);
+        __syncwarp();
+        h = next;
+        Hn = Hn1;
+        if (--to_sample == 0) {
+            to_sample = (int)se;
+            const long long k = k_next++;
+            if (k < p.n_samples) {
+                const float mean = warp_cell_mean(act ? m.z : 0.f, NCELL);
+                if (lane == 0) {
+                    samples[(size_t)rod * p.n_samples + k] = mean;
+                    if (!isfinite(mean)) atomicOr(status, 1);
                 }
             }
         }
@@ -281,6 +348,13 @@ template <int NY, int NZ, int MAXT>
 cudaError_t launch_cells(const KParams &p, const RodPlan &plan, float *m, int n_real, long long step0, int n_steps,
                          float *samples, int *status, cudaStream_t st)
 {
+    if (plan.rods_per_cta == 1) {
+        if (p.axis)
+            return p.shape == 1 ? launch(rod_warp_kernel<NY, NZ, 1, true>, p, plan, m, n_real, step0, n_steps, samples, status, st)
+                                : launch(rod_warp_kernel<NY, NZ, 0, true>, p, plan, m, n_real, step0, n_steps, samples, status, st);
+        return p.shape == 1 ? launch(rod_warp_kernel<NY, NZ, 1, false>, p, plan, m, n_real, step0, n_steps, samples, status, st)
+                            : launch(rod_warp_kernel<NY, NZ, 0, false>, p, plan, m, n_real, step0, n_steps, samples, status, st);
+    }
     if (p.axis)
         return p.shape == 1 ? launch(rod_cells_kernel<NY, NZ, 1, true, MAXT>, p, plan, m, n_real, step0, n_steps, samples,
                                      status, st)

@@ -112,3 +112,15 @@ def test_rods_cut_over_several_ctas_equal_plain_engine(pkg, dims, n_real, disp, 
         ref, ref_s = ensemble(pkg, dims, n_real, plain=True, **kw)
         m, s = ensemble(pkg, dims, n_real, **kw)
         assert torch.equal(m, ref) and torch.equal(s, ref_s)
+
+
+@pytest.mark.parametrize("n_real", [1, 7, 1600])
+@pytest.mark.parametrize("disp,shape", [(0.0, 0), (0.3, 1)])
+def test_small_rods_alone_and_several_to_a_cta_equal_plain_engine(pkg, n_real, disp, shape):
+    """The b = 8 rod: one warp each while there are few, three to a CTA (the last one partly filled)
+    beyond; samples after every step and past a turn of the sweep."""
+    per_step = 1e7 * 1e9 * 20e-15  # Oe: a loop of 30 steps
+    kw = dict(b=8, dt=20e-15, disp=disp, shape=shape, rate=1e7, sample_dH=per_step, steps=(1, 33, 14))
+    ref, ref_s = ensemble(pkg, (1, 3, 7), n_real, plain=True, **kw)
+    m, s = ensemble(pkg, (1, 3, 7), n_real, **kw)
+    assert torch.equal(m, ref) and torch.equal(s, ref_s)
