@@ -30,6 +30,13 @@
 // segment is recomputed and reversed in turn in one launch.  The parameter partial sums are FP32
 // within blocks of 64 steps (aligned to absolute step numbers) and FP64 across blocks and in the
 // per-CTA reduction.
+//
+// What bounds it: the chain of one reversed step (four neighbour sums, four torques' worth of cross
+// products, three barriers), with a warp or two a scheduler.  The chain's independent parts overlap
+// only within straight code, so no branch surrounds a cell's work, and the next reversed step's noise
+// is drawn beside the first of the reverse products.  Gradients of 64 b = 4 rods over 2000 steps 4.22
+// -> 3.80 ms, 60 b = 8 rods over 1500 steps 2.03 -> 1.80, 20 rods of 990 cells over 1000 steps 8.28 ->
+// 6.66.
 #include <cmath>
 
 #include "llg_internal.h"
@@ -64,8 +71,8 @@ struct AdjParams {
     long long n_total;    // ... and the window has n_total steps (the last segment is shorter)
 };
 
-// MAXT: the largest CTA the instance runs with (256 for rods up to 256 cells, which then get up to
-// 255 registers per thread, 1024 otherwise); SHAPE: the sweep shape with 32-bit bookkeeping (0
+// MAXT: the largest CTA the instance runs with (32 for rods of one warp, whose barriers are the warp's,
+// 256 for rods up to 256 cells, which then get up to 255 registers per thread, 1024 otherwise); SHAPE: the sweep shape with 32-bit bookkeeping (0
 // triangle, 1 cosine) or -1 for the 64-bit sweep of any period.
 template <bool AX, int MAXT, int SHAPE>
 __global__ void __launch_bounds__(MAXT) adjoint_segment_kernel(
@@ -78,10 +85,18 @@ __global__ void __launch_bounds__(MAXT) adjoint_segment_kernel(
     const int S = ncell + 1;  // cells and the zero slot
     float4 *M = sm4, *P = M + S, *GT = P + S, *GH = GT + S;
     const int rod = blockIdx.x;
-    const int c = threadIdx.x;
-    const bool act = c < ncell;
+    // A thread without a cell computes cell 0's values again and stores nothing: branches around the work
+    // would keep its parts (neighbour loads, noise, torques) from being interleaved.
+    const bool act = (int)threadIdx.x < ncell;
+    const int c = act ? threadIdx.x : 0;
+    auto sync = [] {
+        if constexpr (MAXT == 32)
+            __syncwarp();
+        else
+            __syncthreads();
+    };
     for (int i = threadIdx.x; i < 4 * S; i += blockDim.x) sm4[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-    const Nbr nb = neighbours(act ? c : 0, p.nx, p.ny, p.nz, ncell);
+    const Nbr nb = neighbours(c, p.nx, p.ny, p.nz, ncell);
     const int q = c;  // this cell's slot
     const uint32_t real = p.real0 + (uint32_t)rod;
     const PhiloxKeys keys = philox_keys(p.seed, real);  // the rod's round keys, formed once
@@ -98,10 +113,10 @@ __global__ void __launch_bounds__(MAXT) adjoint_segment_kernel(
         seg += (size_t)off * n_rods * state;
     }
     float3 m = zero3a();
-    if (act && (ap.phases & 1))
+    if (ap.phases & 1)
         m = make_float3(ckpt[rod_off + 3 * c], ckpt[rod_off + 3 * c + 1], ckpt[rod_off + 3 * c + 2]);
     float3 u = make_float3(0.f, 0.f, 1.f);  // easy axis (dispersed-axis mode, AX)
-    if (AX && act) u = xyz(__ldg(p.axis + (size_t)rod * ncell + c));
+    if (AX) u = xyz(__ldg(p.axis + (size_t)rod * ncell + c));
     auto field_of = [&](float3 nb, float3 mm, float3 hh, float Hz) {
         return effective_field_sel<AX>(nb, mm, hh, p, Hz, u);
     };
@@ -116,34 +131,29 @@ __global__ void __launch_bounds__(MAXT) adjoint_segment_kernel(
         field.inc();
         const float Hn1 = field.value();
         float *sj = seg + (size_t)j * n_rods * state + rod_off;
-        float3 s0 = zero3a(), h = zero3a();
         if (act) {
             sj[3 * c] = m.x;
             sj[3 * c + 1] = m.y;
             sj[3 * c + 2] = m.z;
             M[q] = pad4(m);
         }
-        __syncthreads();
-        if (act) {
-            h = thermal_field(keys, (uint32_t)c, n, p.sigma_bm);
-            const float3 H = field_of(grad::neighbour_sum(M, nb), m, h, Hn);
-            s0 = llg_torque(m, H, p.alpha);
-            P[q] = pad4(normalised(axpy(p.neg_dt_g1, s0, m)));
-        }
-        __syncthreads();
-        if (act) {
-            const float3 t = xyz(P[q]);
-            const float3 H = field_of(grad::neighbour_sum(P, nb), t, h, Hn1);
-            m = normalised(axpy(p.neg_hdt_g1, llg_torque_add(s0, t, H, p.alpha), m));
-        }
-        __syncthreads();
+        sync();
+        const float3 h = thermal_field(keys, (uint32_t)c, n, p.sigma_bm);
+        const float3 s0 = llg_torque(m, field_of(grad::neighbour_sum(M, nb), m, h, Hn), p.alpha);
+        const float3 t = normalised(axpy(p.neg_dt_g1, s0, m));
+        if (act) P[q] = pad4(t);
+        sync();
+        const float3 H = field_of(grad::neighbour_sum(P, nb), t, h, Hn1);
+        m = normalised(axpy(p.neg_hdt_g1, llg_torque_add(s0, t, H, p.alpha), m));
+        // no barrier here: M, written next, was last read before the barrier above, and P is written again
+        // only after the next one
         Hn = Hn1;
     }
 
     if (!(ap.phases & 2)) return;
     // ---- backward through the segment ----
-    float3 g = zero3a();  // dL/d(state after the step being reversed)
-    if (act) g = make_float3(lam[rod_off + 3 * c], lam[rod_off + 3 * c + 1], lam[rod_off + 3 * c + 2]);
+    // dL/d(state after the step being reversed)
+    float3 g = make_float3(lam[rod_off + 3 * c], lam[rod_off + 3 * c + 1], lam[rod_off + 3 * c + 2]);
     // parameter partial sums: FP32 within blocks of kAdjBlock steps (aligned to absolute step
     // numbers, so both reverse schedules form the same block sums), FP64 across blocks -- the
     // GPU's FP64 rate is a small fraction of its FP32 rate, and a per-step FP64 update made the
@@ -172,11 +182,12 @@ __global__ void __launch_bounds__(MAXT) adjoint_segment_kernel(
     // iteration (it is stored there with the last shared write of that iteration, after every
     // read of M), and the stored state of the next step to reverse is loaded one step ahead (a
     // stored window is larger than L2, so each load would otherwise wait on HBM).
-    float3 m_cur = zero3a(), m_ahead = zero3a();
-    if (act && seg_len > 0) {
+    float3 m_cur = zero3a(), m_ahead = zero3a(), h = zero3a();
+    if (seg_len > 0) {
         const float *sl = seg + (size_t)(seg_len - 1) * n_rods * state + rod_off;
         m_cur = make_float3(sl[3 * c], sl[3 * c + 1], sl[3 * c + 2]);
-        M[q] = pad4(m_cur);
+        if (act) M[q] = pad4(m_cur);
+        h = thermal_field(keys, (uint32_t)c, (unsigned long long)(seg_start + seg_len - 1), p.sigma_bm);
     }
     __syncthreads();
     for (int j = seg_len - 1; j >= 0; --j) {
@@ -196,89 +207,76 @@ __global__ void __launch_bounds__(MAXT) adjoint_segment_kernel(
         } else if (r_s > 0) {
             --r_s;
         }
-        float3 mi = zero3a(), h = zero3a(), H = zero3a(), c0 = zero3a(), s0 = zero3a(), t = zero3a();
-        float pn = 1.f;  // 1 / |p|
-        if (act) {
-            mi = m_cur;
-            if (j > 0) {
-                const float *sn = seg + (size_t)(j - 1) * n_rods * state + rod_off;
-                m_ahead = make_float3(sn[3 * c], sn[3 * c + 1], sn[3 * c + 2]);
-            }
+        const float3 mi = m_cur;
+        if (j > 0) {
+            const float *sn = seg + (size_t)(j - 1) * n_rods * state + rod_off;
+            m_ahead = make_float3(sn[3 * c], sn[3 * c + 1], sn[3 * c + 2]);
         }
-        float3 Nm = zero3a();
-        if (act) {
-            h = thermal_field(keys, (uint32_t)c, (unsigned long long)n, p.sigma_bm);
-            Nm = grad::neighbour_sum(M, nb);
-            H = field_of(Nm, mi, h, hn);
-            c0 = cross3(mi, H);
-            s0 = llg_torque(mi, H, alpha);
-            const float3 pv = axpy(p.neg_dt_g1, s0, mi);
-            pn = rsqrt_fast(dot3(pv, pv));  // 1 / |p|
-            t = normalised(pv);
-            P[q] = pad4(t);
+        const float3 Nm = grad::neighbour_sum(M, nb);
+        const float3 H = field_of(Nm, mi, h, hn);
+        const float3 c0 = cross3(mi, H);
+        const float3 s0 = llg_torque(mi, H, alpha);
+        const float3 pv = axpy(p.neg_dt_g1, s0, mi);
+        const float pn = rsqrt_fast(dot3(pv, pv));  // 1 / |p|
+        const float3 t = normalised(pv);
+        if (act) P[q] = pad4(t);
+        sync();
+        const float3 h_ahead = thermal_field(keys, (uint32_t)c, (unsigned long long)(n - 1), p.sigma_bm);
+        const float3 Nt = grad::neighbour_sum(P, nb);
+        const float3 Ht = field_of(Nt, t, h, hn1);
+        const float3 c1 = cross3(t, Ht);
+        const float3 s1 = llg_torque(t, Ht, alpha);
+        const float3 qv = axpy(p.neg_hdt_g1, add3(s0, s1), mi);
+        const float rq = rsqrt_fast(dot3(qv, qv));  // 1 / |q|: m' = rq q, the forward's normalisation
+        const float3 mp = scale3(rq, qv);
+        const float3 gq = scale3(rq, sub3(g, scale3(dot3(mp, g), mp)));
+        const float3 gs1 = scale3(-ha, gq);
+        f_a -= 0.5f * dot3(add3(s0, s1), gq);
+        const float3 gc1 = add3(gs1, scale3(alpha, cross3(gs1, t)));
+        float3 gmt = add3(scale3(alpha, cross3(c1, gs1)), cross3(Ht, gc1));
+        const float3 gHt = cross3(gc1, t);
+        f_alpha += dot3(cross3(t, c1), gs1);
+        if (act) GT[q] = pad4(gHt);
+        sync();
+        gmt = axpy(p.c_ex, grad::neighbour_sum(GT, nb), gmt);
+        if constexpr (AX) {
+            const float gu = dot3(gHt, u);
+            gmt = axpy(p.c_an * gu, u, gmt);
+            f_can += gu * dot3(t, u);
+        } else {
+            gmt.z = fmaf(p.c_an, gHt.z, gmt.z);
+            f_can += gHt.z * t.z;
         }
-        __syncthreads();
-        float3 gHt = zero3a(), Nt = zero3a(), c1 = zero3a(), gq = zero3a(), gmt = zero3a(), Ht = zero3a();
-        float3 s1 = zero3a();
+        f_cex += dot3(gHt, Nt);
+        f_sigma += dot3(gHt, h);  // d/dsigma = (1/sigma) g_H.h, divided on the host
+        const float3 gp = scale3(pn, sub3(gmt, scale3(dot3(t, gmt), t)));
+        float3 gm = add3(gq, gp);                                  // q = m - ..., p = m - a s0
+        const float3 gs0 = add3(scale3(-ha, gq), scale3(-a, gp));  // from q and from p
+        f_a -= dot3(s0, gp);
+        const float3 gc0 = add3(gs0, scale3(alpha, cross3(gs0, mi)));
+        gm = add3(gm, add3(scale3(alpha, cross3(c0, gs0)), cross3(H, gc0)));
+        const float3 gH = cross3(gc0, mi);
+        f_alpha += dot3(cross3(mi, c0), gs0);
         if (act) {
-            Nt = grad::neighbour_sum(P, nb);
-            Ht = field_of(Nt, t, h, hn1);
-            c1 = cross3(t, Ht);
-            s1 = llg_torque(t, Ht, alpha);
-            const float3 qv = axpy(p.neg_hdt_g1, add3(s0, s1), mi);
-            const float rq = rsqrt_fast(dot3(qv, qv));  // 1 / |q|: m' = rq q, the forward's normalisation
-            const float3 mp = scale3(rq, qv);
-            gq = scale3(rq, sub3(g, scale3(dot3(mp, g), mp)));
-            const float3 gs1 = scale3(-ha, gq);
-            f_a -= 0.5f * dot3(add3(s0, s1), gq);
-            const float3 gc1 = add3(gs1, scale3(alpha, cross3(gs1, t)));
-            gmt = add3(scale3(alpha, cross3(c1, gs1)), cross3(Ht, gc1));
-            gHt = cross3(gc1, t);
-            f_alpha += dot3(cross3(t, c1), gs1);
-            GT[q] = pad4(gHt);
-        }
-        __syncthreads();
-        float3 gH = zero3a(), gm = zero3a();
-        if (act) {
-            gmt = axpy(p.c_ex, grad::neighbour_sum(GT, nb), gmt);
-            if constexpr (AX) {
-                const float gu = dot3(gHt, u);
-                gmt = axpy(p.c_an * gu, u, gmt);
-                f_can += gu * dot3(t, u);
-            } else {
-                gmt.z = fmaf(p.c_an, gHt.z, gmt.z);
-                f_can += gHt.z * t.z;
-            }
-            f_cex += dot3(gHt, Nt);
-            f_sigma += dot3(gHt, h);  // d/dsigma = (1/sigma) g_H.h, divided on the host
-            const float3 gp = scale3(pn, sub3(gmt, scale3(dot3(t, gmt), t)));
-            gm = add3(gq, gp);                                     // q = m - ..., p = m - a s0
-            const float3 gs0 = add3(scale3(-ha, gq), scale3(-a, gp));  // from q and from p
-            f_a -= dot3(s0, gp);
-            const float3 gc0 = add3(gs0, scale3(alpha, cross3(gs0, mi)));
-            gm = add3(gm, add3(scale3(alpha, cross3(c0, gs0)), cross3(H, gc0)));
-            gH = cross3(gc0, mi);
-            f_alpha += dot3(cross3(mi, c0), gs0);
             GH[q] = pad4(gH);
             if (j > 0) M[q] = pad4(m_ahead);  // M was last read before the previous barrier
         }
-        __syncthreads();
-        if (act) {
-            gm = axpy(p.c_ex, grad::neighbour_sum(GH, nb), gm);
-            if constexpr (AX) {
-                const float gu = dot3(gH, u);
-                gm = axpy(p.c_an * gu, u, gm);
-                f_can += gu * dot3(mi, u);
-            } else {
-                gm.z = fmaf(p.c_an, gH.z, gm.z);
-                f_can += gH.z * mi.z;
-            }
-            f_cex += dot3(gH, Nm);
-            f_sigma += dot3(gH, h);
-            g = gm;
-            m_cur = m_ahead;
-            if (n % kAdjBlock == 0) flush();
+        sync();
+        gm = axpy(p.c_ex, grad::neighbour_sum(GH, nb), gm);
+        if constexpr (AX) {
+            const float gu = dot3(gH, u);
+            gm = axpy(p.c_an * gu, u, gm);
+            f_can += gu * dot3(mi, u);
+        } else {
+            gm.z = fmaf(p.c_an, gH.z, gm.z);
+            f_can += gH.z * mi.z;
         }
+        f_cex += dot3(gH, Nm);
+        f_sigma += dot3(gH, h);
+        g = gm;
+        m_cur = m_ahead;
+        h = h_ahead;
+        if (n % kAdjBlock == 0) flush();
         // no barrier here: the next iteration's first shared write (P) follows reads of P that
         // ended before this iteration's second barrier, and GH is next written after two barriers
         // step back the field phase
@@ -292,7 +290,7 @@ __global__ void __launch_bounds__(MAXT) adjoint_segment_kernel(
     }
     // per-CTA partial sums of the parameter adjoints, fixed order
     __shared__ double red[5][32];
-    double v[5] = {g_alpha, g_a, g_cex, g_can, g_sigma};
+    double v[5] = {act ? g_alpha : 0.0, act ? g_a : 0.0, act ? g_cex : 0.0, act ? g_can : 0.0, act ? g_sigma : 0.0};
 #pragma unroll
     for (int k = 0; k < 5; ++k) {
         double x = v[k];
@@ -337,6 +335,7 @@ cudaError_t launch_adjoint(const AdjParams &ap, int n_real, int n_seg, const flo
     auto by_shape = [&](auto k0, auto k1, auto kg) { return shape == 0 ? go(k0) : shape == 1 ? go(k1) : go(kg); };
 #define LLG_ADJ(AXV, T) \
     adjoint_segment_kernel<AXV, T, 0>, adjoint_segment_kernel<AXV, T, 1>, adjoint_segment_kernel<AXV, T, -1>
+    if (threads <= 32) return p.axis ? by_shape(LLG_ADJ(true, 32)) : by_shape(LLG_ADJ(false, 32));
     if (threads <= 256) return p.axis ? by_shape(LLG_ADJ(true, 256)) : by_shape(LLG_ADJ(false, 256));
     return p.axis ? by_shape(LLG_ADJ(true, 1024)) : by_shape(LLG_ADJ(false, 1024));
 #undef LLG_ADJ

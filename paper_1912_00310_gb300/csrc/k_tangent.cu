@@ -25,6 +25,10 @@
 // the bank conflicts of a ghost-padded layout whose rows are only partly used.  Four such arrays:
 // m and dm/dtheta_j for the state and for the predictor (64 bytes a cell); rods of at most 1408
 // cells, the b = 2 rod included.
+//
+// What bounds it is the chain of a half-step, primal and tangent; the CTA has a warp or two a
+// scheduler.  60 b = 4 rods over 1500 steps 2.04 -> 1.82 ms and 60 b = 8 rods 1.06 -> 0.97 without
+// branches around a cell's work (and the warp's barriers for rods of one warp).
 #include <cmath>
 
 #include "llg_internal.h"
@@ -79,16 +83,26 @@ __global__ void __launch_bounds__(MAXT, MAXT <= 256 ? 1 : 0) tangent_kernel(TanP
     const PhiloxKeys keys = philox_keys(p.seed, real);  // the rod's round keys, formed once
     // this CTA's coefficient derivatives (a uniform index into the parameter block)
     const float dcex = d.dcex[j], dcan = d.dcan[j], dalpha = d.dalpha[j], da = d.da[j], rsig = d.rsig[j];
+    // With one cell a thread, a thread without one computes cell 0's values again and stores nothing: branches
+    // around the work would keep its parts (neighbour loads, noise, torques) from being interleaved.  With two
+    // the instance has no registers for that (100 b = 2 rods 10.4 us a step with the branches, 11.1 without).
+    auto act = [&](int k) { return (int)(threadIdx.x + k * blockDim.x) < ncell; };
+    auto cell = [&](int k) { return act(k) ? (int)(threadIdx.x + k * blockDim.x) : 0; };
+    auto sync = [] {
+        if constexpr (MAXT == 32)
+            __syncwarp();
+        else
+            __syncthreads();
+    };
     Nbr nb[CPT];
     float3 m[CPT], dm[CPT], u[CPT], hpre[CPT];  // the tangent starts at zero: m0 is fixed
 #pragma unroll
     for (int k = 0; k < CPT; ++k) {
-        const int c = threadIdx.x + k * blockDim.x;
-        nb[k] = neighbours(0, p.nx, p.ny, p.nz, ncell);
+        const int c = cell(k);
+        nb[k] = neighbours(c, p.nx, p.ny, p.nz, ncell);
         m[k] = dm[k] = hpre[k] = zr3();
         u[k] = make_float3(0.f, 0.f, 1.f);
-        if (c < ncell) {
-            nb[k] = neighbours(c, p.nx, p.ny, p.nz, ncell);
+        if (CPT == 1 || act(k)) {
             const float *src = m_glob + ((size_t)rod * ncell + c) * 3;
             m[k] = make_float3(src[0], src[1], src[2]);
             if (AX) u[k] = xyz(__ldg(p.axis + (size_t)rod * ncell + c));
@@ -99,7 +113,7 @@ __global__ void __launch_bounds__(MAXT, MAXT <= 256 ? 1 : 0) tangent_kernel(TanP
     __syncthreads();
 #pragma unroll
     for (int k = 0; k < CPT; ++k)
-        if (threadIdx.x + k * blockDim.x < ncell) M[threadIdx.x + k * blockDim.x] = pad4(m[k]);
+        if (act(k)) M[cell(k)] = pad4(m[k]);
     __syncthreads();
     const float alpha = p.alpha, a = -p.neg_dt_g1;
     const int lane = threadIdx.x & 31;
@@ -130,11 +144,13 @@ __global__ void __launch_bounds__(MAXT, MAXT <= 256 ? 1 : 0) tangent_kernel(TanP
         field.inc();
         const float Hn1 = field.value();
         float3 s0[CPT], dacc[CPT], t[CPT], dtt[CPT];
+        if constexpr (CPT > 1)
+#pragma unroll
+            for (int k = 0; k < CPT; ++k) s0[k] = dacc[k] = t[k] = dtt[k] = zr3();
 #pragma unroll
         for (int k = 0; k < CPT; ++k) {
-            s0[k] = dacc[k] = t[k] = dtt[k] = zr3();
-            const int c = threadIdx.x + k * blockDim.x;
-            if (c >= ncell) continue;
+            const int c = CPT > 1 ? (int)(threadIdx.x + k * blockDim.x) : cell(k);
+            if (CPT > 1 && c >= ncell) continue;
             const float3 N = grad::neighbour_sum(M, nb[k]), Nd = grad::neighbour_sum(Md, nb[k]);
             const float3 H = effective_field_sel<AX>(N, m[k], hpre[k], p, Hn, u[k]);
             s0[k] = llg_torque(m[k], H, alpha);
@@ -145,14 +161,16 @@ __global__ void __launch_bounds__(MAXT, MAXT <= 256 ? 1 : 0) tangent_kernel(TanP
             const float3 dp = sb3(sb3(dm[k], sc3(da, s0[k])), sc3(a, ds0));
             dtt[k] = sc3(r, sb3(dp, sc3(dt3(t[k], dp), t[k])));
             dacc[k] = sb3(dm[k], sc3(0.5f * a, ds0));
-            Pd[c] = pad4(dtt[k]);
-            P[c] = pad4(t[k]);
+            if (CPT > 1 || act(k)) {
+                Pd[c] = pad4(dtt[k]);
+                P[c] = pad4(t[k]);
+            }
         }
-        __syncthreads();
+        sync();
 #pragma unroll
         for (int k = 0; k < CPT; ++k) {
-            const int c = threadIdx.x + k * blockDim.x;
-            if (c >= ncell) continue;
+            const int c = CPT > 1 ? (int)(threadIdx.x + k * blockDim.x) : cell(k);
+            if (CPT > 1 && c >= ncell) continue;
             const float3 N = grad::neighbour_sum(P, nb[k]), Nd = grad::neighbour_sum(Pd, nb[k]);
             const float3 H = effective_field_sel<AX>(N, t[k], hpre[k], p, Hn1, u[k]);
             const float3 s01 = llg_torque_add(s0[k], t[k], H, alpha);
@@ -162,11 +180,13 @@ __global__ void __launch_bounds__(MAXT, MAXT <= 256 ? 1 : 0) tangent_kernel(TanP
             m[k] = make_float3(qv.x * r, qv.y * r, qv.z * r);
             const float3 dq = sb3(sb3(dacc[k], sc3(0.5f * da, s01)), sc3(0.5f * a, ds1));
             dm[k] = sc3(r, sb3(dq, sc3(dt3(m[k], dq), m[k])));
-            Md[c] = pad4(dm[k]);
-            M[c] = pad4(m[k]);
+            if (CPT > 1 || act(k)) {
+                Md[c] = pad4(dm[k]);
+                M[c] = pad4(m[k]);
+            }
             hpre[k] = thermal_field(keys, (uint32_t)c, n + 1, p.sigma_bm);
         }
-        __syncthreads();
+        sync();
         Hn = Hn1;
         if (--to_sample == 0) {
             to_sample = (int)se;
@@ -237,6 +257,7 @@ cudaError_t tangent_forward(const KParams &p, const double dcoef[15], int n_real
         return shape == 0 ? go(k0, threads) : shape == 1 ? go(k1, threads) : go(kg, threads);
     };
 #define LLG_TAN(AXV, C, T) tangent_kernel<AXV, C, T, 0>, tangent_kernel<AXV, C, T, 1>, tangent_kernel<AXV, C, T, -1>
+    if (t1 <= 32) return p.axis ? by_shape(LLG_TAN(true, 1, 32), t1) : by_shape(LLG_TAN(false, 1, 32), t1);
     if (t1 <= 192) return p.axis ? by_shape(LLG_TAN(true, 1, 192), t1) : by_shape(LLG_TAN(false, 1, 192), t1);
     if (t1 <= 768) return p.axis ? by_shape(LLG_TAN(true, 1, 768), t1) : by_shape(LLG_TAN(false, 1, 768), t1);
     if (t2 <= 704) return p.axis ? by_shape(LLG_TAN(true, 2, 704), t2) : by_shape(LLG_TAN(false, 2, 704), t2);

@@ -279,3 +279,23 @@ def test_window_within_one_checkpoint_interval(pkg, n_steps, ckpt_every):
     assert L == Lr
     assert np.allclose(grad, gr, rtol=1e-7, atol=0)
     g.close()
+
+
+@pytest.mark.parametrize("dims", [(1, 1, 2), (1, 3, 7), (2, 4, 4), (3, 11, 1), (5, 7, 5), (4, 8, 8), (6, 7, 9)])
+@pytest.mark.parametrize("method", [0, 1])
+def test_gradient_of_rods_that_fill_their_warps_or_not(pkg, orc, dims, method):
+    """Rods of one warp (2, 21 and 32 cells), of a cell more (33), and of several warps with and without
+    threads to spare: the loss and gradient against the FP64 replica."""
+    n_real, step0, n_steps = 4, 300, 700
+    g = grid(pkg, dims)
+    g.set_tuning(pkg.TUNE_GRAD_METHOD, method)
+    g.reset(seed=0, n_real=n_real)
+    m0 = random_unit_state(n_real, g.ncells, seed=21, cone=0.6).astype(np.float32)
+    g.set_state(m0, step0)
+    target = target_for(g)
+    L, got = g.loss_grad(n_steps, target, objective=0, ckpt_every=256)
+    Lo, go, _ = oracle_grad(orc, dims, m0.astype(np.float64), (1.0, 1.0, 1.0), step0, n_steps, target)
+    g.close()
+    assert L == pytest.approx(Lo, rel=1e-3)
+    for k in range(3):
+        assert got[k] == pytest.approx(go[k], rel=1e-2, abs=1e-3 * np.abs(go).max()), (k, got, go)
