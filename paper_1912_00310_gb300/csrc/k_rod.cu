@@ -252,15 +252,22 @@ bool rod_plan(const KParams &p, int n_real, int dev, RodPlan *plan, int force_ki
     const bool twophase_fits = rod_bytes <= (size_t)smem_optin && p.ncells <= 4 * kMaxThreads;
     const bool pipelined_fits = pipe_bytes <= (size_t)smem_optin && rows <= 4 * 672;
     // Default (measured on GB300): the b = 2, 4, 8 rods of the paper's ladder use the row kernel (four
-    // b = 4 rods 0.47 us a step against 0.60 with the two-phase kernel, 608 0.86 against 0.96); other
-    // rods whose pairs fit one to a thread the two-phase kernel with one rod per CTA (152 rods of
-    // 5x11x23 cells 2.15 us against 3.09 with the plane-pipelined one, 7x9x13 1.57 against 3.42; with
-    // several rods to an SM the two are level); larger rods the plane-pipelined kernels.
+    // b = 4 rods 0.44 us a step against 0.60 with the two-phase kernel, 608 0.82 against 1.09); other
+    // rods whose pairs fit one to a thread, or two where the rod is not eight cells wide, the two-phase
+    // kernel with one rod per CTA (152 rods of 5x11x23 cells 2.11 us against 3.09 with the plane-pipelined
+    // one, 7x9x13 1.51 against 3.42, 9x16x20 4.28 against 6.49, 16x10x12 2.68 against 7.67; 456 rods of
+    // 7x12x20 7.99 against 9.06); larger rods the plane-pipelined kernels (12x12x21 7.25 against 8.80), and
+    // eight-wide rods of two pairs a thread their own (8x24x15 4.09 against 4.29, 456 rods of 8x16x20 9.55
+    // against 10.95).
     int kind = force_kind;
     if (kind == 0) {
         RodPlan one{};
-        const bool pair_each = twophase_fits && twophase_shape(p, 1, &one) && one.pairs_per_thread == 1;
-        kind = rows_supported(p) ? 3 : (pair_each ? 1 : (pipelined_fits ? 2 : 1));
+        // (a request for a launch shape is the kernel's that it was always made to)
+        const bool few_cells = twophase_fits && p.ncells <= kMaxThreads;
+        const bool few_pairs = twophase_fits && force_rods == 0 && force_rows == 0 && force_cpt == 0 &&
+                               p.sample_every < (1LL << 31) && twophase_shape(p, 1, &one) &&
+                               one.pairs_per_thread <= (pairs_supported(p) ? 1 : 2);
+        kind = rows_supported(p) ? 3 : (few_cells || few_pairs ? 1 : (pipelined_fits ? 2 : 1));
         // few rods: several SMs to each, where that is faster than what a step of one rod on one SM takes
         // (us, measured: b = 2, 4, 8 rods 1.63, 0.44, 0.25; two-phase rods of 75, 441 and 660 pairs 0.63,
         // 1.54 and 2.15; the b = 1 rod 11.2; 6x16x30 cells on the runtime-size pipelined kernel 5.4)

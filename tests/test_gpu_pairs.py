@@ -124,3 +124,14 @@ def test_small_rods_alone_and_several_to_a_cta_equal_plain_engine(pkg, n_real, d
     ref, ref_s = ensemble(pkg, (1, 3, 7), n_real, plain=True, **kw)
     m, s = ensemble(pkg, (1, 3, 7), n_real, **kw)
     assert torch.equal(m, ref) and torch.equal(s, ref_s)
+
+
+@pytest.mark.parametrize("dims", [(7, 12, 20), (9, 13, 26), (12, 12, 21), (8, 16, 20), (2, 31, 26)])
+@pytest.mark.parametrize("request_", [(), ("TUNE_RODS_PER_CTA", 3), ("TUNE_ROWS_PER_THREAD", 3), ("TUNE_CELLS_PER_THREAD", 4)])
+def test_automatic_plan_of_larger_rods_equals_plain_engine(pkg, dims, request_):
+    """Rods of one to four pairs a thread under the automatic plan (200 of them, so that none is cut over
+    several CTAs), also where the caller asks for a launch shape and leaves the kernel open."""
+    ref, ref_s = ensemble(pkg, dims, 200, disp=0.3, shape=1, steps=(23,), plain=True)
+    m, s = ensemble(pkg, dims, 200, disp=0.3, shape=1, steps=(23,),
+                    tune=((getattr(pkg, request_[0]), request_[1]),) if request_ else ())
+    assert torch.equal(m, ref) and torch.equal(s, ref_s)
