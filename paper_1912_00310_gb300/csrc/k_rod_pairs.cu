@@ -225,7 +225,6 @@ struct PairRod {
 #pragma unroll
             for (int X = 0; X < NXP; ++X) {
                 const int XC = X > 0 ? X - 1 : NXP - 1;  // the corrector's plane
-                const bool corr = X > 0 || s > 0;
                 ulonglong2 *const SWA = SA + (X & 1) * PL, *const SRA = SA + (XC & 1) * PL;
                 pair_t *const SWB = SB + (X & 1) * PL, *const SRB = SB + (XC & 1) * PL;
                 const pair_t Hp = both(Hs), Hc = both(X > 0 ? Hs1 : Hprev);
@@ -236,8 +235,7 @@ struct PairRod {
                     // ---- predictor at (s, X) ----
                     const Pair3 h = thermal_field_p3(keys, now, cell_m0(j, X), p.sigma_bm);
                     const Pair3 u = axes(axr, X, i - ny());
-                    Pair3 mo = zero_p3();  // the state at the corrector's plane
-                    if (corr) mo = load(MA, MB, XC * PL + i);
+                    const Pair3 mo = load(MA, MB, XC * PL + i);  // the state at the corrector's plane
                     const Pair3 m = load(MA, MB, X * PL + i);
                     const float3 ml = X > 0 ? hi3(mo) : make_float3(0.f, 0.f, 0.f);
                     const float3 mr = X + 1 < NXP ? lo3(load(MA, MB, (X + 1) * PL + i)) : make_float3(0.f, 0.f, 0.f);
@@ -245,18 +243,18 @@ struct PairRod {
                     const Pair3 sv = llg_torque_p3(m, effective_field_p3<AX>(nb, m, h, cf, Hp, u), cf.alpha);
                     const Pair3 t = normalised_p3(axpy_p3(cf.neg_dt_g1, sv, m));
                     store(SWA, SWB, i, t);
-                    // ---- corrector one plane behind: (s, X - 1), or (s - 1, NXP - 1) at X = 0 ----
-                    float3 tl = make_float3(0.f, 0.f, 0.f);
-                    if (corr) {
-                        const Pair3 uc = axes(axr, XC, i - ny());
-                        const Pair3 tc = load(SRA, SRB, i);
-                        const float3 tr = X > 0 ? lo3(t) : make_float3(0.f, 0.f, 0.f);
-                        nb = neighbour_sum(pair3(add3(tL[j], hi3(tc)), add3(lo3(tc), tr)), SRA, SRB, i, j);
-                        const Pair3 H = effective_field_p3<AX>(nb, tc, hth[j], cf, Hc, uc);
-                        const Pair3 sc = llg_torque_add_p3(s0c[j], tc, H, cf.alpha);
-                        store(MA, MB, XC * PL + i, normalised_p3(axpy_p3(cf.neg_hdt_g1, sc, mo)));
-                        if (X > 0) tl = hi3(tc);
-                    }
+                    // ---- corrector one plane behind: (s, X - 1), or (s - 1, NXP - 1) at X = 0 (the first
+                    // step's is computed and dropped: a branch would part it from the predictor, 11.27 us a
+                    // step for 152 b = 1 rods instead of 11.15) ----
+                    const Pair3 uc = axes(axr, XC, i - ny());
+                    const Pair3 tc = load(SRA, SRB, i);
+                    const float3 tr = X > 0 ? lo3(t) : make_float3(0.f, 0.f, 0.f);
+                    nb = neighbour_sum(pair3(add3(tL[j], hi3(tc)), add3(lo3(tc), tr)), SRA, SRB, i, j);
+                    const Pair3 H = effective_field_p3<AX>(nb, tc, hth[j], cf, Hc, uc);
+                    const Pair3 sc = llg_torque_add_p3(s0c[j], tc, H, cf.alpha);
+                    const Pair3 mn = normalised_p3(axpy_p3(cf.neg_hdt_g1, sc, mo));
+                    if (X > 0 || s > 0) store(MA, MB, XC * PL + i, mn);
+                    const float3 tl = X > 0 ? hi3(tc) : make_float3(0.f, 0.f, 0.f);
                     tL[j] = tl;
                     s0c[j] = sv;
                     hth[j] = h;
