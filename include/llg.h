@@ -167,7 +167,9 @@ llg_status llg_set_engine(llg_ctx *ctx, int engine);
 
 /* Launch-shape overrides of the resident engine (0 = automatic, the default):
  *   LLG_TUNE_ROD_KIND      1 two-phase kernel, 2 plane-pipelined kernel, 3 row kernel (the
- *                          b = 2, 4, 8 rods of the paper's ladder: a thread per x-row)
+ *                          b = 2, 4, 8 rods of the paper's ladder: a thread per x-row); an
+ *                          ensemble of fewer rods than SMs may be cut over several SMs a rod, which
+ *                          only the automatic choice does
  *   LLG_TUNE_RODS_PER_CTA  rods per CTA of the two-phase and row kernels
  *   LLG_TUNE_CHUNK_STEPS   Heun steps per launch (default 2^20; llg_autotune sets it so the
  *                          launch overhead stays near 1% of a launch)
@@ -185,9 +187,10 @@ llg_status llg_set_engine(llg_ctx *ctx, int engine);
  *                             differently where a segment boundary splits a 64-step block
  *                             (measured: bitwise equal with aligned segments; FP32 blocks differ
  *                             from a per-step FP64 accumulation by at most 2e-8 relative).
- *   LLG_TUNE_CELLS_PER_THREAD cells per thread of the two-phase kernel (0 automatic, 1, 2, 4;
- *                             the b = 4 and b = 8 rods get 768 / cells-per-thread threads per CTA
- *                             at most, other grids 768)
+ *   LLG_TUNE_CELLS_PER_THREAD cells per thread that a CTA of the two-phase kernel is sized by (0
+ *                             automatic, 1, 2, 4): which rods and rods per CTA a request may name
+ *                             (the b = 4 and b = 8 rods get 768 / cells-per-thread threads per CTA
+ *                             at most, other grids 768).  The kernel itself works on pairs of cells.
  *   LLG_TUNE_GRAD_METHOD      llg_loop_area_grad's method: 0 the reverse-mode adjoint (default),
  *                             1 forward-mode tangents (one pass carrying dm/d(s_K, s_alpha, s_Ms);
  *                             no checkpoints or stored window; the same loss and, to FP32

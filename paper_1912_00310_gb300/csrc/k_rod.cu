@@ -1,11 +1,14 @@
 // k_rod.cu -- the resident engine: whole rods live in shared memory for an entire launch of
 // thousands of Heun steps of Eq. 1, and only the sampled M(H) values reach HBM.
 //
-// Two kernels, chosen by rod size:
+// The kernels, chosen by rod size and ensemble (rod_plan):
 //
 //  rod_zpairs_kernel (rods whose state and predictor state both fit), in k_rod_zpairs.cu; for the
-//      b = 2, 4, 8 rods of the paper's ladder rod_rows_kernel and rod_cells_kernel, in k_rod_small.cu.
-//      One or several rods per CTA, two barriers a step.
+//      b = 2, 4, 8 rods of the paper's ladder rod_rows_kernel, rod_cells_kernel and rod_warp_kernel, in
+//      k_rod_small.cu.  One or several rods per CTA, two barriers a step.
+//
+//  rod_split_kernel (ensembles of fewer rods than SMs, where that is faster), in k_rod_split.cu: a rod
+//      cut along z over a cluster of CTAs.
 //
 //  rod_pipelined_kernel (the b = 1 rod, 8x24x56 = 10752 cells: M alone is 129 KB, M and a full
 //      predictor copy do not fit).  One rod per CTA.  Each thread owns rows along x (fixed y, z);
@@ -269,11 +272,11 @@ bool rod_plan(const KParams &p, int n_real, int dev, RodPlan *plan, int force_ki
                                one.pairs_per_thread <= (pairs_supported(p) ? 1 : 2);
         kind = rows_supported(p) ? 3 : (few_cells || few_pairs ? 1 : (pipelined_fits ? 2 : 1));
         // few rods: several SMs to each, where that is faster than what a step of one rod on one SM takes
-        // (us, measured: b = 2, 4, 8 rods 1.63, 0.44, 0.25; two-phase rods of 75, 441 and 660 pairs 0.63,
+        // (us, measured: b = 2, 4, 8 rods 1.63, 0.44, 0.25; two-phase rods of 58, 312, 819 and 1265 cells 0.36, 0.74,
         // 1.54 and 2.15; the b = 1 rod 11.2; 6x16x30 cells on the runtime-size pipelined kernel 5.4)
         if (alone && force_rods == 0 && force_rows == 0 && force_cpt == 0 && n_real < nsm) {
             const double us = kind == 3   ? 0.29 + 0.001 * p.ncells
-                              : kind == 1 ? 0.42 + 0.0013 * p.ncells
+                              : kind == 1 ? (p.ncells <= 400 ? 0.33 + 0.0014 * p.ncells : 0.42 + 0.0013 * p.ncells)
                               : pairs_supported(p) ? 0.3 + 0.00101 * p.ncells
                                                    : 0.00186 * p.ncells;
             if (split_plan(p, n_real, nsm, smem_optin, us, plan)) return true;
@@ -333,6 +336,12 @@ bool rod_plan(const KParams &p, int n_real, int dev, RodPlan *plan, int force_ki
         plan->rows_per_thread = 0;
         plan->smem_bytes = rods * twophase_rod_bytes(p);
         plan->ctas = (n_real + rods - 1) / rods;
+        // small rods a cell to a thread: the chain of a step is shorter by the packed instructions' latency
+        // and the second cell's noise.  Rods of 1x2x29 cells 0.36 us a step against 0.64 (one to an SM) and
+        // 1.28 against 1.35 (16), 3x4x13 0.52 and 3.59 against 0.65 and 3.91, 3x4x26 0.74 against 0.89 with one to an
+        // SM but 1.80 against 1.47 with three; 4x6x20 0.96 against 0.91
+        if (force_rods == 0 && force_cpt == 0 && (p.ncells <= 160 || (p.ncells <= 400 && n_real <= nsm)))
+            compact_shape(p, plan);
         return true;
     }
     if (!pipelined_fits) return false;

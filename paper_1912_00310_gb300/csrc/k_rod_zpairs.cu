@@ -28,6 +28,7 @@
 #include "pair.cuh"
 #include "physics.cuh"
 #include "reduce.cuh"
+#include "rod_compact.cuh"
 #include "sweep32.cuh"
 
 namespace llg {
@@ -267,6 +268,89 @@ __global__ void __launch_bounds__(32) rod_single_kernel(KParams p, float *__rest
     }
 }
 
+// Small rods, one to a CTA, a cell to a thread: float4 cells in cell order and one zero slot for every
+// neighbour beyond a free face.  No branch surrounds a cell's work, so its parts overlap, and with up to four
+// warps each step draws the next one's noise, whose chain is as long as a half-step's, beside the
+// corrector (1x2x29 cells 0.355 us a step, 0.374 without; with more warps the noise of one overlaps the chain of
+// another anyway, and 3x4x26 cells take 0.74, 0.78 with the noise ahead).  What bounds it is that chain:
+// 0.34 us a step for 2 to 32 cells (one warp, which synchronises itself only), 0.52 for 156, 0.74 for 312;
+// many rods to an SM are bound by issue (2432 of 156 cells 3.59).
+template <bool AX, int SHAPE, int MAXT>
+__global__ void __launch_bounds__(MAXT) rod_compact_kernel(KParams p, float *__restrict__ m_glob, long long step0, int n_steps,
+                                                           float *__restrict__ samples, int *__restrict__ status)
+{
+    constexpr bool kAhead = MAXT <= 128;
+    extern __shared__ __align__(16) float4 csm[];
+    const int ncell = p.ncells, S = ncell + 1;  // cells and the zero slot
+    float4 *M = csm, *P = csm + S;
+    const int rod = blockIdx.x, lane = threadIdx.x & 31;
+    auto sync = [] {
+        if constexpr (MAXT == 32)
+            __syncwarp();
+        else
+            __syncthreads();
+    };
+    // a thread without a cell computes cell 0's values again and stores nothing
+    const bool act = (int)threadIdx.x < ncell;
+    const int c = act ? threadIdx.x : 0;
+    const grad::Nbr nb = grad::neighbours(c, p.nx, p.ny, p.nz, ncell);
+    float *g = m_glob + ((size_t)rod * ncell + c) * 3;
+    float3 m = make_float3(g[0], g[1], g[2]), u = make_float3(0.f, 0.f, 1.f);
+    if (act) M[c] = pad4(m);
+    if (threadIdx.x == 0) M[ncell] = P[ncell] = make_float4(0.f, 0.f, 0.f, 0.f);
+    if constexpr (AX) u = xyz(__ldg(p.axis + (size_t)rod * ncell + c));
+    const PhiloxKeys keys = philox_keys(p.seed, p.real0 + (uint32_t)rod);
+    const unsigned long long cell_m0 = (unsigned long long)kPhiloxM0 * (uint32_t)c;
+    sync();
+    FieldAhead<SHAPE> field;
+    field.init(step0);
+    float Hn = field.next(p);
+    const long long se = p.sample_every;
+    const bool sampling = samples && se > 0;
+    long long k_next = sampling ? step0 / se + 1 : 0;
+    int to_sample = sampling ? (int)(k_next * se - step0) : -1;
+    auto draw = [&](unsigned long long n) { return box_muller3(philox4x32_10(keys, philox_step(keys, n), cell_m0), p.sigma_bm); };
+    unsigned long long n = (unsigned long long)step0;
+    float3 h = draw(n);
+    for (int s = 0; s < n_steps; ++s) {
+        if constexpr (!kAhead) h = draw(n);
+        ++n;
+        const float Hn1 = field.next(p);
+        const float3 s0 = llg_torque(m, effective_field_sel<AX>(grad::neighbour_sum(M, nb), m, h, p, Hn, u), p.alpha);
+        const float3 t = normalised(axpy(p.neg_dt_g1, s0, m));
+        if (act) P[c] = pad4(t);
+        sync();
+        float3 next;
+        if constexpr (kAhead) next = draw(n);
+        const float3 sv =
+            llg_torque_add(s0, t, effective_field_sel<AX>(grad::neighbour_sum(P, nb), t, h, p, Hn1, u), p.alpha);
+        m = normalised(axpy(p.neg_hdt_g1, sv, m));
+        if (act) M[c] = pad4(m);
+        if constexpr (kAhead) h = next;
+        sync();
+        Hn = Hn1;
+        if (--to_sample == 0) {
+            // M holds the state after step n until the barrier in the next step's middle
+            to_sample = (int)se;
+            const long long k = k_next++;
+            if (k < p.n_samples && threadIdx.x < 32) {
+                float part = 0.f;
+                for (int i = lane; i < ncell; i += 32) part += M[i].z;
+                const float mean = warp_cell_mean(part, ncell);
+                if (lane == 0) {
+                    samples[(size_t)rod * p.n_samples + k] = mean;
+                    if (!isfinite(mean)) atomicOr(status, 1);
+                }
+            }
+        }
+    }
+    if (act) {
+        g[0] = m.x;
+        g[1] = m.y;
+        g[2] = m.z;
+    }
+}
+
 ZDims pair_dims(const KParams &p)
 {
     if (p.nz > 1) return ZDims{p.nx, p.ny, p.nz};
@@ -318,6 +402,14 @@ size_t twophase_rod_bytes(const KParams &p)
     return 48 * (size_t)d.entries();
 }
 
+void compact_shape(const KParams &p, RodPlan *plan)
+{
+    if (p.ncells < 2 || !sweep_fits_32(p)) return;
+    plan->pairs_per_thread = 0;
+    plan->threads = round32(p.ncells);
+    plan->smem_bytes = 2 * (size_t)(p.ncells + 1) * sizeof(float4);
+}
+
 bool twophase_shape(const KParams &p, int rods, RodPlan *plan)
 {
     const ZDims d = pair_dims(p);
@@ -347,6 +439,19 @@ cudaError_t twophase_advance(const KParams &p, const RodPlan &plan, float *m, in
     }
     const bool one = plan.rods_per_cta == 1;
     const int P = plan.pairs_per_thread;
+    if (P == 0) {
+        auto go = [&](auto kern) {
+            kern<<<n_real, plan.threads, plan.smem_bytes, st>>>(p, m, step0, n_steps, samples, status);
+            return cudaGetLastError();
+        };
+#define LLG_C(T)                                                                                              \
+    (p.shape == 1 ? (p.axis ? go(rod_compact_kernel<true, 1, T>) : go(rod_compact_kernel<false, 1, T>))       \
+                  : (p.axis ? go(rod_compact_kernel<true, 0, T>) : go(rod_compact_kernel<false, 0, T>)))
+        if (plan.threads <= 32) return LLG_C(32);
+        if (plan.threads <= 128) return LLG_C(128);
+        return LLG_C(416);
+#undef LLG_C
+    }
 #define LLG_D(P, MAXT)                                                                                 \
     (one ? launch_by<P, MAXT, true>(p, plan, m, n_real, step0, n_steps, samples, status, st)           \
          : launch_by<P, MAXT, false>(p, plan, m, n_real, step0, n_steps, samples, status, st))

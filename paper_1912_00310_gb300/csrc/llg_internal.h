@@ -135,6 +135,8 @@ bool rod_plan(const KParams &p, int n_real, int dev, RodPlan *plan, int force_ki
 // the launch of n_steps (< 2^31) steps.
 size_t twophase_rod_bytes(const KParams &p);
 bool twophase_shape(const KParams &p, int rods, RodPlan *plan);
+// ... and for small rods a cell to a thread instead (pairs_per_thread 0).
+void compact_shape(const KParams &p, RodPlan *plan);
 // Split kernel (k_rod_split.cu, plan kind 4): whether and over how many CTAs the rods of an ensemble that
 // leaves SMs idle are cut (base_us: a step's time with one rod per SM), and the launch.
 bool split_plan(const KParams &p, int n_real, int nsm, int smem_optin, double base_us, RodPlan *plan);

@@ -135,3 +135,17 @@ def test_automatic_plan_of_larger_rods_equals_plain_engine(pkg, dims, request_):
     m, s = ensemble(pkg, dims, 200, disp=0.3, shape=1, steps=(23,),
                     tune=((getattr(pkg, request_[0]), request_[1]),) if request_ else ())
     assert torch.equal(m, ref) and torch.equal(s, ref_s)
+
+
+@pytest.mark.parametrize("dims,n_real", [((1, 1, 2), 3), ((1, 2, 16), 200), ((3, 11, 1), 3), ((4, 8, 4), 3), ((3, 43, 1), 3), ((2, 4, 20), 200), ((7, 23, 1), 3),
+                                         ((3, 4, 26), 152), ((3, 4, 26), 153), ((4, 10, 10), 40)])
+@pytest.mark.parametrize("disp,shape", [(0.0, 0), (0.3, 1)])
+def test_small_rods_a_cell_to_a_thread_equal_plain_engine(pkg, dims, n_real, disp, shape):
+    """Rods of one warp (2 and 32 cells), a cell more (33), of four warps and a cell more (128, 129), and up to the sizes and ensembles at which the
+    pair kernel takes over (160 and 161 cells; 312 cells with as many rods as SMs and one more; 400)."""
+    kw = dict(disp=disp, shape=shape, steps=(1, 50, 23), sample_dH=0.2, rate=1e5)
+    ref, ref_s = ensemble(pkg, dims, n_real, plain=True, **kw)
+    m, s = ensemble(pkg, dims, n_real, tune=((pkg.TUNE_ROD_KIND, 1),), **kw)
+    assert torch.equal(m, ref) and torch.equal(s, ref_s)
+    m, s = ensemble(pkg, dims, n_real, **kw)
+    assert torch.equal(m, ref) and torch.equal(s, ref_s)
