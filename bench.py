@@ -439,8 +439,8 @@ def side_measurements(args, torch, pkg, cfg, g, samples, S_per_step, flush):
     return out
 
 
-KERNEL_SOURCES = ("paper_1912_00310_gb300/csrc/k_rod.cu", "paper_1912_00310_gb300/csrc/physics.cuh",
-                  "paper_1912_00310_gb300/csrc/reduce.cuh")
+KERNEL_SOURCES = ("paper_1912_00310_gb300/csrc/k_rod_pairs.cu", "paper_1912_00310_gb300/csrc/pair.cuh",
+                  "paper_1912_00310_gb300/csrc/physics.cuh", "paper_1912_00310_gb300/csrc/reduce.cuh")
 
 
 def measured_traffic():
