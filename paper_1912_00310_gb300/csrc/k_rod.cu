@@ -309,6 +309,7 @@ bool rod_plan(const KParams &p, int n_real, int dev, RodPlan *plan, int force_ki
         plan->rows_per_thread = 1;
         plan->smem_bytes = rows_smem_bytes(p, rods);
         plan->ctas = (n_real + rods - 1) / rods;
+        plan->crowded = !alone || plan->ctas > nsm;
         return true;
     }
     if (kind == 1) {

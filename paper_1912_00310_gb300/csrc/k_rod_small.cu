@@ -28,13 +28,18 @@ constexpr int kMaxThreads = 768;
 // What bounds it: the heavy FMA pipe, 61 % busy with 608 b = 4 rods (the noise's 32-bit multiplies and
 // half of every packed operation), and the two barriers' chains between (three warps a scheduler).
 // 608 b = 4 rods 0.83 us a step (1.03 with one cell an instruction), 1216 1.58 (1.83), four alone 0.44
-// (0.71); 152 b = 2 rods 1.63 (1.77), 256 3.22.  Threads without a row compute row 0's again and store
+// (0.71); 152 b = 2 rods 1.55 (1.77), 256 2.98.  Threads without a row compute row 0's again and store
 // nothing: with branches around the work its parts cannot be interleaved (608 b = 4 rods 0.86, four
 // 0.47, 256 b = 2 rods 3.31).  Drawing the next step's noise beside the corrector: 608 b = 4 rods 0.82,
 // but 1216 1.61 and 256 b = 2 rods 3.50.
+// The b = 2 rod's instance has 126 registers, so that one CTA of 352 threads fits an SM; where there are more
+// rods than SMs, or other jobs beside them, an instance of 80 (CTAS = 2) runs two side by side: 256 rods
+// 3.08 -> 2.98 us a step, 512 6.16 -> 5.81, 1024 10.76 -> 10.01, with dispersed axes (spills) 3.33 -> 3.26 and
+// 6.65 -> 6.34 at 512; alone on its SM a rod takes 1.55 us with the first and 1.72 with the second.
 // ------------------------------------------------------------------------------------------
-template <int NX, int NY, int NZ, int SHAPE, bool AX, int MAXT>
-__global__ void __launch_bounds__(MAXT) rod_rows_kernel(KParams p, float *__restrict__ m_glob, int n_real,
+// CTAS: CTAs to an SM that the registers have to allow (0: as the compiler likes).
+template <int NX, int NY, int NZ, int SHAPE, bool AX, int MAXT, int CTAS>
+__global__ void __launch_bounds__(MAXT, CTAS) rod_rows_kernel(KParams p, float *__restrict__ m_glob, int n_real,
                                                         int rods_per_cta, long long step0, int n_steps,
                                                         float *__restrict__ samples, int *__restrict__ status)
 {
@@ -366,19 +371,15 @@ cudaError_t launch_cells(const KParams &p, const RodPlan &plan, float *m, int n_
                                  status, st);
 }
 
-template <int NX, int NY, int NZ, int MAXT>
+template <int NX, int NY, int NZ, int MAXT, int CTAS>
 cudaError_t launch_rows_shaped(const KParams &p, const RodPlan &plan, float *m, int n_real, long long step0,
                                int n_steps, float *samples, int *status, cudaStream_t st)
 {
-    if (p.axis)
-        return p.shape == 1 ? launch(rod_rows_kernel<NX, NY, NZ, 1, true, MAXT>, p, plan, m, n_real, step0, n_steps,
-                                     samples, status, st)
-                            : launch(rod_rows_kernel<NX, NY, NZ, 0, true, MAXT>, p, plan, m, n_real, step0, n_steps,
-                                     samples, status, st);
-    return p.shape == 1 ? launch(rod_rows_kernel<NX, NY, NZ, 1, false, MAXT>, p, plan, m, n_real, step0, n_steps,
-                                 samples, status, st)
-                        : launch(rod_rows_kernel<NX, NY, NZ, 0, false, MAXT>, p, plan, m, n_real, step0, n_steps,
-                                 samples, status, st);
+#define LLG_R(S, AXV) \
+    launch(rod_rows_kernel<NX, NY, NZ, S, AXV, MAXT, CTAS>, p, plan, m, n_real, step0, n_steps, samples, status, st)
+    if (p.axis) return p.shape == 1 ? LLG_R(1, true) : LLG_R(0, true);
+    return p.shape == 1 ? LLG_R(1, false) : LLG_R(0, false);
+#undef LLG_R
 }
 
 // the rows kernel's shapes: b = 2, 4, 8 rods (x-rows of 4, 2, 1 cells)
@@ -421,9 +422,11 @@ cudaError_t rows_advance(const KParams &p, const RodPlan &plan, float *m, int n_
 {
     switch (rows_shape(p)) {
         case 2:
-            return launch_rows_shaped<4, 12, 28, 384>(p, plan, m, n_real, step0, n_steps, samples, status, st);
+            if (plan.crowded)
+                return launch_rows_shaped<4, 12, 28, 384, 2>(p, plan, m, n_real, step0, n_steps, samples, status, st);
+            return launch_rows_shaped<4, 12, 28, 384, 0>(p, plan, m, n_real, step0, n_steps, samples, status, st);
         case 4:
-            return launch_rows_shaped<2, 6, 14, kMaxThreads>(p, plan, m, n_real, step0, n_steps, samples, status, st);
+            return launch_rows_shaped<2, 6, 14, kMaxThreads, 0>(p, plan, m, n_real, step0, n_steps, samples, status, st);
         case 8:
             return launch_cells<3, 7, kMaxThreads>(p, plan, m, n_real, step0, n_steps, samples, status, st);
         default:

@@ -116,6 +116,7 @@ struct RodPlan {
     int rows_per_thread;  // kind 2
     int cells_per_thread; // kind 1: as asked for (the launch takes pairs_per_thread from the sizes)
     int pairs_per_thread = 0;  // kinds 1 and 4
+    bool crowded = false;  // kind 3: several CTAs to an SM, of this launch or of others beside it
     int split = 0, physics_warps = 0;  // kind 4: CTAs per rod, a CTA's warps without the sampler
     size_t smem_bytes;
     int ctas;

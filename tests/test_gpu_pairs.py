@@ -149,3 +149,13 @@ def test_small_rods_a_cell_to_a_thread_equal_plain_engine(pkg, dims, n_real, dis
     assert torch.equal(m, ref) and torch.equal(s, ref_s)
     m, s = ensemble(pkg, dims, n_real, **kw)
     assert torch.equal(m, ref) and torch.equal(s, ref_s)
+
+
+@pytest.mark.parametrize("n_real", [150, 400])
+@pytest.mark.parametrize("disp,shape", [(0.0, 0), (0.3, 1)])
+def test_row_kernel_with_one_and_two_ctas_to_an_sm_equals_plain_engine(pkg, n_real, disp, shape):
+    """The b = 2 rod with at most one rod to an SM and with more."""
+    kw = dict(b=2, dt=5e-15, disp=disp, shape=shape, steps=(41,))
+    ref, ref_s = ensemble(pkg, (4, 12, 28), n_real, plain=True, **kw)
+    m, s = ensemble(pkg, (4, 12, 28), n_real, tune=((pkg.TUNE_ROD_KIND, 3),), **kw)
+    assert torch.equal(m, ref) and torch.equal(s, ref_s)
