@@ -6,8 +6,8 @@
 // behind them.  A packed multiply-add occupies the pipes as long as two scalar ones (measured 2.0
 // scheduler cycles a warp against 1.0) but issues once: one Heun step's fields and torques take 40
 // issue slots per warp and cell instead of 81, and 84 cycles instead of 93 when nothing else runs.
-// Negations are written on the unpacked halves, which the assembler folds into operand modifiers; an
-// exclusive-or on the packed word costs two logic instructions each (87 cycles).
+// Negations are written on the unpacked halves: with an exclusive-or on the packed word the same measured
+// 87 cycles.
 #pragma once
 
 #include "physics.cuh"
@@ -96,8 +96,8 @@ __device__ __forceinline__ Pair3 box_muller_p3(uint4 a, uint4 b, float sigma_bm)
     const pair_t step = both(kAngleStep), first = both(kAngleFirst);
     const pair_t a1 = fma2(pack2(bits24(a.y), bits24(b.y)), step, first);
     const pair_t a3 = fma2(pack2(bits24(a.w), bits24(b.w)), step, first);
-    // z as a multiply-add with zero: the Zeeman field is added to it next, and ptxas contracts a packed
-    // multiply and add (-fmad=false or not) in some kernels, which would round once instead of twice
+    // z as a multiply-add with zero: with a plain product, to which the Zeeman field is added next, one kernel's
+    // states differed from the scalar engines' in the last bit (a bitwise test found it), with this none do
     return Pair3{mul2(r0, pack2(cos_fast(lo2(a1)), cos_fast(hi2(a1)))), mul2(r0, pack2(sin_fast(lo2(a1)), sin_fast(hi2(a1)))),
                  fma2(r2, pack2(cos_fast(lo2(a3)), cos_fast(hi2(a3))), 0ull)};
 }

@@ -11,11 +11,12 @@
 // multiply-add that forms the new state: the sum of two small torques is rounded at their own size
 // and the state once.
 //
-// The special functions are the approximate instructions in their flush-to-zero form: rsqrtf,
-// __log2f and the like compile to the same instruction between a comparison and two scalings for
-// subnormal arguments, which cannot occur here (the norm of a near-unit vector, log2 of a uniform
-// of at least 2^-25, a Box-Muller radius).  On GB300 that and the shorter Box-Muller below took the
-// noise draw alone from 127 to 105 scheduler cycles per warp and cell.
+// The special functions are the approximate instructions of the PTX ISA in their flush-to-zero form
+// (rsqrt, sqrt, lg2, sin and cos .approx.ftz.f32).  By the ISA that form differs from the plain one
+// for subnormal arguments and results only, and those cannot occur here: the arguments are the squared
+// norm of a near-unit vector, a uniform of at least 2^-25 and a Box-Muller radius.  Measured on GB300
+// with them and the shorter Box-Muller below, the noise draw alone went from 127 to 105 scheduler
+// cycles per warp and cell.
 #pragma once
 
 #include <cuda_runtime.h>
