@@ -197,9 +197,11 @@ llg_status llg_set_engine(llg_ctx *ctx, int engine);
  *                             rounding, the same gradient)
  *   LLG_TUNE_HANDOFF_TIMEOUT_MS  longest wait (ms, default 30000, 1 .. 3600000) of a CTA of the
  *                             balanced schedule for the CTA that runs the first part of a rod it
- *                             finishes; on expiry the CTA skips its remaining segments, and the
- *                             next llg_sync returns ETIMEOUT (the ensemble is then incomplete:
- *                             reset or restore it)
+ *                             finishes, and of a CTA of a rod cut over several SMs for its
+ *                             neighbours (the time it takes itself from sample to sample does not
+ *                             count); on expiry the CTA skips its remaining work, and the next
+ *                             llg_sync returns ETIMEOUT (the ensemble is then incomplete: reset or
+ *                             restore it)
  *   LLG_TUNE_WITHHOLD_HANDOFF 1: failure-path test hook -- the balanced schedule's producers do
  *                             not signal their hand-offs, so every wait runs out (default 0)
  * The arithmetic, and so the trajectory, does not depend on these.  Errors: EINVAL (unknown

@@ -18,7 +18,8 @@
 // One more warp forms the samples from snapshots of m_z that the others leave behind, in the canonical order
 // (reduce.cuh): each lane's partial sum runs through the slabs from the first CTA to the last.
 //
-// Every wait is bounded (status bit 1).  Neighbour order, noise keys and arithmetic are every other
+// Every wait is bounded by the hand-off limit (status bit 1); the sampler's, which spans the steps between
+// two samples, from the last step that its CTA began.  Neighbour order, noise keys and arithmetic are every other
 // engine's: bitwise the same states.
 //
 // What bounds it: the chain of a step -- neighbour loads, field, torque, normalisation, store, the lines' way
@@ -38,8 +39,8 @@
 namespace llg {
 namespace {
 
-constexpr unsigned long long kSplitWaitNs = 2000000000ull;  // longest wait inside a launch
 constexpr int kBars = 2 + 8;
+constexpr size_t kTailBytes = kBars * sizeof(uint64_t) + 16;  // the barriers and the step counter after them
 constexpr int kMaxThreads = 384;                            // 168 registers
 
 __host__ __device__ inline int slab_start(int nz, int k, int r) { return (int)((long long)nz * r / k); }
@@ -58,7 +59,8 @@ __host__ __device__ inline int largest_slab(int nz, int k)
 template <int W, bool FULL, bool AX, int SHAPE>
 __global__ void __launch_bounds__(kMaxThreads, 1) rod_split_kernel(KParams p, int k, int wp, float *__restrict__ m_glob,
                                                                    long long step0, int n_steps,
-                                                                   float *__restrict__ samples, int *__restrict__ status)
+                                                                   float *__restrict__ samples, int *__restrict__ status,
+                                                                   unsigned long long limit_ns)
 {
     extern __shared__ __align__(16) unsigned char ssm[];
     const int rank = (int)(blockIdx.x % (unsigned)k), rod = (int)(blockIdx.x / (unsigned)k);
@@ -76,6 +78,7 @@ __global__ void __launch_bounds__(kMaxThreads, 1) rod_split_kernel(KParams p, in
     float *carry = reinterpret_cast<float *>(snap + 2 * N);    // [2][32] partial sums from the slab below
     uint64_t *half = reinterpret_cast<uint64_t *>(carry + 64);
     uint64_t *taken = half + 2, *freed = taken + 2, *chain = freed + 2, *ack = chain + 2;
+    volatile int *step_now = reinterpret_cast<volatile int *>(half + kBars);  // the step this CTA is at
     const int T = blockDim.x;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const bool below = rank > 0, above = rank < k - 1;
@@ -87,6 +90,7 @@ __global__ void __launch_bounds__(kMaxThreads, 1) rod_split_kernel(KParams p, in
         MB[i] = QB[i] = 0ull;
     }
     if (threadIdx.x == 0) {
+        *step_now = 0;
         for (int b = 0; b < 2; ++b) {
             mbar_init(half + b, wp);
             mbar_init(taken + b, wp);
@@ -118,7 +122,7 @@ __global__ void __launch_bounds__(kMaxThreads, 1) rod_split_kernel(KParams p, in
     bool dead = false;  // a wait gave up: no more waiting
     auto wait = [&](uint64_t *bar, unsigned parity) {
         if (dead) return;
-        if (!mbar_wait(bar, parity, kSplitWaitNs)) {
+        if (!mbar_wait(bar, parity, limit_ns)) {
             atomicOr(status, 2);
             dead = true;
         }
@@ -224,6 +228,7 @@ __global__ void __launch_bounds__(kMaxThreads, 1) rod_split_kernel(KParams p, in
         int to_sample = sampling ? (int)(k_first * se - step0) : -1;
         unsigned n_snap = 0;
         for (int s = 0; s < n_steps; ++s) {
+            if (threadIdx.x == 0) *step_now = s;
             const float Hn1 = field.next(p);
             const PhiloxStep next = philox_step(keys, (unsigned long long)(step0 + s + 1));
             const pair_t H0 = both(Hn), H1 = both(Hn1);
@@ -292,14 +297,34 @@ __global__ void __launch_bounds__(kMaxThreads, 1) rod_split_kernel(KParams p, in
             chain_up = in_rank(smem_u32(chain), rank + 1);
             carry_up = in_rank(smem_u32(carry + lane), rank + 1);
         }
+        // A wait of the sampler, the same in all its lanes.  The steps to the next sample may take longer
+        // than any wait's limit: the limit runs from the last change of the CTA's step.
+        auto sampler_wait = [&](uint64_t *bar, unsigned parity) {
+            if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+            int at = *step_now;
+            unsigned long long t0 = timer_ns();
+            while (!__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) {
+                const int now = *step_now;
+                const unsigned long long t = timer_ns();
+                if (now != at) {
+                    at = now;
+                    t0 = t;
+                }
+                if (__any_sync(0xffffffffu, t - t0 > limit_ns)) {
+                    if (lane == 0) atomicOr(status, 2);
+                    return false;
+                }
+            }
+            return true;
+        };
         const long long k_last = (step0 + n_steps) / se;
         unsigned n = 0;
         for (long long kk = k_first; kk <= k_last; ++kk, ++n) {
             const unsigned b = n & 1u, use = (n >> 1) & 1u;
-            wait(taken + b, use);
+            if (!sampler_wait(taken + b, use)) break;  // and no sample after a wait that gave up
             float part = 0.f;
             if (below) {
-                wait(chain + b, use);
+                if (!sampler_wait(chain + b, use)) break;
                 part = carry[b * 32 + lane];
                 __syncwarp();
                 if (lane == 0) mbar_arrive_cluster(ack_down + 8u * b);
@@ -312,7 +337,7 @@ __global__ void __launch_bounds__(kMaxThreads, 1) rod_split_kernel(KParams p, in
             __syncwarp();
             if (lane == 0) mbar_arrive(freed + b);
             if (above) {
-                wait(ack + b, use ^ 1u);  // the slab above has read the carry's last use
+                if (!sampler_wait(ack + b, use ^ 1u)) break;  // the slab above has read the carry's last use
                 st_cluster(carry_up + b * 128u, part);
                 __syncwarp();
                 if (lane == 0) mbar_arrive_cluster(chain_up + 8u * b);
@@ -348,7 +373,8 @@ cudaError_t launch(const KParams &p, const RodPlan &plan, float *m, int n_real, 
     at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
     cfg.attrs = at;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kern, p, plan.split, plan.physics_warps, m, step0, n_steps, samples, status);
+    return cudaLaunchKernelEx(&cfg, kern, p, plan.split, plan.physics_warps, m, step0, n_steps, samples, status,
+                              plan.handoff_timeout_ns);
 }
 
 template <int W, bool FULL>
@@ -380,7 +406,7 @@ static bool split_shape(const KParams &p, int k, int smem_optin, RodPlan *plan)
     }
     if (W == 0) return false;
     const size_t E = (size_t)px * (size_t)(cap + 2 * p.ny), N = (size_t)px * (size_t)cap;
-    const size_t smem = 48 * E + 16 * N + 64 * sizeof(float) + kBars * sizeof(uint64_t);
+    const size_t smem = 48 * E + 16 * N + 64 * sizeof(float) + kTailBytes;
     if (smem + 1024 > (size_t)smem_optin) return false;
     plan->kind = 4;
     plan->split = k;
