@@ -203,7 +203,8 @@ llg_status llg_set_engine(llg_ctx *ctx, int engine);
  *                             llg_sync returns ETIMEOUT (the ensemble is then incomplete: reset or
  *                             restore it)
  *   LLG_TUNE_WITHHOLD_HANDOFF 1: failure-path test hook -- the balanced schedule's producers do
- *                             not signal their hand-offs, so every wait runs out (default 0)
+ *                             not signal their hand-offs, and the CTAs of a cut rod send nothing
+ *                             to the CTA below, so every such wait runs out (default 0)
  * The arithmetic, and so the trajectory, does not depend on these.  Errors: EINVAL (unknown
  * key, negative value); EUNSUPPORTED at the next advance if the shape cannot hold the grid. */
 #define LLG_TUNE_ROD_KIND 1

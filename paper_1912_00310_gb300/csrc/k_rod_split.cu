@@ -19,7 +19,9 @@
 // (reduce.cuh): each lane's partial sum runs through the slabs from the first CTA to the last.
 //
 // Every wait is bounded by the hand-off limit (status bit 1); the sampler's, which spans the steps between
-// two samples, from the last step that its CTA began.  Neighbour order, noise keys and arithmetic are every other
+// two samples, from the last 32 steps that its CTA began.  Where one gives up, the rod's threads store and arrive no
+// more and leave their loops, no state and no further sample is written, and no CTA leaves before the lines
+// that have been sent to it have landed (abandon).  Neighbour order, noise keys and arithmetic are every other
 // engine's: bitwise the same states.
 //
 // What bounds it: the chain of a step -- neighbour loads, field, torque, normalisation, store, the lines' way
@@ -40,8 +42,17 @@ namespace llg {
 namespace {
 
 constexpr int kBars = 2 + 8;
-constexpr size_t kTailBytes = kBars * sizeof(uint64_t) + 16;  // the barriers and the step counter after them
-constexpr int kMaxThreads = 384;                            // 168 registers
+constexpr int kBlock = 32;  // steps between two looks for a thread that gave up (0.1 ms; a limit is 1 ms at least)
+
+// What follows the barriers in shared memory.
+struct Tail {
+    // after a give-up, by half-step of a step: bytes that the neighbours have sent here, arrivals of the CTA's warps
+    unsigned long long inbound[2], arrived[2];
+    int step_now;      // the block of steps that this CTA is at, by its first step
+    unsigned gave_up;  // a wait of some CTA of the cluster ran out
+};
+constexpr size_t kTailBytes = kBars * sizeof(uint64_t) + sizeof(Tail);
+constexpr int kMaxThreads = 384;  // 168 registers
 
 __host__ __device__ inline int slab_start(int nz, int k, int r) { return (int)((long long)nz * r / k); }
 
@@ -55,12 +66,80 @@ __host__ __device__ inline int largest_slab(int nz, int k)
     return most;
 }
 
+// (out of line, as abandon below: inline they cost the step loop up to 7 %)
+__device__ __noinline__ bool slow_wait(uint64_t *bar, unsigned parity, unsigned long long limit_ns)
+{
+    return mbar_wait(bar, parity, limit_ns);
+}
+
+// The sampler's wait for the phase of `parity`, the same in all its lanes.  The steps to the next sample may take
+// longer than any wait's limit: the limit runs from the beginning of the CTA's block of steps.
+__device__ __forceinline__ bool sampler_wait(uint64_t *bar, unsigned parity, const Tail *tail, unsigned long long limit_ns)
+{
+    if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+    const volatile Tail *now = tail;
+    int at = now->step_now;
+    unsigned long long t0 = timer_ns();
+    while (!__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) {
+        const unsigned long long t = timer_ns();
+        const int step = now->step_now;
+        if (step != at) {
+            at = step;
+            t0 = t;
+        }
+        if (__any_sync(0xffffffffu, t - t0 > limit_ns)) return false;
+    }
+    return true;
+}
+
+// After the last store of every CTA of the cluster (a cluster barrier lies between) and with inbound and
+// arrived complete: wait until the neighbours' lines that are still under way to this CTA have landed.  bar is
+// the barrier of one half-step of a step, warp0 the arrivals of warp 0 there, which announce `bytes` each.
+// A phase ends with wp arrivals and `bytes` landed; a warp arrives for the next one only after that, and so
+// do the neighbours' lines, so min(arrived / wp, inbound / bytes) phases end by themselves.  What has been
+// sent into the open one is made to end it: its count of bytes is set to what was sent and the missing
+// arrivals are made.
+__device__ void settle(uint64_t *bar, unsigned long long arrived, unsigned long long inbound, unsigned bytes,
+                       unsigned wp, unsigned long long warp0, unsigned long long limit_ns)
+{
+    const unsigned long long by_arrivals = arrived / wp, by_bytes = inbound / bytes;
+    const unsigned long long phases = by_arrivals < by_bytes ? by_arrivals : by_bytes;
+    if (phases > 0 && !mbar_wait(bar, (unsigned)(phases - 1) & 1u, limit_ns)) return;
+    const unsigned sent = (unsigned)(inbound - phases * bytes), there = (unsigned)(arrived - phases * wp);
+    if (sent == 0) return;
+    const unsigned announced = warp0 > phases ? bytes : 0u;
+    if (sent > announced) mbar_expect_bytes(bar, sent - announced);
+    if (sent < announced) mbar_complete_bytes(bar, announced - sent);
+    if (there < wp) mbar_arrive_many(bar, wp - there);
+    mbar_wait(bar, (unsigned)phases & 1u, limit_ns);
+}
+
+// The way out of a rod after a give-up, for the physics warps of all its CTAs, when none stores into a neighbour
+// any more: what has been sent lands before the CTA that it is sent to leaves.  stored: the half-steps whose values
+// this thread has stored, `pairs` pairs each, below (sides bit 0) and above (bit 1) the slab.
+__device__ __noinline__ void abandon(uint64_t *half, Tail *tail, unsigned stored, int pairs, int sides, int rank,
+                                     unsigned line_bytes, int wp, unsigned long long limit_ns)
+{
+    const unsigned sent[2] = {(stored + 1) / 2, stored / 2};
+    for (int b = 0; b < 2; ++b) {
+        const unsigned long long bytes = 24ull * (unsigned)pairs * sent[b];
+        if (sides & 1) add_cluster(in_rank(smem_u32(&tail->inbound[b]), rank - 1), bytes);
+        if (sides & 2) add_cluster(in_rank(smem_u32(&tail->inbound[b]), rank + 1), bytes);
+        if ((threadIdx.x & 31) == 0) atomicAdd(&tail->arrived[b], (unsigned long long)sent[b]);
+    }
+    __syncwarp();
+    cluster_sync();
+    if (threadIdx.x == 0)
+        for (int b = 0; b < 2; ++b)
+            settle(half + b, tail->arrived[b], tail->inbound[b], line_bytes, (unsigned)wp, sent[b], limit_ns);
+}
+
 // FULL: every segment has W pairs and every pair two cells.
 template <int W, bool FULL, bool AX, int SHAPE>
 __global__ void __launch_bounds__(kMaxThreads, 1) rod_split_kernel(KParams p, int k, int wp, float *__restrict__ m_glob,
                                                                    long long step0, int n_steps,
                                                                    float *__restrict__ samples, int *__restrict__ status,
-                                                                   unsigned long long limit_ns)
+                                                                   unsigned long long limit_ns, int withhold)
 {
     extern __shared__ __align__(16) unsigned char ssm[];
     const int rank = (int)(blockIdx.x % (unsigned)k), rod = (int)(blockIdx.x / (unsigned)k);
@@ -78,7 +157,7 @@ __global__ void __launch_bounds__(kMaxThreads, 1) rod_split_kernel(KParams p, in
     float *carry = reinterpret_cast<float *>(snap + 2 * N);    // [2][32] partial sums from the slab below
     uint64_t *half = reinterpret_cast<uint64_t *>(carry + 64);
     uint64_t *taken = half + 2, *freed = taken + 2, *chain = freed + 2, *ack = chain + 2;
-    volatile int *step_now = reinterpret_cast<volatile int *>(half + kBars);  // the step this CTA is at
+    Tail *tail = reinterpret_cast<Tail *>(half + kBars);
     const int T = blockDim.x;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const bool below = rank > 0, above = rank < k - 1;
@@ -90,7 +169,7 @@ __global__ void __launch_bounds__(kMaxThreads, 1) rod_split_kernel(KParams p, in
         MB[i] = QB[i] = 0ull;
     }
     if (threadIdx.x == 0) {
-        *step_now = 0;
+        *tail = Tail{};
         for (int b = 0; b < 2; ++b) {
             mbar_init(half + b, wp);
             mbar_init(taken + b, wp);
@@ -119,18 +198,17 @@ __global__ void __launch_bounds__(kMaxThreads, 1) rod_split_kernel(KParams p, in
     const long long se = p.sample_every;
     const bool sampling = samples && se > 0;
     const long long k_first = sampling ? step0 / se + 1 : 0;
-    bool dead = false;  // a wait gave up: no more waiting
-    auto wait = [&](uint64_t *bar, unsigned parity) {
-        if (dead) return;
-        if (!mbar_wait(bar, parity, limit_ns)) {
+    // a warp with a wait that gave up tells the cluster
+    auto tell = [&] {
+        if (lane == 0) {
             atomicOr(status, 2);
-            dead = true;
+            for (int r = 0; r < k; ++r) st_cluster(in_rank(smem_u32(&tail->gave_up), r), 1u);
         }
     };
 
     if (warp < wp) {
         // thread t has segment t / rows of row t mod rows
-        const bool act = (int)threadIdx.x < nseg * rows;
+        bool act = (int)threadIdx.x < nseg * rows;
         const int seg = act ? (int)threadIdx.x / rows : 0, row = act ? (int)threadIdx.x - seg * rows : 0;
         const int y = row % ny, X0 = seg * W, q = X0 * PL + ny + row;
         const int nw = FULL ? W : min(W, px - X0);                  // pairs of this segment
@@ -152,13 +230,14 @@ __global__ void __launch_bounds__(kMaxThreads, 1) rod_split_kernel(KParams p, in
         }
         // a first- or last-line segment's place in the neighbours' ghost lines of M, and their barriers
         unsigned belowA = 0, belowB = 0, aboveA = 0, aboveB = 0, bar_below = 0, bar_above = 0;
-        if (below && act && row < ny) {
+        const bool to_below = below && act && row < ny && !withhold, to_above = above && act && row >= rows - ny;
+        if (to_below) {
             const int r = X0 * PL + ny + (z0 - slab_start(nz, k, rank - 1)) * ny + row;
             belowA = in_rank(smem_u32(MA + r), rank - 1);
             belowB = in_rank(smem_u32(MB + r), rank - 1);
             bar_below = in_rank(smem_u32(half), rank - 1);
         }
-        if (above && act && row >= rows - ny) {
+        if (to_above) {
             const int r = X0 * PL + row - (rows - ny);
             aboveA = in_rank(smem_u32(MA + r), rank + 1);
             aboveB = in_rank(smem_u32(MB + r), rank + 1);
@@ -203,12 +282,26 @@ __global__ void __launch_bounds__(kMaxThreads, 1) rod_split_kernel(KParams p, in
             if (w >= nw) return zero_p3();
             return lone && w == nw - 1 ? pair3(lo3(v), none) : v;
         };
+        // A thread whose wait ran out stores and arrives no more, here or beside the slab, and its warp leaves the
+        // loop within a block of steps (a vote in every wait cost up to 13 % of a step).  What starves it starves the
+        // cluster within a few half-steps, so that all of it gives up at about the same time.
+        bool alive = true;
+        unsigned stored = 0;  // the half-steps whose values it had stored
         auto arrive = [&](int b) {
             __syncwarp();
-            if (threadIdx.x == 0)
-                mbar_arrive_expect(half + b, line_bytes);
-            else if (lane == 0)
-                mbar_arrive(half + b);
+            if (lane == 0 && alive) {
+                if (threadIdx.x == 0)
+                    mbar_arrive_expect(half + b, line_bytes);
+                else
+                    mbar_arrive(half + b);
+            }
+        };
+        auto wait = [&](uint64_t *bar, unsigned parity, unsigned so_far) {
+            if (!alive) return;
+            if (!mbar_try_wait(bar, parity) && !slow_wait(bar, parity, limit_ns)) {
+                stored = so_far;
+                alive = act = false;
+            }
         };
         const PairCoeffs cf = pair_coeffs(p);
         const PhiloxKeys keys = philox_keys(p.seed, p.real0 + (uint32_t)rod);
@@ -227,50 +320,62 @@ __global__ void __launch_bounds__(kMaxThreads, 1) rod_split_kernel(KParams p, in
         float Hn = field.next(p);
         int to_sample = sampling ? (int)(k_first * se - step0) : -1;
         unsigned n_snap = 0;
-        for (int s = 0; s < n_steps; ++s) {
-            if (threadIdx.x == 0) *step_now = s;
-            const float Hn1 = field.next(p);
-            const PhiloxStep next = philox_step(keys, (unsigned long long)(step0 + s + 1));
-            const pair_t H0 = both(Hn), H1 = both(Hn1);
-            Pair3 t[W], s0[W], h[W];
-            float3 l = beside_left(MA, MB), r = beside_right(MA, MB);
+        int s = 0;
+        while (s < n_steps && __all_sync(0xffffffffu, alive)) {
+            const int until = min(n_steps, s + kBlock);
+            if (threadIdx.x == 0) *(volatile int *)&tail->step_now = s;
+            for (; s < until; ++s) {
+                const float Hn1 = field.next(p);
+                const PhiloxStep next = philox_step(keys, (unsigned long long)(step0 + s + 1));
+                const pair_t H0 = both(Hn), H1 = both(Hn1);
+                Pair3 t[W], s0[W], h[W];
+                float3 l = beside_left(MA, MB), r = beside_right(MA, MB);
 #pragma unroll
-            for (int w = 0; w < W; ++w) {
-                h[w] = hn[w];
-                s0[w] = llg_torque_p3(m[w], effective_field_p3<AX>(sum(m, w, l, r, MA, MB), m[w], h[w], cf, H0, u[w]), cf.alpha);
-                t[w] = real_cells(normalised_p3(axpy_p3(cf.neg_dt_g1, s0[w], m[w])), w);
+                for (int w = 0; w < W; ++w) {
+                    h[w] = hn[w];
+                    s0[w] = llg_torque_p3(m[w], effective_field_p3<AX>(sum(m, w, l, r, MA, MB), m[w], h[w], cf, H0, u[w]), cf.alpha);
+                    t[w] = real_cells(normalised_p3(axpy_p3(cf.neg_dt_g1, s0[w], m[w])), w);
+                }
+#pragma unroll
+                for (int w = 0; w < W; ++w) put(0, w, t[w]);
+                arrive(0);
+#pragma unroll
+                for (int w = 0; w < (W + 1) / 2; ++w) hn[w] = draw(next, w);
+                wait(half, (unsigned)s & 1u, 2u * s + 1u);
+                l = beside_left(QA, QB), r = beside_right(QA, QB);
+#pragma unroll
+                for (int w = 0; w < W; ++w) {
+                    const Pair3 H = effective_field_p3<AX>(sum(t, w, l, r, QA, QB), t[w], h[w], cf, H1, u[w]);
+                    const Pair3 sv = llg_torque_add_p3(s0[w], t[w], H, cf.alpha);
+                    m[w] = real_cells(normalised_p3(axpy_p3(cf.neg_hdt_g1, sv, m[w])), w);
+                }
+#pragma unroll
+                for (int w = 0; w < W; ++w) put(1, w, m[w]);
+                arrive(1);
+#pragma unroll
+                for (int w = (W + 1) / 2; w < W; ++w) hn[w] = draw(next, w);
+                wait(half + 1, (unsigned)s & 1u, 2u * s + 2u);
+                Hn = Hn1;
+                if (--to_sample == 0) {
+                    to_sample = (int)se;
+                    const unsigned b = n_snap & 1u;
+                    wait(freed + b, ((n_snap >> 1) & 1u) ^ 1u, 2u * s + 2u);  // the sampler is done with the buffer's last use
+#pragma unroll
+                    for (int w = 0; w < W; ++w)
+                        if (has(w)) snap[(b * px + X0 + w) * cap + row] = m[w].z;
+                    __syncwarp();
+                    if (lane == 0 && alive) mbar_arrive(taken + b);
+                    ++n_snap;
+                }
             }
-#pragma unroll
-            for (int w = 0; w < W; ++w) put(0, w, t[w]);
-            arrive(0);
-#pragma unroll
-            for (int w = 0; w < (W + 1) / 2; ++w) hn[w] = draw(next, w);
-            wait(half, (unsigned)s & 1u);
-            l = beside_left(QA, QB), r = beside_right(QA, QB);
-#pragma unroll
-            for (int w = 0; w < W; ++w) {
-                const Pair3 H = effective_field_p3<AX>(sum(t, w, l, r, QA, QB), t[w], h[w], cf, H1, u[w]);
-                const Pair3 sv = llg_torque_add_p3(s0[w], t[w], H, cf.alpha);
-                m[w] = real_cells(normalised_p3(axpy_p3(cf.neg_hdt_g1, sv, m[w])), w);
-            }
-#pragma unroll
-            for (int w = 0; w < W; ++w) put(1, w, m[w]);
-            arrive(1);
-#pragma unroll
-            for (int w = (W + 1) / 2; w < W; ++w) hn[w] = draw(next, w);
-            wait(half + 1, (unsigned)s & 1u);
-            Hn = Hn1;
-            if (--to_sample == 0) {
-                to_sample = (int)se;
-                const unsigned b = n_snap & 1u;
-                wait(freed + b, ((n_snap >> 1) & 1u) ^ 1u);  // the sampler is done with the buffer's last use
-#pragma unroll
-                for (int w = 0; w < W; ++w)
-                    if (has(w)) snap[(b * px + X0 + w) * cap + row] = m[w].z;
-                __syncwarp();
-                if (lane == 0) mbar_arrive(taken + b);
-                ++n_snap;
-            }
+        }
+        if (__any_sync(0xffffffffu, !alive)) tell();
+        if (alive) stored = 2u * s;
+        __syncwarp();
+        cluster_sync();  // no CTA stores into a neighbour any more
+        if (*(volatile unsigned *)&tail->gave_up) {  // the state stays what it was
+            abandon(half, tail, stored, nw, (to_below ? 1 : 0) | (to_above ? 2 : 0), rank, line_bytes, wp, limit_ns);
+            return;
         }
         if (act) {
 #pragma unroll
@@ -288,7 +393,9 @@ __global__ void __launch_bounds__(kMaxThreads, 1) rod_split_kernel(KParams p, in
                 }
             }
         }
-    } else if (sampling) {
+        return;
+    }
+    if (sampling) {
         const int first = z0 * ny * nx, count = rows * nx;  // the slab's cells
         const int o = first & 31;                           // the lane of the first
         unsigned chain_up = 0, carry_up = 0, ack_down = 0;
@@ -297,34 +404,16 @@ __global__ void __launch_bounds__(kMaxThreads, 1) rod_split_kernel(KParams p, in
             chain_up = in_rank(smem_u32(chain), rank + 1);
             carry_up = in_rank(smem_u32(carry + lane), rank + 1);
         }
-        // A wait of the sampler, the same in all its lanes.  The steps to the next sample may take longer
-        // than any wait's limit: the limit runs from the last change of the CTA's step.
-        auto sampler_wait = [&](uint64_t *bar, unsigned parity) {
-            if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
-            int at = *step_now;
-            unsigned long long t0 = timer_ns();
-            while (!__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) {
-                const int now = *step_now;
-                const unsigned long long t = timer_ns();
-                if (now != at) {
-                    at = now;
-                    t0 = t;
-                }
-                if (__any_sync(0xffffffffu, t - t0 > limit_ns)) {
-                    if (lane == 0) atomicOr(status, 2);
-                    return false;
-                }
-            }
-            return true;
-        };
+        auto wait = [&](uint64_t *bar, unsigned parity) { return sampler_wait(bar, parity, tail, limit_ns); };
         const long long k_last = (step0 + n_steps) / se;
         unsigned n = 0;
+        bool ok = true;
         for (long long kk = k_first; kk <= k_last; ++kk, ++n) {
             const unsigned b = n & 1u, use = (n >> 1) & 1u;
-            if (!sampler_wait(taken + b, use)) break;  // and no sample after a wait that gave up
+            if (!(ok = wait(taken + b, use))) break;
             float part = 0.f;
             if (below) {
-                if (!sampler_wait(chain + b, use)) break;
+                if (!(ok = wait(chain + b, use))) break;
                 part = carry[b * 32 + lane];
                 __syncwarp();
                 if (lane == 0) mbar_arrive_cluster(ack_down + 8u * b);
@@ -337,7 +426,7 @@ __global__ void __launch_bounds__(kMaxThreads, 1) rod_split_kernel(KParams p, in
             __syncwarp();
             if (lane == 0) mbar_arrive(freed + b);
             if (above) {
-                if (!sampler_wait(ack + b, use ^ 1u)) break;  // the slab above has read the carry's last use
+                if (!(ok = wait(ack + b, use ^ 1u))) break;  // the slab above has read the carry's last use
                 st_cluster(carry_up + b * 128u, part);
                 __syncwarp();
                 if (lane == 0) mbar_arrive_cluster(chain_up + 8u * b);
@@ -349,10 +438,11 @@ __global__ void __launch_bounds__(kMaxThreads, 1) rod_split_kernel(KParams p, in
                 }
             }
         }
+        if (!ok) tell();  // and no sample after it
     }
-    // no CTA leaves while a neighbour may still store into it
     __syncwarp();
     cluster_sync();
+    if (*(volatile unsigned *)&tail->gave_up) cluster_sync();
 }
 
 template <int W, bool FULL, bool AX, int SHAPE>
@@ -374,7 +464,7 @@ cudaError_t launch(const KParams &p, const RodPlan &plan, float *m, int n_real, 
     cfg.attrs = at;
     cfg.numAttrs = 1;
     return cudaLaunchKernelEx(&cfg, kern, p, plan.split, plan.physics_warps, m, step0, n_steps, samples, status,
-                              plan.handoff_timeout_ns);
+                              plan.handoff_timeout_ns, plan.withhold_handoff ? 1 : 0);
 }
 
 template <int W, bool FULL>

@@ -123,7 +123,8 @@ struct RodPlan {
     bool generic = false;  // kind 2: use the runtime-nx kernel even where a specialised one exists
     bool balance = true;   // kind 2: balance rod-steps over a co-resident grid (needs flags)
     unsigned long long handoff_timeout_ns = 30000000000ull;  // kinds 2 (balanced) and 4: longest hand-off wait
-    bool withhold_handoff = false;  // test hook: balanced producers never release (waits run out)
+    bool withhold_handoff = false;  // test hook: balanced producers never release, cut rods' CTAs
+                                    // send the one below nothing (waits run out)
 };
 // Choose a launch plan for n_real rods of this grid on device `dev`; returns false if no
 // resident kernel can hold the rod.

@@ -1,7 +1,8 @@
-"""Rods cut over several CTAs: the waits' limit."""
+"""Rods cut over several CTAs: the waits' limit and what happens when one runs out."""
 import pytest
 
 from test_gpu_pairs import ensemble, pkg  # noqa: F401  (pkg: the fixture)
+from workloads import MAGNETITE as M
 
 pytestmark = pytest.mark.gpu
 
@@ -20,3 +21,46 @@ def test_samples_further_apart_than_the_wait_limit(pkg, dims, n_real, b, dt):  #
     assert ref_s.shape[1] == 2
     m, s = ensemble(pkg, dims, n_real, tune=((pkg.TUNE_HANDOFF_TIMEOUT_MS, 2),), **kw)
     assert torch.equal(m, ref) and torch.equal(s, ref_s)
+
+
+def cut_grid(pkg, dims):  # noqa: F811
+    g = pkg.Grid(*dims, a0=M["a0"])
+    g.set_material(A0=M["A0"], Ms=M["Ms"], K0=M["K0"], alpha=M["alpha"], T=M["T"])
+    g.set_scaling(mode=1, Tc=M["Tc"])
+    g.set_sweep(H_start=1500.0, H_turn=-1500.0, rate=1e5, dt=2e-15, sample_dH=0.2)  # a sample every step
+    g.set_engine(pkg.ENGINE_RESIDENT)
+    return g
+
+
+@pytest.mark.parametrize("dims,n_real", [((8, 24, 56), 2), ((8, 24, 56), 32), ((4, 12, 28), 3), ((4, 12, 28), 70),
+                                         ((5, 11, 23), 3), ((7, 9, 13), 2), ((6, 16, 30), 30), ((1, 15, 40), 2)])
+def test_wait_that_runs_out_then_recovery(pkg, dims, n_real):  # noqa: F811
+    """With the lines to the slab below withheld on purpose and a limit of 20 ms every rod's CTAs give up: the
+    launch ends, llg_sync reports ETIMEOUT, no sample is written and the state stays what it was.  The same
+    context then runs normally, bitwise the plain engine."""
+    g = cut_grid(pkg, dims)
+    g.set_tuning(pkg.TUNE_HANDOFF_TIMEOUT_MS, 20)
+    g.set_tuning(pkg.TUNE_WITHHOLD_HANDOFF, 1)
+    g.reset(seed=3, n_real=n_real)
+    before = torch.empty((n_real, g.ncells, 3), device="cuda")
+    g.get_state(before)
+    S = torch.full((n_real, g.n_samples), 7.0, device="cuda")
+    g.advance(50, S)
+    with pytest.raises(pkg.LLGError) as e:
+        g.sync(120)
+    assert e.value.status == 5 and "hand-off" in str(e.value)
+    after = torch.empty_like(before)
+    g.get_state(after)
+    assert torch.equal(after, before) and bool((S == 7.0).all())
+    g.set_tuning(pkg.TUNE_WITHHOLD_HANDOFF, 0)
+    out = []
+    for engine in (pkg.ENGINE_RESIDENT, pkg.ENGINE_PLAIN):
+        g.set_engine(engine)
+        g.reset(seed=3, n_real=n_real)
+        S.fill_(7.0)
+        g.advance(50, S)
+        g.get_state(after)
+        g.sync(120)
+        out.append((after.clone(), S.clone()))
+    assert torch.equal(out[0][0], out[1][0]) and torch.equal(out[0][1], out[1][1])
+    g.close()
