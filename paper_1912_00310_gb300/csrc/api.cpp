@@ -183,16 +183,24 @@ struct DeviceGuard {
     }
 };
 
+// What a resident launch takes from the context's settings beside its shape, and whether it may take several
+// SMs for a rod.
+void set_launch_options(const llg_ctx *c, llg::RodPlan *plan)
+{
+    plan->generic = c->tune_generic != 0;
+    plan->balance = c->tune_balance != 0;
+    plan->handoff_timeout_ns = (unsigned long long)c->handoff_timeout_ms * 1000000ull;
+    plan->withhold_handoff = c->withhold_handoff != 0;
+}
+bool launches_alone(const llg_ctx *c) { return !c->tune_generic && c->tune_balance; }
+
 int resolve_engine(const llg_ctx *c, const llg::KParams &kp, int n_real, llg::RodPlan *plan,
                    llg::SlabPlan *splan)
 {
     const bool rod_ok =
         llg::rod_plan(kp, n_real, c->device, plan, c->tune_kind, c->tune_rods, c->tune_rows, c->tune_cpt,
-                       !c->tune_generic && c->tune_balance);
-    plan->generic = c->tune_generic != 0;
-    plan->balance = c->tune_balance != 0;
-    plan->handoff_timeout_ns = (unsigned long long)c->handoff_timeout_ms * 1000000ull;
-    plan->withhold_handoff = c->withhold_handoff != 0;
+                       launches_alone(c));
+    set_launch_options(c, plan);
     auto slab_ok = [&]() {  // planned only where it may be taken
         llg::SlabPlan tmp;
         return llg::slab_plan(kp, n_real, c->device, splan ? splan : &tmp);
@@ -843,8 +851,9 @@ llg_status llg_loop_area_grad(llg_ctx *c, int64_t n_steps, int objective, const 
     if (!llg::adjoint_supported(kp, c->device))
         return fail(LLG_EUNSUPPORTED, "the adjoint handles rods of at most 1024 cells with free faces");
     llg::RodPlan plan{};
-    if (!llg::rod_plan(kp, c->n_real, c->device, &plan, 0, 0, 0, 0, true))
+    if (!llg::rod_plan(kp, c->n_real, c->device, &plan, 0, 0, 0, 0, launches_alone(c)))
         return fail(LLG_EUNSUPPORTED, "no resident forward plan for this grid");
+    set_launch_options(c, &plan);
     const long long ns_total = std::max<long long>(d.n_samples, k_last + 1);
     // store the whole window's states when they fit the budget and a quarter of the free memory
     bool store_all = false;
@@ -880,7 +889,10 @@ llg_status llg_loop_area_grad(llg_ctx *c, int64_t n_steps, int objective, const 
     if (e == cudaSuccess) e = cudaMalloc(&work, sizeof(float) * state);
     if (e == cudaSuccess) e = cudaMalloc(&smp, sizeof(float) * (size_t)c->n_real * (size_t)ns_total);
     if (e == cudaSuccess) e = cudaMalloc(&w, sizeof(double) * (size_t)K);
-    if (e == cudaSuccess) e = cudaMalloc(&partial, sizeof(double) * 5 * (size_t)c->n_real);
+    // the partial sums and, after them, the forward pass's own status word: the ensemble's keeps what an advance
+    // left there
+    const size_t n_partial = 5 * (size_t)c->n_real;
+    if (e == cudaSuccess) e = cudaMalloc(&partial, sizeof(double) * (n_partial + 1));
     if (e != cudaSuccess) {
         cleanup();
         cudaGetLastError();
@@ -890,20 +902,34 @@ llg_status llg_loop_area_grad(llg_ctx *c, int64_t n_steps, int objective, const 
     kps.n_samples = ns_total;
     const cudaStream_t st = c->stream;
     // forward pass with a checkpoint at the start of every segment
+    int *const fwd_status = reinterpret_cast<int *>(partial + n_partial);
     e = cudaMemcpyAsync(work, c->d_m, sizeof(float) * state, cudaMemcpyDeviceToDevice, st);
+    if (e == cudaSuccess) e = cudaMemsetAsync(fwd_status, 0, sizeof(int), st);
     for (long long sg = 0; sg < S && e == cudaSuccess; ++sg) {
         e = cudaMemcpyAsync(ckpt + (size_t)sg * state, work, sizeof(float) * state, cudaMemcpyDeviceToDevice, st);
         const long long len = std::min(C, N - sg * C);
         if (e == cudaSuccess)
-            e = llg::rod_advance(kps, plan, work, c->n_real, step0 + sg * C, len, smp, c->d_status, nullptr, st);
+            e = llg::rod_advance(kps, plan, work, c->n_real, step0 + sg * C, len, smp, fwd_status, nullptr, st);
     }
     std::vector<float> hs((size_t)c->n_real * (size_t)ns_total);
+    int hst = 0;
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(hs.data(), smp, sizeof(float) * hs.size(), cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(&hst, fwd_status, sizeof(int), cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    if (e == cudaSuccess && (hst & 1)) {  // a non-finite sample: the loss says so, and so does the next llg_sync
+        int all = 0;
+        e = cudaMemcpy(&all, c->d_status, sizeof(int), cudaMemcpyDeviceToHost);
+        all |= 1;
+        if (e == cudaSuccess) e = cudaMemcpy(c->d_status, &all, sizeof(int), cudaMemcpyHostToDevice);
+    }
     if (e != cudaSuccess) {
         cleanup();
         return cuda_fail(e, "adjoint forward");
+    }
+    if (hst & 2) {
+        cleanup();
+        return fail(LLG_ETIMEOUT, "a resident-engine hand-off wait gave up in the gradient's forward pass");
     }
     // loss and its weights on the realisation-mean samples
     std::vector<double> mbar((size_t)K, 0.0), wk;
@@ -915,7 +941,7 @@ llg_status llg_loop_area_grad(llg_ctx *c, int64_t n_steps, int objective, const 
     const double L = window_loss(d, c->sw, objective, target, k_first, K, mbar, wk);
     e = cudaMemcpyAsync(w, wk.data(), sizeof(double) * (size_t)K, cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess) e = cudaMemsetAsync(lam, 0, sizeof(float) * state, st);
-    if (e == cudaSuccess) e = cudaMemsetAsync(partial, 0, sizeof(double) * 5 * (size_t)c->n_real, st);
+    if (e == cudaSuccess) e = cudaMemsetAsync(partial, 0, sizeof(double) * n_partial, st);
     if (store_all) {
         if (e == cudaSuccess) e = llg::adjoint_recompute_all(kps, c->n_real, step0, N, (int)C, ckpt, seg, st);
         if (e == cudaSuccess)
@@ -927,7 +953,7 @@ llg_status llg_loop_area_grad(llg_ctx *c, int64_t n_steps, int objective, const 
                                      ckpt + (size_t)sg * state, seg, lam, w, partial, st);
         }
     }
-    std::vector<double> hp((size_t)c->n_real * 5);
+    std::vector<double> hp(n_partial);
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(hp.data(), partial, sizeof(double) * hp.size(), cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);

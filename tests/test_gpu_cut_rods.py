@@ -1,4 +1,7 @@
 """Rods cut over several CTAs: the waits' limit and what happens when one runs out."""
+import math
+
+import numpy as np
 import pytest
 
 from test_gpu_pairs import ensemble, pkg  # noqa: F401  (pkg: the fixture)
@@ -63,4 +66,42 @@ def test_wait_that_runs_out_then_recovery(pkg, dims, n_real):  # noqa: F811
         g.sync(120)
         out.append((after.clone(), S.clone()))
     assert torch.equal(out[0][0], out[1][0]) and torch.equal(out[0][1], out[1][1])
+    g.close()
+
+
+def test_gradient_reports_a_wait_that_ran_out(pkg):  # noqa: F811
+    """The gradient's forward pass may cut its rods too: a wait that runs out there is ETIMEOUT and no loss, the
+    ensemble (whose state the gradient does not touch) is not marked, and the next gradient is the one that
+    the rods give uncut."""
+    g = cut_grid(pkg, (5, 11, 17))  # 935 cells
+    g.reset(seed=3, n_real=3)
+    target = np.linspace(1.0, -1.0, g.n_samples)
+    g.set_tuning(pkg.TUNE_HANDOFF_TIMEOUT_MS, 20)
+    g.set_tuning(pkg.TUNE_WITHHOLD_HANDOFF, 1)
+    with pytest.raises(pkg.LLGError) as e:
+        g.loss_grad(100, target, 0, 64)
+    assert e.value.status == 5 and "hand-off" in str(e.value)
+    g.sync(60)
+    g.set_tuning(pkg.TUNE_WITHHOLD_HANDOFF, 0)
+    L, grad = g.loss_grad(100, target, 0, 64)
+    g.set_tuning(pkg.TUNE_BALANCE, 0)  # one SM a rod
+    L1, grad1 = g.loss_grad(100, target, 0, 64)
+    assert L == L1 and np.array_equal(grad, grad1)
+    g.close()
+
+
+@pytest.mark.parametrize("n_real", [3, 200])
+def test_gradient_of_a_non_finite_state(pkg, n_real):  # noqa: F811
+    """A loss that is not a number is returned as such and reported by the next llg_sync."""
+    g = cut_grid(pkg, (5, 11, 17))
+    g.reset(seed=3, n_real=n_real)
+    m = torch.zeros((n_real, g.ncells, 3), device="cuda")
+    m[..., 2] = 1.0
+    m[1, 7, 0] = float("nan")
+    g.set_state(m, 0)
+    L, _ = g.loss_grad(100, np.zeros(g.n_samples), 0, 64)
+    assert math.isnan(L)
+    with pytest.raises(pkg.LLGError) as e:
+        g.sync(60)
+    assert e.value.status == 4
     g.close()
