@@ -850,8 +850,11 @@ llg_status llg_loop_area_grad(llg_ctx *c, int64_t n_steps, int objective, const 
                                                  grad_out);
     if (!llg::adjoint_supported(kp, c->device))
         return fail(LLG_EUNSUPPORTED, "the adjoint handles rods of at most 1024 cells with free faces");
+    // the forward pass runs on the automatic plan; the grids are those that the two-phase kernel takes (which
+    // leaves out thin ones of many cells, and sample intervals of 2^31 steps, as the reverse pass does)
     llg::RodPlan plan{};
-    if (!llg::rod_plan(kp, c->n_real, c->device, &plan, 0, 0, 0, 0, launches_alone(c)))
+    if (!llg::rod_plan(kp, c->n_real, c->device, &plan, 1) ||
+        !llg::rod_plan(kp, c->n_real, c->device, &plan, 0, 0, 0, 0, launches_alone(c)))
         return fail(LLG_EUNSUPPORTED, "no resident forward plan for this grid");
     set_launch_options(c, &plan);
     const long long ns_total = std::max<long long>(d.n_samples, k_last + 1);

@@ -299,3 +299,25 @@ def test_gradient_of_rods_that_fill_their_warps_or_not(pkg, orc, dims, method):
     assert L == pytest.approx(Lo, rel=1e-3)
     for k in range(3):
         assert got[k] == pytest.approx(go[k], rel=1e-2, abs=1e-3 * np.abs(go).max()), (k, got, go)
+
+
+def test_gradient_refuses_what_no_two_phase_rod_holds(pkg):
+    """A thin grid whose ghost-padded rod exceeds shared memory, and samples more than 2^31 steps apart, are
+    EUNSUPPORTED for the adjoint before any work, whichever kernel the forward pass would take."""
+    g = grid(pkg, (1, 1, 1024))
+    g.reset(seed=0, n_real=3)
+    with pytest.raises(pkg.LLGError) as e:
+        g.loss_grad(100, target_for(g), 0, 64)
+    assert e.value.status == 6
+    g.close()
+    g = grid(pkg, (5, 11, 17))
+    g.set_sweep(H_start=5000.0, H_turn=-5000.0, rate=1.0, dt=2e-15, sample_dH=5000.0)
+    assert g.sample_every >= 2 ** 31
+    g.reset(seed=0, n_real=3)
+    m = np.zeros((3, g.ncells, 3), dtype=np.float32)
+    m[..., 2] = 1.0
+    g.set_state(m, g.sample_every - 50)
+    with pytest.raises(pkg.LLGError) as e:
+        g.loss_grad(100, np.zeros(g.n_samples), 0, 64)
+    assert e.value.status == 6
+    g.close()
