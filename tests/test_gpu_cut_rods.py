@@ -26,6 +26,15 @@ def test_samples_further_apart_than_the_wait_limit(pkg, dims, n_real, b, dt):  #
     assert torch.equal(m, ref) and torch.equal(s, ref_s)
 
 
+def test_samples_seconds_apart(pkg):  # noqa: F811
+    """The same under the default limit, 750000 steps (2.6 s) to the sample within one launch."""
+    kw = dict(rate=1000.0, sample_dH=1500.0, steps=(750_007,))
+    ref, ref_s = ensemble(pkg, (8, 24, 56), 32, tune=((pkg.TUNE_ROD_KIND, 2),), **kw)
+    assert ref_s.shape[1] == 1
+    m, s = ensemble(pkg, (8, 24, 56), 32, **kw)
+    assert torch.equal(m, ref) and torch.equal(s, ref_s)
+
+
 def cut_grid(pkg, dims):  # noqa: F811
     g = pkg.Grid(*dims, a0=M["a0"])
     g.set_material(A0=M["A0"], Ms=M["Ms"], K0=M["K0"], alpha=M["alpha"], T=M["T"])
