@@ -239,6 +239,15 @@ int round_warp(int n) { return (n + 31) / 32 * 32; }
 
 }  // namespace
 
+// Measured, us: b = 2, 4, 8 rods 1.63, 0.44, 0.25; two-phase rods of 58, 312, 819 and 1265 cells 0.36, 0.74, 1.54 and
+// 2.15; the b = 1 rod 11.2; 6x16x30 cells on the runtime-size pipelined kernel 5.4.
+double one_sm_us(const KParams &p, int kind)
+{
+    if (kind == 3) return 0.29 + 0.001 * p.ncells;
+    if (kind == 1) return p.ncells <= 400 ? 0.33 + 0.0014 * p.ncells : 0.42 + 0.0013 * p.ncells;
+    return pairs_supported(p) ? 0.3 + 0.00101 * p.ncells : 0.00186 * p.ncells;
+}
+
 bool rod_plan(const KParams &p, int n_real, int dev, RodPlan *plan, int force_kind, int force_rods,
               int force_rows, int force_cpt, bool alone)
 {
@@ -271,16 +280,10 @@ bool rod_plan(const KParams &p, int n_real, int dev, RodPlan *plan, int force_ki
                                p.sample_every < (1LL << 31) && twophase_shape(p, 1, &one) &&
                                one.pairs_per_thread <= (pairs_supported(p) ? 1 : 2);
         kind = rows_supported(p) ? 3 : (few_cells || few_pairs ? 1 : (pipelined_fits ? 2 : 1));
-        // few rods: several SMs to each, where that is faster than what a step of one rod on one SM takes
-        // (us, measured: b = 2, 4, 8 rods 1.63, 0.44, 0.25; two-phase rods of 58, 312, 819 and 1265 cells 0.36, 0.74,
-        // 1.54 and 2.15; the b = 1 rod 11.2; 6x16x30 cells on the runtime-size pipelined kernel 5.4)
-        if (alone && force_rods == 0 && force_rows == 0 && force_cpt == 0 && n_real < nsm) {
-            const double us = kind == 3   ? 0.29 + 0.001 * p.ncells
-                              : kind == 1 ? (p.ncells <= 400 ? 0.33 + 0.0014 * p.ncells : 0.42 + 0.0013 * p.ncells)
-                              : pairs_supported(p) ? 0.3 + 0.00101 * p.ncells
-                                                   : 0.00186 * p.ncells;
-            if (split_plan(p, n_real, nsm, smem_optin, us, plan)) return true;
-        }
+        // few rods: several SMs to each, where that is faster than one
+        if (alone && force_rods == 0 && force_rows == 0 && force_cpt == 0 && n_real < nsm &&
+            split_plan(p, n_real, nsm, smem_optin, dev, one_sm_us(p, kind), plan))
+            return true;
     }
     if (kind == 3) {
         if (!rows_supported(p)) return false;

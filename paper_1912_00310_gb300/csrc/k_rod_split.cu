@@ -445,35 +445,39 @@ __global__ void __launch_bounds__(kMaxThreads, 1) rod_split_kernel(KParams p, in
     if (*(volatile unsigned *)&tail->gave_up) cluster_sync();
 }
 
-template <int W, bool FULL, bool AX, int SHAPE>
-cudaError_t launch(const KParams &p, const RodPlan &plan, float *m, int n_real, long long step0, int n_steps,
-                   float *samples, int *status, cudaStream_t st)
+// A kernel of the plan's shape and the launch that it takes; cfg's one attribute is *at.
+template <typename K>
+cudaError_t configure(K kern, const RodPlan &plan, int n_real, cudaStream_t st, cudaLaunchConfig_t *cfg, cudaLaunchAttribute *at)
 {
-    auto kern = rod_split_kernel<W, FULL, AX, SHAPE>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)plan.smem_bytes);
-    if (e != cudaSuccess) return e;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(n_real * plan.split));
-    cfg.blockDim = dim3((unsigned)plan.threads);
-    cfg.dynamicSmemBytes = plan.smem_bytes;
-    cfg.stream = st;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = (unsigned)plan.split;
-    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kern, p, plan.split, plan.physics_warps, m, step0, n_steps, samples, status,
-                              plan.handoff_timeout_ns, plan.withhold_handoff ? 1 : 0);
+    *cfg = cudaLaunchConfig_t{};
+    cfg->gridDim = dim3((unsigned)(n_real * plan.split));
+    cfg->blockDim = dim3((unsigned)plan.threads);
+    cfg->dynamicSmemBytes = plan.smem_bytes;
+    cfg->stream = st;
+    at->id = cudaLaunchAttributeClusterDimension;
+    at->val.clusterDim.x = (unsigned)plan.split;
+    at->val.clusterDim.y = at->val.clusterDim.z = 1;
+    cfg->attrs = at;
+    cfg->numAttrs = 1;
+    return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)plan.smem_bytes);
 }
 
-template <int W, bool FULL>
-cudaError_t launch_by(const KParams &p, const RodPlan &plan, float *m, int n_real, long long step0, int n_steps,
-                      float *samples, int *status, cudaStream_t st)
+// use(kernel) with the instance for this grid and plan.
+template <typename F>
+cudaError_t with_kernel(const KParams &p, const RodPlan &plan, F use)
 {
-#define LLG_S(AXV, S) launch<W, FULL, AXV, S>(p, plan, m, n_real, step0, n_steps, samples, status, st)
-    if (p.shape == 1) return p.axis ? LLG_S(true, 1) : LLG_S(false, 1);
-    return p.axis ? LLG_S(true, 0) : LLG_S(false, 0);
+    const bool full = p.nx % (2 * plan.pairs_per_thread) == 0;
+#define LLG_S(W, FULLV, AXV) (p.shape == 1 ? use(rod_split_kernel<W, FULLV, AXV, 1>) : use(rod_split_kernel<W, FULLV, AXV, 0>))
+#define LLG_W(W)                                                                            \
+    (full ? (p.axis ? LLG_S(W, true, true) : LLG_S(W, true, false))                         \
+          : (p.axis ? LLG_S(W, false, true) : LLG_S(W, false, false)))
+    switch (plan.pairs_per_thread) {
+        case 1: return LLG_W(1);
+        case 2: return LLG_W(2);
+        case 4: return LLG_W(4);
+        default: return cudaErrorInvalidValue;
+    }
+#undef LLG_W
 #undef LLG_S
 }
 
@@ -509,49 +513,81 @@ static bool split_shape(const KParams &p, int k, int smem_optin, RodPlan *plan)
     return true;
 }
 
+int split_clusters_at_once(const KParams &p, const RodPlan &plan, int dev)
+{
+    int prev = -1, n = 0;
+    if (cudaGetDevice(&prev) != cudaSuccess || (prev != dev && cudaSetDevice(dev) != cudaSuccess)) {
+        cudaGetLastError();
+        return 0;
+    }
+    const cudaError_t e = with_kernel(p, plan, [&](auto kern) {
+        cudaLaunchConfig_t cfg;
+        cudaLaunchAttribute at;
+        const cudaError_t c = configure(kern, plan, 1, nullptr, &cfg, &at);
+        return c != cudaSuccess ? c : cudaOccupancyMaxActiveClusters(&n, kern, &cfg);
+    });
+    if (prev != dev) cudaSetDevice(prev);
+    if (e == cudaSuccess) return n;
+    cudaGetLastError();
+    return 0;
+}
+
 // Whether cutting the rods beats one rod per SM, which takes base_us a step, and over how many CTAs.  A
 // step of a slab of c pairs takes about 0.72 us + 2 ns c, with four pairs to a thread 2.1 ns where they fill
-// their rows and 3.2 where not: measured 2.06 us at 672 pairs (b = 1 over 8 CTAs), 3.53 at 1344 (over 4),
-// 0.83, 1.02 and 1.29 at 96, 168 and 336 (b = 2 over 8, 4 and 2), 0.90 and 1.12 at 99 and 198 (5x11x23 cells
-// over 8 and 4), 3.03 at 720 (6x16x30 over 2).  Clusters run side by side as far as the GPCs hold them (at
-// one CTA to an SM: 76 of 2, 36 of 4, 28 of 5, 23 of 6, 15 of 7 or 8 on 152 SMs), the rest in further waves.
-bool split_plan(const KParams &p, int n_real, int nsm, int smem_optin, double base_us, RodPlan *plan)
+// their rows and 3.2 where not: measured 2.1 us at 672 pairs (b = 1 over 8 CTAs), 3.5 at 1344 (over 4),
+// 0.80, 1.01 and 1.24 at 96, 168 and 336 (b = 2 over 8, 4 and 2), 0.87 and 1.12 at 99 and 198 (5x11x23 cells
+// over 8 and 4), 3.03 at 720 (6x16x30 over 2).  Clusters run side by side as far as the GPCs hold them, the
+// rest in further waves: kAtOnce is what a GB300 of 152 SMs holds at one CTA to an SM; the device at hand is asked
+// about the choice (one call, not one for each k) and has the last word where it holds fewer, or none: that
+// choice is made again without it, down to one rod per SM.
+bool split_plan(const KParams &p, int n_real, int nsm, int smem_optin, int dev, double base_us, RodPlan *plan,
+                int (*clusters_at_once)(const KParams &, const RodPlan &, int))
 {
-    constexpr int kAtOnce[9] = {0, 152, 76, 48, 36, 28, 23, 15, 15};
-    double best = 0.9 * base_us;
-    bool found = false;
-    for (int k = 2; k <= 8; ++k) {
-        RodPlan t{};
-        if (!split_shape(p, k, smem_optin, &t)) continue;
-        const int at_once = std::max(1, nsm * kAtOnce[k] / 152);
-        const int waves = (n_real + at_once - 1) / at_once;
-        const double c = (double)largest_slab(p.nz, k) * p.ny * ((p.nx + 1) / 2);
-        const double ns = t.pairs_per_thread < 4 ? 2.0 : (p.nx % 8 == 0 ? 2.1 : 3.2);
-        const double us = waves * (0.72 + 1e-3 * ns * c);
-        if (us < best) {
-            best = us;
-            *plan = t;
-            found = true;
+    int at_once[9] = {0, 152, 76, 48, 36, 28, 23, 15, 15};
+    bool asked[9] = {};
+    for (int k = 2; k <= 8; ++k) at_once[k] = std::max(1, nsm * at_once[k] / 152);
+    for (;;) {
+        double best = 0.9 * base_us;
+        RodPlan choice{};
+        for (int k = 2; k <= 8; ++k) {
+            RodPlan t{};
+            if (at_once[k] < 1 || !split_shape(p, k, smem_optin, &t)) continue;
+            const int waves = (n_real + at_once[k] - 1) / at_once[k];
+            const double c = (double)largest_slab(p.nz, k) * p.ny * ((p.nx + 1) / 2);
+            const double ns = t.pairs_per_thread < 4 ? 2.0 : (p.nx % (2 * t.pairs_per_thread) == 0 ? 2.1 : 3.2);
+            const double us = waves * (0.72 + 1e-3 * ns * c);
+            if (us < best) {
+                best = us;
+                choice = t;
+            }
         }
+        const int k = choice.split;
+        if (k == 0) return false;
+        if (!asked[k]) {
+            asked[k] = true;
+            const int n = clusters_at_once(p, choice, dev);
+            if (n < at_once[k]) {
+                at_once[k] = n;
+                continue;
+            }
+        }
+        *plan = choice;
+        plan->ctas = n_real * plan->split;
+        return true;
     }
-    if (found) plan->ctas = n_real * plan->split;
-    return found;
 }
 
 cudaError_t split_advance(const KParams &p, const RodPlan &plan, float *m, int n_real, long long step0, int n_steps,
                           float *samples, int *status, cudaStream_t st)
 {
-    const bool full = p.nx % (2 * plan.pairs_per_thread) == 0;
-#define LLG_W(W)                                                                                          \
-    (full ? launch_by<W, true>(p, plan, m, n_real, step0, n_steps, samples, status, st)                   \
-          : launch_by<W, false>(p, plan, m, n_real, step0, n_steps, samples, status, st))
-    switch (plan.pairs_per_thread) {
-        case 1: return LLG_W(1);
-        case 2: return LLG_W(2);
-        case 4: return LLG_W(4);
-        default: return cudaErrorInvalidValue;
-    }
-#undef LLG_W
+    return with_kernel(p, plan, [&](auto kern) {
+        cudaLaunchConfig_t cfg;
+        cudaLaunchAttribute at;
+        const cudaError_t e = configure(kern, plan, n_real, st, &cfg, &at);
+        if (e != cudaSuccess) return e;
+        return cudaLaunchKernelEx(&cfg, kern, p, plan.split, plan.physics_warps, m, step0, n_steps, samples, status,
+                                  plan.handoff_timeout_ns, plan.withhold_handoff ? 1 : 0);
+    });
 }
 
 }  // namespace llg

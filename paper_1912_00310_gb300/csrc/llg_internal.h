@@ -130,6 +130,8 @@ struct RodPlan {
 // resident kernel can hold the rod.
 // force_kind / force_rods: 0 = automatic.  alone: nothing else is meant to run beside this launch, so
 // that an ensemble of few rods may take several SMs for each (automatic plans only).
+// one_sm_us: about what a step takes with one rod of that kind per SM.
+double one_sm_us(const KParams &p, int kind);
 bool rod_plan(const KParams &p, int n_real, int dev, RodPlan *plan, int force_kind = 0,
               int force_rods = 0, int force_rows = 0, int force_cpt = 0, bool alone = false);
 // Two-phase kernel (k_rod_zpairs.cu): shared memory of one rod, the pairs per thread and threads of
@@ -140,8 +142,11 @@ bool twophase_shape(const KParams &p, int rods, RodPlan *plan);
 // ... and for small rods a cell to a thread instead (pairs_per_thread 0).
 void compact_shape(const KParams &p, RodPlan *plan);
 // Split kernel (k_rod_split.cu, plan kind 4): whether and over how many CTAs the rods of an ensemble that
-// leaves SMs idle are cut (base_us: a step's time with one rod per SM), and the launch.
-bool split_plan(const KParams &p, int n_real, int nsm, int smem_optin, double base_us, RodPlan *plan);
+// leaves SMs idle are cut (base_us: a step's time with one rod per SM), and the launch.  clusters_at_once: how
+// many clusters of a plan the device runs side by side (0: it cannot place one).
+int split_clusters_at_once(const KParams &p, const RodPlan &plan, int dev);
+bool split_plan(const KParams &p, int n_real, int nsm, int smem_optin, int dev, double base_us, RodPlan *plan,
+                int (*clusters_at_once)(const KParams &, const RodPlan &, int) = split_clusters_at_once);
 cudaError_t split_advance(const KParams &p, const RodPlan &plan, float *m, int n_real, long long step0, int n_steps,
                           float *samples, int *status, cudaStream_t st);
 // Row kernel (k_rod_small.cu, plan kind 3): the b = 2, 4, 8 rods with a compile-time instance,

@@ -4,6 +4,7 @@ import math
 import numpy as np
 import pytest
 
+from test_cut_plan import CASES
 from test_gpu_pairs import ensemble, pkg  # noqa: F401  (pkg: the fixture)
 from workloads import MAGNETITE as M
 
@@ -44,12 +45,12 @@ def cut_grid(pkg, dims):  # noqa: F811
     return g
 
 
-@pytest.mark.parametrize("dims,n_real", [((8, 24, 56), 2), ((8, 24, 56), 32), ((4, 12, 28), 3), ((4, 12, 28), 70),
-                                         ((5, 11, 23), 3), ((7, 9, 13), 2), ((6, 16, 30), 30), ((1, 15, 40), 2)])
+@pytest.mark.parametrize("dims,n_real", [c[0:3:2] for c in CASES])
 def test_wait_that_runs_out_then_recovery(pkg, dims, n_real):  # noqa: F811
     """With the lines to the slab below withheld on purpose and a limit of 20 ms every rod's CTAs give up: the
-    launch ends, llg_sync reports ETIMEOUT, no sample is written and the state stays what it was.  The same
-    context then runs normally, bitwise the plain engine."""
+    launch ends, llg_sync reports ETIMEOUT (which shows that the rods were cut: no other kernel waits with fewer
+    rods than SMs), no sample is written and the state stays what it was.  The same context then runs
+    normally, bitwise the plain engine."""
     g = cut_grid(pkg, dims)
     g.set_tuning(pkg.TUNE_HANDOFF_TIMEOUT_MS, 20)
     g.set_tuning(pkg.TUNE_WITHHOLD_HANDOFF, 1)
