@@ -168,8 +168,9 @@ llg_status llg_set_engine(llg_ctx *ctx, int engine);
 /* Launch-shape overrides of the resident engine (0 = automatic, the default):
  *   LLG_TUNE_ROD_KIND      1 two-phase kernel, 2 plane-pipelined kernel, 3 row kernel (the
  *                          b = 2, 4, 8 rods of the paper's ladder: a thread per x-row); an
- *                          ensemble of fewer rods than SMs may be cut over several SMs a rod, which
- *                          only the automatic choice does
+ *                          ensemble of fewer rods than SMs may be cut over several SMs a rod: only
+ *                          by the automatic choice, with LLG_TUNE_BALANCE 1, and on the legacy
+ *                          default stream (contexts on streams of their own run side by side)
  *   LLG_TUNE_RODS_PER_CTA  rods per CTA of the two-phase and row kernels
  *   LLG_TUNE_CHUNK_STEPS   Heun steps per launch (default 2^20; llg_autotune sets it so the
  *                          launch overhead stays near 1% of a launch)
@@ -177,7 +178,8 @@ llg_status llg_set_engine(llg_ctx *ctx, int engine);
  *   LLG_TUNE_GENERIC_KERNEL   1: the runtime-size plane-pipelined kernel even where a kernel
  *                             specialised for the plane count exists
  *   LLG_TUNE_BALANCE          0: one rod per CTA even when the rods do not fill whole waves
- *                             (default 1: rod-steps balanced over a co-resident grid)
+ *                             (default 1: rod-steps balanced over a co-resident grid); 0 also
+ *                             keeps the rods of a small ensemble whole
  *   LLG_TUNE_ADJOINT_STATE_MB device memory (MB, default 16384) that llg_loop_area_grad may hold
  *                             for the whole window's states (12 bytes per cell, realisation and
  *                             step); within it every checkpoint segment is recomputed in one
@@ -288,7 +290,7 @@ llg_status llg_run_batch(llg_ctx *const *jobs, int n_jobs, int64_t max_steps,
  * from the measured time of a one-step launch, so that the launch overhead stays near 1% of a
  * launch.  Results are cached for the life of the process per (device, grid, realisation
  * count, sweep shape, whether the sweep and sample counts fit 32 bits, dispersed axes, periodic
- * faces), and a cached shape is used only while it still plans for the context.  The ensemble
+ * faces, whether rods may be cut over several SMs), and a cached shape is used only while it still plans for the context.  The ensemble
  * itself is not advanced.  best_rate (optional) receives the fastest
  * cell-steps/s.  Synchronises.  Errors: EINVAL (no ensemble), ENOMEM, EUNSUPPORTED. */
 llg_status llg_autotune(llg_ctx *ctx, int64_t trial_steps, double *best_rate);

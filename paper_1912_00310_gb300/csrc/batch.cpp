@@ -37,14 +37,14 @@ namespace {
 
 // Autotuned launch shapes, keyed by what selects the kernel instances: the device, the grid, the
 // ensemble size, the sweep shape, whether the sweep and sample bookkeeping fit 32 bits, dispersed
-// axes and the periodic faces.
+// axes, the periodic faces and whether the rods may be cut over several SMs.
 struct TuneKey {
     std::string device;
-    int nx, ny, nz, n_real, shape, fits32, axes, periodic;
+    int nx, ny, nz, n_real, shape, fits32, axes, periodic, may_cut;
     bool operator<(const TuneKey &o) const
     {
-        return std::tie(device, nx, ny, nz, n_real, shape, fits32, axes, periodic) <
-               std::tie(o.device, o.nx, o.ny, o.nz, o.n_real, o.shape, o.fits32, o.axes, o.periodic);
+        return std::tie(device, nx, ny, nz, n_real, shape, fits32, axes, periodic, may_cut) <
+               std::tie(o.device, o.nx, o.ny, o.nz, o.n_real, o.shape, o.fits32, o.axes, o.periodic, o.may_cut);
     }
 };
 struct TuneValue {
@@ -132,7 +132,7 @@ extern "C" llg_status llg_autotune(llg_ctx *ctx, int64_t trial_steps, double *be
     const long long period = v.kp.shape == 1 ? v.kp.period : 2 * v.kp.n_half;
     const int fits32 = period < (1LL << 31) && v.kp.sample_every < (1LL << 31);
     const TuneKey key{prop.name, v.kp.nx, v.kp.ny, v.kp.nz, v.n_real, v.kp.shape, fits32,
-                      v.kp.axis != nullptr, (int)v.kp.periodic};
+                      v.kp.axis != nullptr, (int)v.kp.periodic, v.may_cut};
     {
         std::lock_guard<std::mutex> lock(g_tune_mutex);
         auto it = g_tune_cache.find(key);
@@ -173,7 +173,7 @@ extern "C" llg_status llg_autotune(llg_ctx *ctx, int64_t trial_steps, double *be
     double best_ms = 0.0;
     for (auto [kind, rods, rows, cpt] : cand) {
         llg::RodPlan plan{};
-        if (!llg::rod_plan(v.kp, v.n_real, v.device, &plan, kind, rods, rows, cpt, true)) continue;
+        if (!llg::rod_plan(v.kp, v.n_real, v.device, &plan, kind, rods, rows, cpt, v.may_cut)) continue;
         if (kind == 2 && rows == 0 && plan.kind != 2) continue;
         plan.balance = true;
         double t_best = 1e30;
@@ -268,7 +268,7 @@ extern "C" llg_status llg_run_batch(llg_ctx *const *jobs, int n_jobs, int64_t ma
         const long long left = v.steps_per_loop > 0 ? std::max(0LL, v.steps_per_loop - v.step) : max_steps;
         steps[(size_t)j] = std::min<long long>(left, max_steps);
         if (!llg::rod_plan(v.kp, v.n_real, v.device, &plans[(size_t)j], v.tune_kind, v.tune_rods, v.tune_rows,
-                           v.tune_cpt)) {
+                           v.tune_cpt, false, true)) {
             char msg[128];
             std::snprintf(msg, sizeof msg, "batch job %d: the resident engine cannot hold its grid", j);
             llg::set_last_error(msg);

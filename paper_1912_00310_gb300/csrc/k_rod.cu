@@ -249,7 +249,7 @@ double one_sm_us(const KParams &p, int kind)
 }
 
 bool rod_plan(const KParams &p, int n_real, int dev, RodPlan *plan, int force_kind, int force_rods,
-              int force_rows, int force_cpt, bool alone)
+              int force_rows, int force_cpt, bool may_cut, bool in_batch)
 {
     int smem_optin = 0, nsm = 0;
     if (cudaDeviceGetAttribute(&smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess ||
@@ -281,7 +281,7 @@ bool rod_plan(const KParams &p, int n_real, int dev, RodPlan *plan, int force_ki
                                one.pairs_per_thread <= (pairs_supported(p) ? 1 : 2);
         kind = rows_supported(p) ? 3 : (few_cells || few_pairs ? 1 : (pipelined_fits ? 2 : 1));
         // few rods: several SMs to each, where that is faster than one
-        if (alone && force_rods == 0 && force_rows == 0 && force_cpt == 0 && n_real < nsm &&
+        if (may_cut && force_rods == 0 && force_rows == 0 && force_cpt == 0 && n_real < nsm &&
             split_plan(p, n_real, nsm, smem_optin, dev, one_sm_us(p, kind), plan))
             return true;
     }
@@ -312,7 +312,7 @@ bool rod_plan(const KParams &p, int n_real, int dev, RodPlan *plan, int force_ki
         plan->rows_per_thread = 1;
         plan->smem_bytes = rows_smem_bytes(p, rods);
         plan->ctas = (n_real + rods - 1) / rods;
-        plan->crowded = !alone || plan->ctas > nsm;
+        plan->crowded = in_batch || plan->ctas > nsm;
         return true;
     }
     if (kind == 1) {

@@ -128,12 +128,13 @@ struct RodPlan {
 };
 // Choose a launch plan for n_real rods of this grid on device `dev`; returns false if no
 // resident kernel can hold the rod.
-// force_kind / force_rods: 0 = automatic.  alone: nothing else is meant to run beside this launch, so
-// that an ensemble of few rods may take several SMs for each (automatic plans only).
-// one_sm_us: about what a step takes with one rod of that kind per SM.
-double one_sm_us(const KParams &p, int kind);
+// force_kind / force_rods: 0 = automatic.  may_cut: an ensemble of few rods may take several SMs for
+// each (automatic plans only).  in_batch: other jobs' launches run beside this one.
 bool rod_plan(const KParams &p, int n_real, int dev, RodPlan *plan, int force_kind = 0,
-              int force_rods = 0, int force_rows = 0, int force_cpt = 0, bool alone = false);
+              int force_rods = 0, int force_rows = 0, int force_cpt = 0, bool may_cut = false,
+              bool in_batch = false);
+// About what a step takes with one rod of that kind per SM.
+double one_sm_us(const KParams &p, int kind);
 // Two-phase kernel (k_rod_zpairs.cu): shared memory of one rod, the pairs per thread and threads of
 // `rods` rods in a CTA (false: too many), the largest CTA of a request for cpt cells per thread, and
 // the launch of n_steps (< 2^31) steps.
@@ -242,6 +243,7 @@ struct CtxView {
     KParams kp;  // with the ensemble's seed and real0
     int tune_kind, tune_rods, tune_rows, tune_cpt;
     bool tune_generic;
+    bool may_cut;  // an automatic plan may take several SMs for a rod
     long long chunk_steps;  // steps per launch
 };
 llg_status ctx_view(llg_ctx *ctx, CtxView *out);

@@ -115,3 +115,34 @@ def test_gradient_of_a_non_finite_state(pkg, n_real):  # noqa: F811
         g.sync(60)
     assert e.value.status == 4
     g.close()
+
+
+def test_rods_stay_whole_beside_other_streams(pkg):  # noqa: F811
+    """A context on a stream of its own may run beside others, which a cut rod would take SMs from: its rods are
+    not cut (no wait to run out), the context moved to the default stream cuts them; the states agree."""
+    g = cut_grid(pkg, (4, 12, 28))
+    g.set_tuning(pkg.TUNE_HANDOFF_TIMEOUT_MS, 20)
+    g.set_tuning(pkg.TUNE_WITHHOLD_HANDOFF, 1)
+    out = []
+    stream = torch.cuda.Stream()
+    for own in (True, False):
+        g.set_stream(stream.cuda_stream if own else 0)
+        g.reset(seed=3, n_real=3)
+        g.advance(50)
+        if own:
+            g.sync(60)
+        else:
+            with pytest.raises(pkg.LLGError) as e:
+                g.sync(60)
+            assert e.value.status == 5
+            g.set_tuning(pkg.TUNE_WITHHOLD_HANDOFF, 0)
+            g.reset(seed=3, n_real=3)
+            g.advance(50)
+            g.sync(60)
+        m = torch.empty((3, g.ncells, 3), device="cuda")
+        g.get_state(m)
+        g.sync(60)
+        out.append(m.clone())
+    torch.cuda.synchronize()
+    assert torch.equal(out[0], out[1])
+    g.close()
