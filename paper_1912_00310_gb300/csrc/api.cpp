@@ -896,12 +896,12 @@ llg_status llg_loop_area_grad(llg_ctx *c, int64_t n_steps, int objective, const 
     if (e == cudaSuccess && !store_all) e = cudaMalloc(&seg, sizeof(float) * state * (size_t)std::min(C, N));
     if (e == cudaSuccess) e = cudaMalloc(&lam, sizeof(float) * state);
     if (e == cudaSuccess) e = cudaMalloc(&work, sizeof(float) * state);
-    if (e == cudaSuccess) e = cudaMalloc(&smp, sizeof(float) * (size_t)c->n_real * (size_t)ns_total);
+    // the forward pass's samples and, after them, its own status word (the ensemble's keeps what an advance left
+    // there), read in one copy
+    const size_t n_smp = (size_t)c->n_real * (size_t)ns_total;
+    if (e == cudaSuccess) e = cudaMalloc(&smp, sizeof(float) * (n_smp + 1));
     if (e == cudaSuccess) e = cudaMalloc(&w, sizeof(double) * (size_t)K);
-    // the partial sums and, after them, the forward pass's own status word: the ensemble's keeps what an advance
-    // left there
-    const size_t n_partial = 5 * (size_t)c->n_real;
-    if (e == cudaSuccess) e = cudaMalloc(&partial, sizeof(double) * (n_partial + 1));
+    if (e == cudaSuccess) e = cudaMalloc(&partial, sizeof(double) * 5 * (size_t)c->n_real);
     if (e != cudaSuccess) {
         cleanup();
         cudaGetLastError();
@@ -911,7 +911,7 @@ llg_status llg_loop_area_grad(llg_ctx *c, int64_t n_steps, int objective, const 
     kps.n_samples = ns_total;
     const cudaStream_t st = c->stream;
     // forward pass with a checkpoint at the start of every segment
-    int *const fwd_status = reinterpret_cast<int *>(partial + n_partial);
+    int *const fwd_status = reinterpret_cast<int *>(smp + n_smp);
     e = cudaMemcpyAsync(work, c->d_m, sizeof(float) * state, cudaMemcpyDeviceToDevice, st);
     if (e == cudaSuccess) e = cudaMemsetAsync(fwd_status, 0, sizeof(int), st);
     for (long long sg = 0; sg < S && e == cudaSuccess; ++sg) {
@@ -920,12 +920,12 @@ llg_status llg_loop_area_grad(llg_ctx *c, int64_t n_steps, int objective, const 
         if (e == cudaSuccess)
             e = llg::rod_advance(kps, plan, work, c->n_real, step0 + sg * C, len, smp, fwd_status, nullptr, st);
     }
-    std::vector<float> hs((size_t)c->n_real * (size_t)ns_total);
-    int hst = 0;
+    std::vector<float> hs(n_smp + 1);
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(hs.data(), smp, sizeof(float) * hs.size(), cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(&hst, fwd_status, sizeof(int), cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    int hst;
+    std::memcpy(&hst, &hs[n_smp], sizeof hst);
     if (e == cudaSuccess && (hst & 1)) {  // a non-finite sample: the loss says so, and so does the next llg_sync
         int all = 0;
         e = cudaMemcpy(&all, c->d_status, sizeof(int), cudaMemcpyDeviceToHost);
@@ -950,7 +950,7 @@ llg_status llg_loop_area_grad(llg_ctx *c, int64_t n_steps, int objective, const 
     const double L = window_loss(d, c->sw, objective, target, k_first, K, mbar, wk);
     e = cudaMemcpyAsync(w, wk.data(), sizeof(double) * (size_t)K, cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess) e = cudaMemsetAsync(lam, 0, sizeof(float) * state, st);
-    if (e == cudaSuccess) e = cudaMemsetAsync(partial, 0, sizeof(double) * n_partial, st);
+    if (e == cudaSuccess) e = cudaMemsetAsync(partial, 0, sizeof(double) * 5 * (size_t)c->n_real, st);
     if (store_all) {
         if (e == cudaSuccess) e = llg::adjoint_recompute_all(kps, c->n_real, step0, N, (int)C, ckpt, seg, st);
         if (e == cudaSuccess)
@@ -962,7 +962,7 @@ llg_status llg_loop_area_grad(llg_ctx *c, int64_t n_steps, int objective, const 
                                      ckpt + (size_t)sg * state, seg, lam, w, partial, st);
         }
     }
-    std::vector<double> hp(n_partial);
+    std::vector<double> hp((size_t)c->n_real * 5);
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(hp.data(), partial, sizeof(double) * hp.size(), cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
