@@ -26,6 +26,7 @@
 #include <cstring>
 
 #include "llg_internal.h"
+#include "mbarrier.cuh"
 #include "pair.cuh"
 #include "physics.cuh"
 #include "reduce.cuh"
@@ -319,13 +320,6 @@ __device__ __forceinline__ void st_release_gpu(unsigned *p, unsigned v)
     asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
 
-__device__ __forceinline__ unsigned long long globaltimer_ns()
-{
-    unsigned long long t;
-    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-    return t;
-}
-
 // Balanced schedule of one launch (McNaughton's wrap-around rule): all n_real * N rod-steps laid
 // end to end and cut into gridDim.x equal slices; a rod cut at a slice boundary runs its first
 // steps at the start of the next CTA's slice and its last steps at the end of this CTA's slice,
@@ -366,10 +360,10 @@ __global__ void __launch_bounds__(NY > 0 && NZ > 0 ? pipelined_threads(NY * NZ, 
         if (sg.z <= 0) continue;
         if (sg.w == 2) {
             if (threadIdx.x == 0) {
-                const unsigned long long t0 = globaltimer_ns();
+                const unsigned long long t0 = timer_ns();
                 int ok = 1;
                 while (ld_acquire_gpu(flags + sg.x) == 0u) {
-                    if (globaltimer_ns() - t0 > hc.timeout_ns) {
+                    if (timer_ns() - t0 > hc.timeout_ns) {
                         ok = 0;
                         atomicOr(status, 2);
                         break;

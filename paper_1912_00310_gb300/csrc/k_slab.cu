@@ -46,6 +46,7 @@
 #include <cstring>
 
 #include "llg_internal.h"
+#include "mbarrier.cuh"
 #include "physics.cuh"
 
 namespace llg {
@@ -60,49 +61,6 @@ constexpr int kFixedPitch = 64 + 4, kFixedBoxRows = 27 + 4;
 constexpr unsigned long long kStageWaitNs = 2000000000ull;  // longest wait for a staged plane
 
 __device__ __forceinline__ float3 zero3s() { return make_float3(0.f, 0.f, 0.f); }
-
-__device__ __forceinline__ unsigned smem_u32(const void *p) { return (unsigned)__cvta_generic_to_shared(p); }
-
-__device__ __forceinline__ unsigned long long gtimer_ns()
-{
-    unsigned long long t;
-    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-    return t;
-}
-
-__device__ __forceinline__ void mbar_init(uint64_t *bar, unsigned count)
-{
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count) : "memory");
-}
-
-__device__ __forceinline__ void mbar_expect_tx(uint64_t *bar, unsigned bytes)
-{
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes)
-                 : "memory");
-}
-
-__device__ __forceinline__ bool mbar_try_wait(uint64_t *bar, unsigned parity)
-{
-    unsigned ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(ok)
-        : "r"(smem_u32(bar)), "r"(parity)
-        : "memory");
-    return ok != 0;
-}
-
-// Wait for the phase of `parity` to complete, giving up after kStageWaitNs.
-__device__ __forceinline__ bool mbar_wait(uint64_t *bar, unsigned parity)
-{
-    if (mbar_try_wait(bar, parity)) return true;
-    const unsigned long long t0 = gtimer_ns();
-    while (!mbar_try_wait(bar, parity))
-        if (gtimer_ns() - t0 > kStageWaitNs) return false;
-    return true;
-}
 
 // One box of the padded state: coordinates (float component, x, y, z, realisation).
 __device__ __forceinline__ void tma_load_plane(void *dst, const CUtensorMap *map, uint64_t *bar, int x, int y, int z,
@@ -138,7 +96,7 @@ struct SlabSweep {
     static constexpr bool kFixed = FIXED;
     float4 *Mb, *Tb;     // [3][slot] state planes; [3][tslot] predictor planes (Tb one row early)
     uint64_t *bar;       // [3] one mbarrier per state slot
-    int pitch_rt, slot_rt, NZ;
+    int pitch_rt, slot_rt;
     // the CTA's part of z: planes [za, zb) get their corrector, [zs, ze) their predictor (one more on either
     // side), [l0, l1) are staged (one more again)
     int za, zb, zs, ze, l0, l1;
@@ -152,7 +110,6 @@ struct SlabSweep {
     PhiloxStep now;      // the noise's first rounds for this step
     const float4 *axr;
     float Hn, Hn1;
-    unsigned long long n;
     int *status;
     // columns of this thread (kFixed: only [0] is kept; column k is [0] plus k row strides)
     int q_[kFixed ? 1 : CPT];          // position in a staged plane
@@ -222,7 +179,7 @@ struct SlabSweep {
 
     __device__ __forceinline__ void issue(int z, int s)
     {
-        mbar_expect_tx(bar + s, box_bytes);
+        mbar_arrive_expect(bar + s, box_bytes);
         tma_load_plane(Mb + s * slot(), tin, bar + s, tile_x, tile_y, z, real);
         last_issued = z;
     }
@@ -233,7 +190,7 @@ struct SlabSweep {
     __device__ void drain()
     {
         for (int t = max(0, last_issued - l0 - 2); t <= last_issued - l0; ++t)
-            mbar_wait(bar + t % 3, (unsigned)((t / 3) & 1));
+            mbar_wait<false>(bar + t % 3, (unsigned)((t / 3) & 1), kStageWaitNs);
     }
 
     // A column's new state goes to its padded position and, near a periodic face, to the images
@@ -252,8 +209,8 @@ struct SlabSweep {
         }
     }
 
-    // Iteration t = z - l0 of the sweep, t = 3 j + U: predictor of plane z and corrector of plane z - 1,
-    // where they belong to the CTA's part (a first plane staged only for the predictor above it is just
+    // Iteration z of the sweep: predictor of plane z and corrector of plane z - 1, where they belong to the CTA's
+    // part (a first plane staged only for the predictor above it is just
     // remembered).  Ends in a CTA barrier; returns true (in every thread) when some thread's staging wait
     // gave up.
     template <bool INNER>
@@ -264,7 +221,7 @@ struct SlabSweep {
         const bool has_next = INNER || z + 1 < l1;
         int fail = 0;
         // plane z+1, issued an iteration ago
-        if (has_next && !mbar_wait(bar + sp1, par_next)) {
+        if (has_next && !mbar_wait<false>(bar + sp1, par_next, kStageWaitNs)) {
             atomicOr(status, 4);
             fail = 1;
         }
@@ -369,7 +326,6 @@ __global__ void __launch_bounds__(FIXED ? kFixedThreads : CPT == 1 ? kSlabThread
     w.Tb = sm4 + 3 * slot - w.pitch();  // row 0 of a predictor slot is row 1 of the box
     w.Hs = sm4 + 3 * slot + 3 * tslot;
     w.bar = reinterpret_cast<uint64_t *>(w.Hs + CPT * blockDim.x);
-    w.NZ = G.NZ;
     w.NX = G.NX;
     w.NY = G.NY;
     w.NXp = G.NXp;
@@ -378,7 +334,6 @@ __global__ void __launch_bounds__(FIXED ? kFixedThreads : CPT == 1 ? kSlabThread
     w.lead = threadIdx.x == 0;
     w.tin = &tin;
     w.box_bytes = G.box_bytes;
-    w.n = n;
     w.status = status;
     const int tx = blockIdx.x, ty = blockIdx.y, real = blockIdx.z / G.parts, part = blockIdx.z % G.parts;
     w.za = (int)((long long)part * G.NZ / G.parts);
@@ -474,7 +429,7 @@ __global__ void __launch_bounds__(FIXED ? kFixedThreads : CPT == 1 ? kSlabThread
     }
     // the first plane before the sweep starts
     int fail = 0;
-    if (!mbar_wait(w.bar, 0u)) {
+    if (!mbar_wait<false>(w.bar, 0u, kStageWaitNs)) {
         atomicOr(status, 4);
         fail = 1;
     }
