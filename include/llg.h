@@ -315,7 +315,7 @@ llg_status llg_autotune(llg_ctx *ctx, int64_t trial_steps, double *best_rate);
  * synchronises.
  * loss_out (optional) receives L; grad_out receives dL/d(s_K, s_alpha, s_Ms).
  * Errors: EINVAL (no ensemble, no sample in the window, window past the loop end),
- * EUNSUPPORTED (grid), ENOMEM, ECUDA. */
+ * EUNSUPPORTED (grid), ENOMEM, ETIMEOUT (a wait of method 0's forward pass gave up), ECUDA. */
 llg_status llg_loop_area_grad(llg_ctx *ctx, int64_t n_steps, int objective, const double *target,
                               int64_t ckpt_every, double *loss_out, double grad_out[3]);
 

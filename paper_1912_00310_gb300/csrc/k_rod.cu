@@ -7,8 +7,8 @@
 //      b = 2, 4, 8 rods of the paper's ladder rod_rows_kernel, rod_cells_kernel and rod_warp_kernel, in
 //      k_rod_small.cu.  One or several rods per CTA, two barriers a step.
 //
-//  rod_split_kernel (ensembles of fewer rods than SMs, where that is faster), in k_rod_split.cu: a rod
-//      cut along z over a cluster of CTAs.
+//  rod_split_kernel (ensembles of fewer rods than SMs, where that is faster and the launch has the GPU to
+//      itself), in k_rod_split.cu: a rod cut along z over a cluster of CTAs.
 //
 //  rod_pipelined_kernel (the b = 1 rod, 8x24x56 = 10752 cells: M alone is 129 KB, M and a full
 //      predictor copy do not fit).  One rod per CTA.  Each thread owns rows along x (fixed y, z);
@@ -240,7 +240,7 @@ int round_warp(int n) { return (n + 31) / 32 * 32; }
 }  // namespace
 
 // Measured, us: b = 2, 4, 8 rods 1.63, 0.44, 0.25; two-phase rods of 58, 312, 819 and 1265 cells 0.36, 0.74, 1.54 and
-// 2.15; the b = 1 rod 11.2; 6x16x30 cells on the runtime-size pipelined kernel 5.4.
+// 2.15; the b = 1 rod 11.2; on the runtime-size pipelined kernel 5.4 for 2880 cells.
 double one_sm_us(const KParams &p, int kind)
 {
     if (kind == 3) return 0.29 + 0.001 * p.ncells;

@@ -28,12 +28,12 @@ constexpr int kMaxThreads = 768;
 // What bounds it: the heavy FMA pipe, 61 % busy with 608 b = 4 rods (the noise's 32-bit multiplies and
 // half of every packed operation), and the two barriers' chains between (three warps a scheduler).
 // 608 b = 4 rods 0.83 us a step (1.03 with one cell an instruction), 1216 1.58 (1.83), four alone 0.44
-// (0.71); 152 b = 2 rods 1.55 (1.77), 256 2.98.  Threads without a row compute row 0's again and store
-// nothing: with branches around the work its parts cannot be interleaved (608 b = 4 rods 0.86, four
-// 0.47, 256 b = 2 rods 3.31).  Drawing the next step's noise beside the corrector: 608 b = 4 rods 0.82,
+// (0.71); 152 b = 2 rods 1.55 (1.77), 256 2.98.  Threads without a row go through the work on row 0's
+// places with values of no meaning and store nothing: with branches around it its parts cannot be
+// interleaved (608 b = 4 rods 0.86, four 0.47, 256 b = 2 rods 3.31).  Drawing the next step's noise beside the corrector: 608 b = 4 rods 0.82,
 // but 1216 1.61 and 256 b = 2 rods 3.50.
 // The b = 2 rod's instance has 126 registers, so that one CTA of 352 threads fits an SM; where there are more
-// rods than SMs, or other jobs beside them, an instance of 80 (CTAS = 2) runs two side by side: 256 rods
+// rods than SMs, or jobs of a batch beside them, an instance of 80 (CTAS = 2) runs two side by side: 256 rods
 // 3.08 -> 2.98 us a step, 512 6.16 -> 5.81, 1024 10.76 -> 10.01, with dispersed axes (spills) 3.33 -> 3.26 and
 // 6.65 -> 6.34 at 512; alone on its SM a rod takes 1.55 us with the first and 1.72 with the second.
 // ------------------------------------------------------------------------------------------

@@ -25,8 +25,9 @@
 // engine's: bitwise the same states.
 //
 // What bounds it: the chain of a step -- neighbour loads, field, torque, normalisation, store, the lines' way
-// to the next CTA, twice -- with one or two warps a scheduler to hide it.  One b = 1 rod takes 2.06 us a step
-// over 8 CTAs (11.2 on one SM; 15 rods as many), 32 rods 3.53 over 4; one b = 2 rod 0.83 (1.63).  Tried:
+// to the next CTA, twice -- with one or two warps a scheduler to hide it.  One b = 1 rod takes 2.12 us a step
+// over 8 CTAs (11.1 on one SM; 15 rods as many), 32 rods 3.49 over 4; three b = 2 rods 0.80 over 7 (1.55).  A way
+// out of the step loop for waits that give up costs b = 1 rods up to 5 % of that, the others nothing.  Tried:
 // noise drawn by warps of its own into a ring (one b = 1 rod 3.2 us: the two kinds of warp wait for one
 // another's pipes), whole rows to a thread (2.70), remote arrivals as above.
 #include <algorithm>

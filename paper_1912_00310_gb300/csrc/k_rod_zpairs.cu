@@ -20,8 +20,8 @@
 //
 // What bounds it: with one rod per SM the chain of a step (field, torque, normalisation twice, the noise,
 // two barriers), with several the FMA pipes (heavy pipe 60 % busy with 608 b = 4 rods).  152 rods of
-// 5x11x23 cells held in a field for 1500 steps: 4.91 -> 3.25 ms; one cell to a thread in a ghost-padded
-// float4 rod issued 325 instructions per cell and step, this 173.
+// 5x11x23 cells held in a field for 1500 steps: 4.91 -> 3.19 ms, 209 thread-instructions per cell and step; the
+// b = 4 rod's were 325 with one cell to a thread in a ghost-padded float4 rod and are 173 here.
 #include <algorithm>
 
 #include "llg_internal.h"

@@ -1,5 +1,5 @@
-// rod_compact.cuh -- pieces shared by the gradient kernels (k_adjoint.cu, k_tangent.cu): small
-// FP32 vector helpers with explicit fused multiply-adds, and the compact shared-memory rod.
+// rod_compact.cuh -- pieces shared by the gradient kernels (k_adjoint.cu, k_tangent.cu) and the kernel for small
+// rods (rod_compact_kernel of k_rod_zpairs.cu): small FP32 vector helpers with explicit fused multiply-adds, and the compact shared-memory rod.
 //
 // Compact rod: one float4 per cell in cell order (x fastest, then y, then z), followed by one zero
 // slot that stands for every neighbour beyond a free face.  Consecutive threads then read
