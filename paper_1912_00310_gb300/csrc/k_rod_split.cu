@@ -25,8 +25,8 @@
 // engine's: bitwise the same states.
 //
 // What bounds it: the chain of a step -- neighbour loads, field, torque, normalisation, store, the lines' way
-// to the next CTA, twice -- with one or two warps a scheduler to hide it.  One b = 1 rod takes 2.12 us a step
-// over 8 CTAs (11.1 on one SM; 15 rods as many), 32 rods 3.49 over 4; three b = 2 rods 0.80 over 7 (1.55).  A way
+// to the next CTA, twice -- with one or two warps a scheduler to hide it.  One b = 1 rod takes 2.06 us a step
+// over 8 CTAs (11.1 on one SM; 15 rods as many), 32 rods 3.49 over 4; three b = 2 rods 0.77 over 7 (1.55).  A way
 // out of the step loop for waits that give up costs b = 1 rods up to 5 % of that, the others nothing.  Tried:
 // noise drawn by warps of its own into a ring (one b = 1 rod 3.2 us: the two kinds of warp wait for one
 // another's pipes), whole rows to a thread (2.70), remote arrivals as above.
@@ -291,7 +291,11 @@ __global__ void __launch_bounds__(kMaxThreads, 1) rod_split_kernel(KParams p, in
         auto arrive = [&](int b) {
             __syncwarp();
             if (lane == 0 && alive) {
-                if (threadIdx.x == 0)
+                // (one instruction for both: three b = 2 rods 0.80 -> 0.77 us a step, b = 1 rods of two pairs a
+                // thread 2.12 -> 2.06, but of four 3.49 -> 3.84)
+                if constexpr (W < 4)
+                    mbar_arrive_expect(half + b, warp == 0 ? line_bytes : 0u);
+                else if (threadIdx.x == 0)
                     mbar_arrive_expect(half + b, line_bytes);
                 else
                     mbar_arrive(half + b);
@@ -535,8 +539,8 @@ int split_clusters_at_once(const KParams &p, const RodPlan &plan, int dev)
 
 // Whether cutting the rods beats one rod per SM, which takes base_us a step, and over how many CTAs.  A
 // step of a slab of c pairs takes about 0.72 us + 2 ns c, with four pairs to a thread 2.1 ns where they fill
-// their rows and 3.2 where not: measured 2.1 us at 672 pairs (b = 1 over 8 CTAs), 3.5 at 1344 (over 4),
-// 0.80, 1.01 and 1.24 at 96, 168 and 336 (b = 2 over 8, 4 and 2), 0.87 and 1.12 at 99 and 198 (5x11x23 cells
+// their rows and 3.2 where not: measured 2.06 us at 672 pairs (b = 1 over 8 CTAs), 3.5 at 1344 (over 4),
+// 0.77, 0.98 and 1.24 at 96, 168 and 336 (b = 2 over 8, 4 and 2), 0.84 and 1.12 at 99 and 198 (5x11x23 cells
 // over 8 and 4), 3.03 at 720 (6x16x30 over 2).  Clusters run side by side as far as the GPCs hold them, the
 // rest in further waves: kAtOnce is what a GB300 of 152 SMs holds at one CTA to an SM; the device at hand is asked
 // about the choice (one call, not one for each k) and has the last word where it holds fewer, or none: that
